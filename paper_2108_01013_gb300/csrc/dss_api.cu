@@ -1,6 +1,7 @@
 // Host side of the C ABI declared in include/dss.h: validation, buffer
 // management, the per-step launch sequence and its CUDA-graph capture.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -51,7 +52,6 @@ void free_buffers(dss_handle* h) {
   dfree(h->own); dfree(h->bw_count); dfree(h->bw_rec); dfree(h->carry); dfree(h->own_s);
   h->own = nullptr; h->bw_count = nullptr; h->bw_rec = nullptr; h->carry = nullptr; h->own_s = nullptr;
   h->pb_blocks = 0;
-  h->compact_ok[0] = h->compact_ok[1] = false;
   dfree(h->io3); dfree(h->io3b); dfree(h->io_id); dfree(h->stage);
   h->stage = nullptr; dfree(h->scan_status); dfree(h->scan_ticket);
   dfree(h->sigma);
@@ -60,6 +60,9 @@ void free_buffers(dss_handle* h) {
   dfree(h->inst_map);
   dfree(h->cls_map);
   h->cls_map = nullptr;
+  dfree(h->enum_inst);
+  h->enum_inst = nullptr;
+  h->enum_inst_cap = 0;
   dfree(h->ig);
   dfree(h->sg);
   h->sigma_sum = nullptr;
@@ -135,12 +138,11 @@ int alloc_pair_buffers(dss_handle* h, int64_t pcap, bool keep_hist) {
     h->carry = carry;
     h->pb_blocks = pair_pb_blocks(h);
   }
-  h->compact_ok[0] = h->compact_ok[1] = false;
   double* sp = nullptr;
   // (the balanced grid holds at most 4 blocks per SM; batched instances keep
   // 16 stress slices each)
-  const int pb = std::max(std::max(pair_grid_blocks(h), h->K == 1 ? 4 * h->sms : 0), 16 * h->K);
-  if ((r = dalloc(h, &sp, 18 * (size_t)pb))) return r;
+  const int pb = std::max(4 * h->sms, 16 * h->K);
+  if ((r = dalloc(h, &sp, 9 * (size_t)pb))) return r;
   dfree(h->spart);
   h->spart = sp;
   h->spart_blocks = pb;
@@ -200,7 +202,7 @@ int alloc_buffers(dss_handle* h) {
       h->own_s = own_s;
     }
   }
-  int tiles = std::max(scan_tiles_for(h->g.ncell), enum_scan_tiles_for((int)n));
+  const int tiles = std::max(scan_tiles_for(h->g.ncell), enum_scan_tiles_for((int)n));
   h->scan_tiles_max = std::max(tiles, 1);
   if ((r = dalloc(h, &h->scan_status, 2 * (size_t)h->scan_tiles_max)) ||
       (r = dalloc(h, &h->scan_ticket, 2)))
@@ -484,7 +486,8 @@ int status_error(dss_handle* h) {
 
 // Outside a step (where the pair kernel reports an overflow and the step is
 // replayed), a list just built may hold more pairs than the pair buffers fit:
-// grow them before anything writes per-pair data.  Waits for the list and
+// grow them before anything writes per-pair data, and list the pairs again
+// (the compact arrays ended at the old capacity).  Waits for the list and
 // returns the status of the kernels before it.
 int ensure_pair_capacity(dss_handle* h, int list) {
   int r = sync_status(h);
@@ -493,7 +496,36 @@ int ensure_pair_capacity(dss_handle* h, int list) {
   int P = 0;
   CK(cudaMemcpyAsync(&P, h->lb[list].start + h->n, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
-  if (P > h->pcap) return alloc_pair_buffers(h, (int64_t)(P * 1.25) + 1024, true);
+  if (P > h->pcap) {
+    if ((r = alloc_pair_buffers(h, (int64_t)(P * 1.25) + 1024, true))) return r;
+    CK(cudaMemsetAsync(h->scan_status + h->scan_tiles_max, 0, sizeof(unsigned long long) * h->scan_tiles_max,
+                       h->stream));
+    CK(cudaMemsetAsync(h->scan_ticket + 1, 0, sizeof(int), h->stream));
+    CK(cudaMemsetAsync(&h->status->w[ST_BAND], 0, sizeof(int), h->stream));
+    launch_enumerate(h, h->cur, list, 0);
+    CK(cudaGetLastError());
+  }
+  return DSS_OK;
+}
+
+// The enumeration's walk for the current grid (and, batched, the instance of
+// each of its blocks on the device); before the instance table goes up.
+int plan_enumeration(dss_handle* h) {
+  std::vector<int> inst;
+  const int64_t blocks = enum_plan(h, h->K > 1 ? &inst : nullptr);
+  if (blocks > (int64_t)INT_MAX) return DSS_ERR_ARG;
+  if (inst.empty()) return DSS_OK;
+  if (blocks > h->enum_inst_cap) {
+    int* p = nullptr;
+    int r = dalloc(h, &p, (size_t)blocks);
+    if (r) return r;
+    dfree(h->enum_inst);
+    h->bytes -= (int64_t)(sizeof(int) * h->enum_inst_cap);
+    h->enum_inst = p;
+    h->enum_inst_cap = blocks;
+  }
+  CK(cudaMemcpyAsync(h->enum_inst, inst.data(), sizeof(int) * (size_t)blocks, cudaMemcpyHostToDevice, h->stream));
+  CK(cudaStreamSynchronize(h->stream));
   return DSS_OK;
 }
 
@@ -898,6 +930,10 @@ int dss_set_state(dss_handle* h, const double* x, const double* a, const int32_t
     h->hist = 0;
     h->mean_steps = 0;
     StateBuf& s = h->st[0];
+    {
+      const int r = plan_enumeration(h);
+      if (r) return r;
+    }
     CK(cudaMemcpyAsync(h->ig, h->ig_host, sizeof(InstGeo) * h->K, cudaMemcpyHostToDevice, h->stream));
     CK(cudaMemcpyAsync(h->inst_map, imap.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, h->stream));
     CK(cudaMemcpyAsync(s.inst, h->inst_map, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, h->stream));

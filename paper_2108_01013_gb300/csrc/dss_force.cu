@@ -1,20 +1,17 @@
 // Pair forces and their deterministic symmetric accumulation.
 //
-// k_pairs<MIXED, MINB, EXT>: a warp takes 32 consecutive owners and deals out their
-//   listed pairs (owner-sorted) 32 at a time.  Per pair: lubrication of
-//   App. A (Eq. A2, A3 with the coefficients of Eq. A6, A7 and the
-//   6 pi eta0 prefactor), stick-and-slide contact of Eq. 4-5 with the
-//   tangential stretch carried from the previous step's rows, and the pair
-//   stresslet of Eq. 9.  The owner's share is summed by a warp-segmented
-//   reduction (lanes holding the same owner are contiguous) into a per-warp
-//   shared-memory accumulator and written once per owner; the partner's share
-//   (-F and its torque) is appended to the partner's fixed-capacity row
-//   together with the owner's index.  No float is ever accumulated with an
-//   atomic.
-// k_pairs_pb<MIXED, MINB, EXT> (one instance): the same per pair, with the
-//   pairs in owner order dealt out 32 to a warp over the resident blocks
-//   (every lane busy whatever the row lengths); owners whose pairs cross a
-//   warp boundary leave head / tail partial sums the gather adds in order.
+// k_pairs_pb<MIXED, MINB, EXT, PERS>: the listed pairs in owner order, dealt
+//   out 32 to a warp over the resident blocks (every lane busy whatever the
+//   row lengths).  Per pair: lubrication of App. A (Eq. A2, A3 with the
+//   coefficients of Eq. A6, A7 and the 6 pi eta0 prefactor), stick-and-slide
+//   contact of Eq. 4-5 with the tangential stretch carried from the previous
+//   step's rows, and the pair stresslet of Eq. 9.  The owner's share is
+//   summed by a warp-segmented reduction (lanes holding the same owner are
+//   contiguous) and written once per owner, or, for owners whose pairs cross
+//   a warp boundary, as head / tail partial sums the gather adds in order;
+//   the partner's share (-F and its torque) is appended to the partner's
+//   fixed-capacity row together with the owner's index.  No float is ever
+//   accumulated with an atomic.
 // k_gather<MIXED, EXT>: one thread per particle: its own sum plus the partner
 //   records of its row taken in increasing owner index (a fixed order, so the
 //   result is bitwise reproducible; rows of 9 to 24 FP32 records and longer
@@ -539,47 +536,28 @@ __device__ __forceinline__ void owner_scan(int lane, int seg, R v[NV]) {
 }
 
 // The block's stresslet partials (fixed tree over lanes, warps and blocks):
-// x0 the thread's sums for the instance of the block's first owner, x1 for
-// the next instance (zero unless `second`), e0/e1 the single-particle wave
-// stresslets the thread adds to them.  FP64 throughout in FP64.  In mixed
-// precision the thread sums (one to a few pairs each) are FP32, the lanes and
-// warps of the block are summed with compensation (Knuth's TwoSum on every
-// addition, ~48 significant bits: an FP64 butterfly on every lane costs ~90
-// additions per thread on GB300's narrow FP64 pipe, +40% on this kernel),
-// and the block's sum is converted to FP64 once; every sum beyond the block
-// is FP64.
+// x the thread's sums, e the single-particle wave stresslets the thread adds
+// to them.  FP64 throughout in FP64.  In mixed precision the thread sums (one
+// to a few pairs each) are FP32, the lanes and warps of the block are summed
+// with compensation (Knuth's TwoSum on every addition, ~48 significant bits:
+// an FP64 butterfly on every lane costs ~90 additions per thread on GB300's
+// narrow FP64 pipe, +40% on this kernel), and the block's sum is converted to
+// FP64 once; every sum beyond the block is FP64.
 template <bool MIXED, bool EXT>
 __device__ __forceinline__ void stress_partials(
-    const typename std::conditional<MIXED, float, double>::type* x0,
-    const typename std::conditional<MIXED, float, double>::type* x1, bool second, double e0, double e1,
-    int ncont, double* __restrict__ spart, DevStatus* st) {
-  using R = typename std::conditional<MIXED, float, double>::type;
-  __shared__ double red[MIXED ? 1 : kWarps][18];
-  __shared__ float redh[MIXED ? kWarps : 1][18], redl[MIXED ? kWarps : 1][18];
+    const typename std::conditional<MIXED, float, double>::type* x, double e, int ncont,
+    double* __restrict__ spart, DevStatus* st) {
+  __shared__ double red[MIXED ? 1 : kWarps][9];
+  __shared__ float redh[MIXED ? kWarps : 1][9], redl[MIXED ? kWarps : 1][9];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  // the second instance slot holds anything only where a lane of the warp
-  // met a second instance (in its pairs, or as the owner of a wave stresslet)
-  const int nq = __any_sync(0xffffffffu, second || e1 != 0.0) ? 18 : 9;
 #pragma unroll
-  for (int q = 0; q < 18; ++q) {
-    if (q >= nq) {
-      if (lane == 0) {
-        if constexpr (MIXED) {
-          redh[wid][q] = 0.0f;
-          redl[wid][q] = 0.0f;
-        } else {
-          red[wid][q] = 0.0;
-        }
-      }
-      continue;
-    }
-    const R x = q < 9 ? x0[q] : (second ? x1[q - 9] : R(0));
-    const double e = (q == 1 || q == 3) ? e0 : ((q == 10 || q == 12) ? e1 : 0.0);
+  for (int q = 0; q < 9; ++q) {
+    const double eq = (q == 1 || q == 3) ? e : 0.0;
     if constexpr (MIXED) {
-      FF v{x, 0.0f};
-      if (EXT && e != 0.0) {
-        v = two_sum(x, (float)e);
-        v.lo += (float)(e - (double)(float)e);
+      FF v{x[q], 0.0f};
+      if (EXT && eq != 0.0) {
+        v = two_sum(x[q], (float)eq);
+        v.lo += (float)(eq - (double)(float)eq);
       }
       for (int dlt = 16; dlt > 0; dlt >>= 1) {
         const float h2 = __shfl_down_sync(0xffffffffu, v.hi, dlt);
@@ -593,154 +571,30 @@ __device__ __forceinline__ void stress_partials(
         redl[wid][q] = v.lo;
       }
     } else {
-      double v = (double)x + e;
+      double v = x[q] + eq;
       for (int dlt = 16; dlt > 0; dlt >>= 1) v += __shfl_down_sync(0xffffffffu, v, dlt);
       if (lane == 0) red[wid][q] = v;
     }
   }
-  int c = ncont;
-  for (int dlt = 16; dlt > 0; dlt >>= 1) c += __shfl_down_sync(0xffffffffu, c, dlt);
+  const int c = __reduce_add_sync(0xffffffffu, ncont);
   if (lane == 0 && c) atomicAdd(&st->w[ST_NCONT], c);
   __syncthreads();
-  if (threadIdx.x < 18) {
+  if (threadIdx.x < 9) {
+    const int q = threadIdx.x;
     if constexpr (MIXED) {
-      const int q = threadIdx.x;
       FF v{redh[0][q], redl[0][q]};
       for (int w = 1; w < kWarps; ++w) {
         const FF t = two_sum(v.hi, redh[w][q]);
         v.hi = t.hi;
         v.lo = (v.lo + redl[w][q]) + t.lo;
       }
-      spart[blockIdx.x * 18 + q] = (double)v.hi + (double)v.lo;
+      spart[blockIdx.x * 9 + q] = (double)v.hi + (double)v.lo;
     } else {
       double v = 0.0;
-      for (int w = 0; w < kWarps; ++w) v += red[w][threadIdx.x];
-      spart[blockIdx.x * 18 + threadIdx.x] = v;
+      for (int w = 0; w < kWarps; ++w) v += red[w][q];
+      spart[blockIdx.x * 9 + q] = v;
     }
   }
-}
-
-// MINB: resident blocks per SM the register budget is cut for (a grid that
-// fills more than three blocks per SM gains from the fourth; smaller grids
-// run faster with the larger budget).
-template <bool MIXED, int MINB, bool EXT>
-__global__ void __launch_bounds__(kPairThreads, MINB)
-k_pairs(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sgk, StateBuf s, ListBuf W,
-        ListBuf H, const float4* __restrict__ posf, void* __restrict__ own_v, int* __restrict__ bw_count,
-        void* __restrict__ bw_v, double* __restrict__ spart, DevStatus* st,
-        const int* __restrict__ perm) {
-  using R = typename std::conditional<MIXED, float, double>::type;
-  if (dev_err(st)) return;
-  R* __restrict__ own = static_cast<R*>(own_v);
-  R* __restrict__ bw = static_cast<R*>(bw_v);
-  const int n = g.n;
-  const int P = W.start[n];
-  const HistRef hr{perm, *((volatile const int*)&st->w[ST_IDORDER])};
-  if (P > g.pcap) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      st->w[ST_NPAIRS] = P;
-      set_err(st, DSS_ERR_CAPACITY);
-    }
-    return;
-  }
-  __shared__ R acc[kWarps][32][6];
-  // The block's owners span at most two instances (an instance has at least
-  // as many particles as a block has threads), and a lane meets its pairs in
-  // increasing owner order, so its instance changes at most once: the
-  // stresslet sum of the first instance is parked in shared memory then.
-  __shared__ R park[kPairThreads][9];
-  const int inst0 = s.inst[min((int)(blockIdx.x * blockDim.x), n - 1)];
-  int cur_inst = inst0;
-  R Sx[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-  int ncont = 0;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-#pragma unroll
-  for (int c = 0; c < 6; ++c) acc[wid][lane][c] = R(0);
-  __syncwarp();
-  for (int w0 = gw * 32; w0 < n; w0 += nw * 32) {
-    const int il = w0 + lane;
-    const int cnt = il < n ? W.count[il] : 0;
-    int incl = cnt;
-    for (int d = 1; d < 32; d <<= 1) {
-      const int t = __shfl_up_sync(0xffffffffu, incl, d);
-      if (lane >= d) incl += t;
-    }
-    const int excl = incl - cnt;
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    const int base = W.start[w0];
-    for (int t0 = 0; t0 < total; t0 += 32) {
-      const int t = t0 + lane;
-      int Lw = 0;
-      for (int step = 16; step >= 1; step >>= 1) {
-        const int e = __shfl_sync(0xffffffffu, excl, Lw + step);
-        if (e <= t) Lw += step;
-      }
-      const int kk = t - __shfl_sync(0xffffffffu, excl, Lw);
-      const bool valid = t < total;
-      R v[6] = {0, 0, 0, 0, 0, 0};
-      int seg = valid ? Lw : 32 + lane;      // owner lane, unique sentinel when idle
-      if (valid) {
-        const int i = w0 + Lw;
-        const int p = base + t;
-        const int j = W.list[(int64_t)i * g.Ms + kk];
-        const int inst = s.inst[i];
-        const InstGeo& I = ig[inst];
-        const StepGeo sg = sgk[inst];
-        PairRes<R> q;
-        if constexpr (MIXED) q = pair_eval_mixed<EXT>(g, I, s, H, hr, sg, posf, i, j);
-        else q = pair_eval_fp64<EXT>(g, I, s, H, hr, sg.off, i, j);
-        v[0] = q.F[0]; v[1] = q.F[1]; v[2] = q.F[2];
-        v[3] = q.Ti[0]; v[4] = q.Ti[1]; v[5] = q.Ti[2];
-        if (inst != cur_inst) {
-#pragma unroll
-          for (int c = 0; c < 9; ++c) {
-            park[threadIdx.x][c] = Sx[c];
-            Sx[c] = R(0);
-          }
-          cur_inst = inst;
-        }
-        pair_commit<R, EXT>(g, q, i, j, p, W, atomicAdd(&bw_count[j], 1), bw, st, Sx, ncont);
-      }
-      owner_scan<R>(lane, seg, v);
-      const int nxt = __shfl_down_sync(0xffffffffu, seg, 1);
-      if (valid && (lane == 31 || nxt != seg)) {
-#pragma unroll
-        for (int c = 0; c < 6; ++c) acc[wid][Lw][c] += v[c];
-      }
-      __syncwarp();
-    }
-    // one write per owner, then clear for the next group
-    if (il < n) {
-#pragma unroll
-      for (int c = 0; c < 6; ++c) own[(int64_t)c * n + il] = acc[wid][lane][c];
-    }
-#pragma unroll
-    for (int c = 0; c < 6; ++c) acc[wid][lane][c] = R(0);
-    __syncwarp();
-  }
-  const bool moved = cur_inst != inst0;
-  // With the wave of Eq. 17 the single-particle stresslets 20/3 pi eta0 a^3
-  // E_inf(x) carry a local part, (10/3) pi eta0 a^3 U k cos(k y) on xy and
-  // yx: one owner per thread (the grid covers each owner once), added to its
-  // instance's slot.
-  double ew0 = 0.0, ew1 = 0.0;
-  if (EXT && g.wave) {
-    const int il0 = blockIdx.x * blockDim.x + threadIdx.x;
-    if (il0 < n) {
-      const double a = s.a[il0];
-      const double e = (10.0 / 3.0) * DSS_PI * g.eta0 * a * a * a * s.wv[il0].y;
-      if (s.inst[il0] == inst0) ew0 = e; else ew1 = e;
-    }
-  }
-  R x0[9], x1[9];
-#pragma unroll
-  for (int c = 0; c < 9; ++c) {
-    x0[c] = moved ? park[threadIdx.x][c] : Sx[c];
-    x1[c] = moved ? Sx[c] : R(0);
-  }
-  stress_partials<MIXED, EXT>(x0, x1, moved, ew0, ew1, ncont, spart, st);
 }
 
 // Pair-balanced pair kernel.  The listed pairs in owner order (the compact
@@ -757,6 +611,7 @@ k_pairs(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sgk, 
 // the stresslet of Eq. 9 rides along in the owner scan, so that each owner's
 // stresslet sum is written with its force (own_s, or the boundary slots) and
 // the gather's instance blocks add them up over the instance's particles.
+// MINB: resident blocks per SM the register budget is cut for.
 template <bool MIXED, int MINB, bool EXT, bool PERS>
 __global__ void __launch_bounds__(kPairThreads, MINB)
 k_pairs_pb(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sgk, StateBuf s, ListBuf W,
@@ -843,8 +698,9 @@ k_pairs_pb(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sg
     const int c = __reduce_add_sync(0xffffffffu, ncont);
     if (lane == 0 && c) atomicAdd(&st->w[ST_NCONT], c);
   } else {
-    // the wave's single-particle stresslets (see k_pairs), particles strided
-    // over the grid's threads
+    // with the wave of Eq. 17 the single-particle stresslets 20/3 pi eta0 a^3
+    // E_inf(x) carry a local part, (10/3) pi eta0 a^3 U k cos(k y) on xy and
+    // yx: particles strided over the grid's threads
     double ew0 = 0.0;
     if (EXT && g.wave) {
       for (int il = blockIdx.x * blockDim.x + threadIdx.x; il < n; il += gridDim.x * blockDim.x) {
@@ -852,24 +708,18 @@ k_pairs_pb(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sg
         ew0 += (10.0 / 3.0) * DSS_PI * g.eta0 * a * a * a * s.wv[il].y;
       }
     }
-    stress_partials<MIXED, EXT>(Sx, Sx, false, ew0, 0.0, ncont, spart, st);
+    stress_partials<MIXED, EXT>(Sx, ew0, ncont, spart, st);
   }
 }
 
 // Bulk stress (Eq. 8) of one instance from the pair blocks' partials, by one
-// block of the gather (fixed strided assignment and fixed tree).  Pair block b
-// holds the sums of the instance containing its first owner (slot 0) and of
-// the next instance (slot 1).
-// With the pair-balanced kernel (one instance, pb_blocks > 0) every block's
-// first slot belongs to the instance.
+// block of the gather (fixed strided assignment and fixed tree).
 __device__ void inst_stress(const Geo& g, const InstGeo& I, const double* __restrict__ spart,
                             double* __restrict__ sigma, int pb_blocks) {
   __shared__ double red[kThreads / 32][9];
   double v[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-  const int b0 = pb_blocks ? 0 : I.p_begin / kPairThreads;
-  const int b1 = pb_blocks ? pb_blocks - 1 : (I.p_end - 1) / kPairThreads;
-  for (int b = b0 + threadIdx.x; b <= b1; b += blockDim.x) {
-    const double* p = spart + b * 18 + (pb_blocks || b * kPairThreads >= I.p_begin ? 0 : 9);
+  for (int b = threadIdx.x; b < pb_blocks; b += blockDim.x) {
+    const double* p = spart + b * 9;
 #pragma unroll
     for (int q = 0; q < 9; ++q) v[q] += p[q];
   }
@@ -941,7 +791,7 @@ k_owner_stress(Geo g, const InstGeo* __restrict__ ig, StateBuf s, const void* __
       ew += (10.0 / 3.0) * DSS_PI * g.eta0 * a * a * a * s.wv[j].y;
     }
   }
-  stress_partials<MIXED, EXT>(v, v, false, ew, 0.0, 0, spart, st);
+  stress_partials<MIXED, EXT>(v, ew, 0, spart, st);
 }
 
 // The instance's stress from its kOsParts slices (by one block of the gather).
@@ -950,7 +800,7 @@ __device__ void inst_stress_parts(const Geo& g, const InstGeo& I, const double* 
   if (threadIdx.x < 9) {
     const int q = threadIdx.x;
     double S = 0.0;
-    for (int p = 0; p < kOsParts; ++p) S += parts[p * 18 + q];
+    for (int p = 0; p < kOsParts; ++p) S += parts[p * 9 + q];
     const double E = (q == 1 || q == 3) ? 0.5 * I.gdot : 0.0;
     const double V = I.L[0] * I.L[1] * I.L[2];
     const double ein = 20.0 / 3.0 * DSS_PI * g.eta0 * I.sumA3;
@@ -1148,39 +998,31 @@ __device__ __forceinline__ bool gather_one(const Geo& g, const InstGeo* __restri
   const int j = valid ? j0 : 0;
   int cnt = valid ? __ldg(bw_count + j) : 0;
   R F[3], T[3];
-  if (carry) {
-    // pair-balanced sums: none (no owned pair), the owner's single write, or
-    // the tail slot of its first warp plus the head slots of the next ones
-    const int s0 = __ldg(start + j), s1 = __ldg(start + j + 1);
-    const int w0 = s0 >> 5, w1 = (s1 - 1) >> 5;
+  // pair-balanced sums: none (no owned pair), the owner's single write, or
+  // the tail slot of its first warp plus the head slots of the next ones
+  const int s0 = __ldg(start + j), s1 = __ldg(start + j + 1);
+  const int w0 = s0 >> 5, w1 = (s1 - 1) >> 5;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) F[c] = T[c] = R(0);
-    if (s1 > s0 && w0 == w1) {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        F[c] = own[(int64_t)c * n + j];
-        T[c] = own[(int64_t)(3 + c) * n + j];
-      }
-    } else if (s1 > s0) {
-      const int64_t cs = 2 * cnv;   // head slot, tail slot
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        F[c] = carry[w0 * cs + cnv + c];
-        T[c] = carry[w0 * cs + cnv + 3 + c];
-      }
-      for (int w = w0 + 1; w <= w1; ++w) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          F[c] += carry[w * cs + c];
-          T[c] += carry[w * cs + 3 + c];
-        }
-      }
-    }
-  } else {
+  for (int c = 0; c < 3; ++c) F[c] = T[c] = R(0);
+  if (s1 > s0 && w0 == w1) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       F[c] = own[(int64_t)c * n + j];
       T[c] = own[(int64_t)(3 + c) * n + j];
+    }
+  } else if (s1 > s0) {
+    const int64_t cs = 2 * cnv;   // head slot, tail slot
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      F[c] = carry[w0 * cs + cnv + c];
+      T[c] = carry[w0 * cs + cnv + 3 + c];
+    }
+    for (int w = w0 + 1; w <= w1; ++w) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        F[c] += carry[w * cs + c];
+        T[c] += carry[w * cs + 3 + c];
+      }
     }
   }
   const double a = __ldg(s.a + j);
@@ -1358,7 +1200,7 @@ k_gather(Geo g, const InstGeo* __restrict__ ig, StateBuf s, const void* __restri
   if (!s_err0) {
     if (blockIdx.x < (unsigned)g.K) {
       if (own_s_v)
-        inst_stress_parts(g, ig[blockIdx.x], spart + (int64_t)blockIdx.x * kOsParts * 18,
+        inst_stress_parts(g, ig[blockIdx.x], spart + (int64_t)blockIdx.x * kOsParts * 9,
                           sigma + 9 * blockIdx.x);
       else
         inst_stress(g, ig[blockIdx.x], spart, sigma + 9 * blockIdx.x, pb_blocks);
@@ -1405,8 +1247,7 @@ __global__ void k_pairs_out(Geo g, ListBuf W, long long* __restrict__ out) {
 }
 }  // namespace
 
-// One warp per 32 owners: ceil(n / kPairThreads) blocks cover every owner
-// once (the pair kernel also strides when given fewer).
+// Blocks of the per-pair passes outside the step (outputs, history).
 int pair_grid_blocks(const dss_handle* h) {
   int64_t need = (h->n + kPairThreads - 1) / kPairThreads;
   return (int)(need > 0 ? need : 1);
@@ -1429,50 +1270,34 @@ void launch_forces_t(dss_handle* h, int stbuf, int work_list, int hist_list, int
                      double* F_out, double* T_out) {
   (void)adv;
   const int n = (int)h->n;
-  const int pb = pair_grid_blocks(h);
   const bool mixed = h->g.precision == DSS_MIXED;
   prof_mark(h, 5);
-  // pairs dealt out 32 to a warp over the resident blocks (batched
-  // instances: with per-owner stresslets)
-  const bool pbal = h->pb_blocks > 0 && h->compact_ok[work_list];
+  // pairs dealt out 32 to a warp over the resident blocks of the register
+  // budget (mixed precision: 3 per SM, or, for one instance, 4 when the
+  // kernel autotuner chose the smaller budget); batched instances with
+  // per-owner stresslets
   const bool pers = h->g.K > 1;
-  const bool big = h->tune_pairs_minb ? h->tune_pairs_minb == 4 : pb > 3 * h->sms;
-  // the balanced grid: the resident blocks of its register budget (mixed
-  // precision: 3 per SM, or, for one instance, 4 when the kernel autotuner
-  // chose the smaller budget)
-  const bool pb4 = pbal && mixed && !pers && h->tune_pairs_minb == 4;
+  const bool pb4 = mixed && !pers && h->tune_pairs_minb == 4;
   const int pbg = pb4 ? 4 * h->sms : h->pb_blocks;
 #define DSS_PB_ARGS                                                                                     \
   h->g, h->ig, h->sg, h->st[stbuf], h->lb[work_list], h->lb[hist_list], h->posf, h->own, h->own_s,    \
       h->carry, h->bw_count, h->bw_rec, h->spart, h->status, h->perm
   if (pb4)
     k_pairs_pb<true, 4, EXT, false><<<pbg, kPairThreads, 0, h->stream>>>(DSS_PB_ARGS);
-  else if (pbal && mixed && pers)
+  else if (mixed && pers)
     k_pairs_pb<true, 3, EXT, true><<<pbg, kPairThreads, 0, h->stream>>>(DSS_PB_ARGS);
-  else if (pbal && mixed)
+  else if (mixed)
     k_pairs_pb<true, 3, EXT, false><<<pbg, kPairThreads, 0, h->stream>>>(DSS_PB_ARGS);
-  else if (pbal && pers)
+  else if (pers)
     k_pairs_pb<false, 2, EXT, true><<<pbg, kPairThreads, 0, h->stream>>>(DSS_PB_ARGS);
-  else if (pbal)
+  else
     k_pairs_pb<false, 2, EXT, false><<<pbg, kPairThreads, 0, h->stream>>>(DSS_PB_ARGS);
 #undef DSS_PB_ARGS
-  else if (mixed && big)
-    k_pairs<true, 4, EXT><<<pb, kPairThreads, 0, h->stream>>>(
-        h->g, h->ig, h->sg, h->st[stbuf], h->lb[work_list], h->lb[hist_list], h->posf, h->own, h->bw_count,
-        h->bw_rec, h->spart, h->status, h->perm);
-  else if (mixed)
-    k_pairs<true, 3, EXT><<<pb, kPairThreads, 0, h->stream>>>(
-        h->g, h->ig, h->sg, h->st[stbuf], h->lb[work_list], h->lb[hist_list], h->posf, h->own, h->bw_count,
-        h->bw_rec, h->spart, h->status, h->perm);
-  else
-    k_pairs<false, 2, EXT><<<pb, kPairThreads, 0, h->stream>>>(
-        h->g, h->ig, h->sg, h->st[stbuf], h->lb[work_list], h->lb[hist_list], h->posf, h->own, h->bw_count,
-        h->bw_rec, h->spart, h->status, h->perm);
   prof_mark(h, 6);
   const int gb = (n + kThreads - 1) / kThreads + h->g.K;
-  const void* carry = pbal ? h->carry : nullptr;
-  const int pbb = pbal ? pbg : 0;
-  const void* own_s = pbal && pers ? h->own_s : nullptr;
+  const void* carry = h->carry;
+  const int pbb = pbg;
+  const void* own_s = pers ? h->own_s : nullptr;
   if (own_s) {
     if (mixed)
       k_owner_stress<true, EXT><<<h->g.K * kOsParts, kPairThreads, 0, h->stream>>>(

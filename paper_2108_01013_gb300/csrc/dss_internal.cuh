@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "../../include/dss.h"
 
 #define DSS_PI 3.14159265358979323846
@@ -89,6 +91,9 @@ struct InstGeo {
   int cell_base, ncell;        // first bin and bins (= classes x ncell_layer)
   int ncell_layer;             // cells of one class layer (nc[0] nc[1] nc[2])
   int p_begin, p_end;
+  // the staged search (enum_plan): cells of a segment, segments of a row of
+  // cells, blocks of a segment, the instance's first block
+  int enum_seg, enum_hx, enum_subs, enum_blk;
   double gdot, gn;              // shear rate, normal dashpot
   float gdot_f, gn_f;
   double sumA3;                 // sum of a^3 (Einstein stresslet of Eq. 9)
@@ -337,6 +342,14 @@ __device__ __forceinline__ unsigned long long dev_ns() {
   return t;
 }
 
+// A status word as another block last wrote it (from L2; the word carries its
+// value with its flag, so no ordering beyond it is needed).
+__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+
 __device__ __forceinline__ int lookback_warp(unsigned long long* status, int tile, int agg,
                                              DevStatus* st) {
   const int lane = threadIdx.x & 31;
@@ -351,7 +364,7 @@ __device__ __forceinline__ int lookback_warp(unsigned long long* status, int til
   long long spins = 0;
   while (true) {
     const int idx = t - lane;                 // lane 0: nearest predecessor
-    const unsigned long long w = idx >= 0 ? atomicAdd(&status[idx], 0ull) : 0ull;
+    const unsigned long long w = idx >= 0 ? ld_relaxed(&status[idx]) : 0ull;
     const unsigned f = (unsigned)(w >> 32);
     const unsigned not_ready = __ballot_sync(0xffffffffu, f == 0u);
     const unsigned pre = __ballot_sync(0xffffffffu, f == 2u);
@@ -366,7 +379,7 @@ __device__ __forceinline__ int lookback_warp(unsigned long long* status, int til
         if (lane == 0) set_err(st, DSS_ERR_TIMEOUT);
         break;
       }
-      __nanosleep(20);
+      __nanosleep(64);
       continue;
     }
     int v = (lane <= p && idx >= 0) ? (int)(unsigned)(w & 0xffffffffull) : 0;
@@ -609,13 +622,11 @@ struct dss_handle {
                      // batched instances also the stresslet, 15 + 15)
   void* own_s;       // batched instances: 9n, each owner's stresslet sum (Eq. 9)
   int pb_blocks;     // blocks of the pair-balanced pair kernel (0: owner rows)
-  bool compact_ok[2];  // the list's compact pair arrays were written by its last enumeration
-                       // (false after the pair buffers are reallocated)
   int* bw_count;     // n: records appended to each particle's partner row
   void* bw_rec;      // n*M slots of 8 values: partner force (3), torque (3), owner index
   int64_t pcap;
   // stress
-  double* spart;     // 18 per pair block: stresslet sums for the block's first instance and the next
+  double* spart;     // 9 per pair block (batched instances: per stress slice): stresslet sums
   int spart_blocks;
   double* sigma;     // 9K: stress of each instance at the last force pass
   double* sigma_sum; // 9K: sum over committed steps since the last reset
@@ -645,9 +656,14 @@ struct dss_handle {
   bool multi_ok[4];
   // kernel shapes chosen by dss_autotune_kernels (0: the built-in rule):
   // resident pair blocks per SM the register budget is cut for (3 or 4), and
-  // candidates loaded ahead in the enumeration's loop (1 or 4)
+  // the enumeration's search (1: walked by owner, 4: staged by segments)
   int tune_pairs_minb;
   int tune_enum_unr;
+  // the enumeration's launch (enum_plan)
+  bool enum_walk;
+  int64_t enum_blocks;
+  int* enum_inst;            // instance of each of its blocks (batched instances; else null)
+  int64_t enum_inst_cap;
   int64_t bytes;
   int64_t host_steps_done;
   AdjBuf* adj;               // adjoint buffers (allocated by dss_adjoint)
@@ -671,7 +687,7 @@ int pair_grid_blocks(const dss_handle* h);
 int pair_pb_blocks(const dss_handle* h);
 void launch_scan(dss_handle* h, const int* in, int* out, int count, int which, bool zero_in);
 int scan_tiles_for(int count);
-int enum_tiles_for(int n);
+int64_t enum_plan(dss_handle* h, std::vector<int>* blk_inst);
 double echem_range(const dss_params* p);
 int enum_scan_tiles_for(int n);
 int bw_slot_values();

@@ -7,13 +7,34 @@
 // candidates within the rounding band of the cutoff are decided by the exact
 // FP64 predicate, so the pair set is the FP64 brute-force set bit for bit.
 //
-// The exclusive scan of the row lengths (the pair offsets of each owner) is
-// fused into the same kernel with a single-pass decoupled look-back over
-// warps (32 owners each) of blocks taken in launch order.
+// Two searches give the same pairs.  On sparse grids and with size classes a
+// thread walks its owner's stencil (k_enumerate, k_enumerate_classes), and the
+// exclusive scan of the row lengths (the pair offsets of each owner) is fused
+// into the kernel with a single-pass decoupled look-back over warps (32 owners
+// each) of blocks taken in launch order.  On crowded grids a block takes the
+// owners of a few cells and stages the candidates of their stencils in shared
+// memory (k_enumerate_seg); k_rows then scans the rows' lengths.
+#include <algorithm>
+#include <climits>
+#include <cmath>
+#include <vector>
+
 #include "dss_internal.cuh"
 
 namespace {
 constexpr int kThreads = 128;
+constexpr int kRows = 5;           // rows of cells in the half stencil, a warp each
+constexpr int kTile = 128;         // candidates of a row staged at a time
+constexpr int kSegMax = 28;        // cells of a segment (its stencil rows span three more)
+constexpr int kRowThreads = 256;   // row pass
+
+// Cutoffs of the pair (i, j) in FP32, linear in the radii: s = (a_i + a_j) sc + sd
+// (the listing range) and (a_i + a_j) lc + ld (the lubrication range, row
+// order only).  ECH: the listing range is the larger of s and a_i + a_j + de.
+// The FP32 cutoff is within a few ulp of the exact one, far inside the margin.
+struct EnumCut {
+  float sc, sd, lc, ld, de;
+};
 
 // Per-owner state of the enumeration; everything the candidate loop reads is
 // held in registers.
@@ -23,12 +44,10 @@ struct EnumCtx {
   float sc, sa;     // cutoff of pair (i, j): s = a_j sc + sa (a_i + a_j + delta)
   float sa2;        // with electro-chemical forces the cutoff is max(s, a_j + sa2)
   float m2;         // r^2 margin of the FP32 decision
-  float lc, la;     // lubrication cutoff of pair (i, j): a_j lc + la (row order only)
   float hx, hy, hz; // half box: a separation beyond it is decided exactly
   bool img;         // the stencil reaches past half the box along some axis
   int M;
   int cnt;
-  int nnear;        // SPLIT rows: pairs within the lubrication range, at the row's front
   int band;
   int* row;
   // exact FP64 decision
@@ -41,29 +60,12 @@ struct EnumCtx {
 
 __device__ __forceinline__ void enum_init(EnumCtx& e, const Geo& g, const InstGeo& I, const StateBuf& s,
                                           const float4* __restrict__ posf, int i, double off, int* row,
-                                          int reach) {
+                                          int reach, const EnumCut& q) {
   e.posf = posf;
   e.pi = posf[i];
-  // delta of Sec. II A: a fixed multiple of a0 (mode 1) or of the mean
-  // radius (mode 0); the FP32 cutoff is within a few ulp of the exact one,
-  // far inside the margin
-  if (g.mode == 1) {
-    e.sc = 1.0f;
-    e.sa = e.pi.w + (float)(g.delta * g.a0 > g.de ? g.delta * g.a0 : g.de);
-  } else {
-    e.sc = 1.0f + 0.5f * (float)g.delta;
-    e.sa = e.pi.w * e.sc;
-  }
-  // the electro-chemical range (a surface distance): a_i + a_j + de
-  e.sa2 = e.pi.w + (float)g.de;
-  if (g.mode == 1) {
-    e.lc = 1.0f;
-    e.la = e.pi.w + (float)(g.delta * g.a0);
-  } else {
-    e.lc = 1.0f + 0.5f * (float)g.delta;
-    e.la = e.pi.w * e.lc;
-  }
-  e.nnear = 0;
+  e.sc = q.sc;
+  e.sa = fmaf(e.pi.w, q.sc, q.sd);
+  e.sa2 = e.pi.w + q.de;
   e.m2 = I.r2_margin;
   e.hx = I.halfLf[0];
   e.hy = I.halfLf[1];
@@ -86,28 +88,13 @@ __device__ __forceinline__ void enum_init(EnumCtx& e, const Geo& g, const InstGe
 // One candidate j of owner i (positions relative to the candidate cell's
 // origin): FP32 decision on cell-local coordinates, certainly a pair,
 // certainly not, or (within the margin of the cutoff, or past half the box)
-// the exact FP64 predicate; a pair is appended to the row.  SPLIT (pairs
-// listed beyond the lubrication range, i.e. with electro-chemical forces):
-// pairs within the lubrication range by an FP32 test go to the row's front
-// in visiting order, the others to its back from the end; the row is closed
-// up afterwards (close_row).  Only the order within the row changes.
-// r^2 - s^2 of a candidate in FP32 on cell-local coordinates (s: the
-// pair's cutoff), the one value every decision starts from.
+// the exact FP64 predicate; a pair is appended to the row.
 template <bool ECH>
-__device__ __forceinline__ float cand_t(const EnumCtx& e, float4 pj, float px, float py, float pz, float& dx,
-                                       float& dy, float& dz) {
-  dx = pj.x - px;
-  dy = pj.y - py;
-  dz = pj.z - pz;
+__device__ __forceinline__ void take_candidate(EnumCtx& e, float4 pj, int j, float px, float py, float pz) {
+  const float dx = pj.x - px, dy = pj.y - py, dz = pj.z - pz;
   float sv = fmaf(pj.w, e.sc, e.sa);
   if (ECH) sv = fmaxf(sv, pj.w + e.sa2);
-  return fmaf(-sv, sv, fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
-}
-
-template <bool ECH, bool SPLIT>
-__device__ __forceinline__ void take_candidate(EnumCtx& e, float4 pj, int j, float px, float py, float pz) {
-  float dx, dy, dz;
-  const float t = cand_t<ECH>(e, pj, px, py, pz, dx, dy, dz);
+  const float t = fmaf(-sv, sv, fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
   // nearly every candidate lies beyond the cutoff by more than the margin:
   // one test and out (the half-box image test only on boxes narrower than
   // the stencil)
@@ -125,72 +112,17 @@ __device__ __forceinline__ void take_candidate(EnumCtx& e, float4 pj, int j, flo
                         s.x[n + j], s.x[2 * n + j], s.a[j]) ? 1 : 0;
   }
   if (dec) {
-    if (SPLIT) {
-      const float sl = fmaf(pj.w, e.lc, e.la);
-      const bool near = fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < sl * sl;
-      if (e.cnt < e.M) e.row[near ? e.nnear : e.M - 1 - (e.cnt - e.nnear)] = j;
-      e.nnear += near;
-    } else {
-      if (e.cnt < e.M) e.row[e.cnt] = j;
-    }
+    if (e.cnt < e.M) e.row[e.cnt] = j;
     ++e.cnt;
   }
 }
 
-// SPLIT rows: the far block [M - nf, M) moves down to follow the near block
-// (ascending, each entry read before any write reaches it: the source index
-// exceeds the destination by the gap).  Overflowing rows are left as they
-// are (the step is not committed).
-__device__ __forceinline__ void close_row(EnumCtx& e) {
-  if (e.cnt > e.M) return;
-  const int nf = e.cnt - e.nnear;
-  const int gap = e.M - e.cnt;
-  if (nf > 0 && gap > 0)
-    for (int k = 0; k < nf; ++k) e.row[e.nnear + k] = e.row[e.nnear + gap + k];
-}
-
-// SCREEN: the candidates of a range go 32 at a time through a screen first:
-// the one-test rejection alone, unrolled with four loads ahead and no branch
-// in the body, leaves a bit per candidate that may be a pair (about one in a
-// hundred on the polydisperse packings); those take the full decision
-// afterwards in ascending order, so the row is the one the plain loop
-// writes.  It pays on cells of three or more particles (1M log-uniform
-// [1, 10]: 247 -> 212 us; Table 5, radius ratio 3: 59 -> 47 us); on the
-// sparse 100k grid (1.7 per cell) the plain loop is faster (28.7 against
-// 30.7 us).
-template <bool ECH, bool SPLIT>
-__device__ __forceinline__ void scan_screened(EnumCtx& e, int jb, int je, float px, float py, float pz) {
-  for (int base = jb; base < je; base += 32) {
-    const int cnt = min(32, je - base);
-    const float4* __restrict__ q = e.posf + base;
-    unsigned m = 0u;
-#pragma unroll 4
-    for (int k = 0; k < cnt; ++k) {
-      float dx, dy, dz;
-      const float t = cand_t<ECH>(e, __ldg(q + k), px, py, pz, dx, dy, dz);
-      m |= (t > e.m2 ? 0u : 1u) << k;
-    }
-    while (m) {
-      const int k = __ffs(m) - 1;
-      m &= m - 1u;
-      take_candidate<ECH, SPLIT>(e, __ldg(q + k), base + k, px, py, pz);
-    }
-  }
-}
-
 // Visits the candidates [jb, je) of one stencil cell (origin displaced by
-// (cxo, cyo, czo) from the owner's cell) in order, plainly or (SCREEN) through
-// the screen; boxes narrower than the stencil, where every candidate takes
-// the image test, always take the plain loop.  Both make the same decisions
-// in the same order, so the rows are identical.
-template <bool ECH, bool SCREEN, bool SPLIT = false>
+// (cxo, cyo, czo) from the owner's cell) in order.
+template <bool ECH>
 __device__ __forceinline__ void scan_range(EnumCtx& e, int jb, int je, float cxo, float cyo, float czo) {
   const float px = e.pi.x - cxo, py = e.pi.y - cyo, pz = e.pi.z - czo;
-  if (SCREEN && !e.img) {
-    scan_screened<ECH, SPLIT>(e, jb, je, px, py, pz);
-    return;
-  }
-  for (int j = jb; j < je; ++j) take_candidate<ECH, SPLIT>(e, __ldg(e.posf + j), j, px, py, pz);
+  for (int j = jb; j < je; ++j) take_candidate<ECH>(e, __ldg(e.posf + j), j, px, py, pz);
 }
 
 // Row lengths, counters and the fused exclusive scan of the row lengths:
@@ -240,12 +172,12 @@ __device__ __forceinline__ void finish_rows(const Geo& g, const StateBuf& s, Lis
   }
 }
 
-template <bool ECH, bool SCREEN, bool SPLIT>
+template <bool ECH>
 __global__ void __launch_bounds__(kThreads, 8)
 k_enumerate(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sgk, StateBuf s,
             const float4* __restrict__ posf, const int* __restrict__ cellid,
             const int* __restrict__ cell_start, ListBuf L, int* __restrict__ bw_count,
-            unsigned long long* scan_status, int* scan_ticket, DevStatus* st, int adv) {
+            unsigned long long* scan_status, int* scan_ticket, DevStatus* st, EnumCut q) {
   if (dev_err(st)) return;
   __shared__ int s_tile;
   if (threadIdx.x == 0) s_tile = atomicAdd(scan_ticket, 1);
@@ -260,7 +192,7 @@ k_enumerate(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ s
     const int inst = s.inst[i];
     const InstGeo& I = ig[inst];
     const StepGeo sg = sgk[inst];
-    enum_init(e, g, I, s, posf, i, sg.off, L.list + (int64_t)i * g.Ms, 1);
+    enum_init(e, g, I, s, posf, i, sg.off, L.list + (int64_t)i * g.Ms, 1, q);
     const int fsh = sg.fsh;
     const float offr = sg.offr_hi;
     const int nx = I.nc[0], ny = I.nc[1], nz = I.nc[2];
@@ -272,17 +204,17 @@ k_enumerate(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ s
     const int xm = cx == 0 ? nx - 1 : cx - 1, xp = cx + 1 == nx ? 0 : cx + 1;
     const int zm = cz == 0 ? nz - 1 : cz - 1, zp = cz + 1 == nz ? 0 : cz + 1;
     // own cell (partners after i) and the cell x+1
-    scan_range<ECH, SCREEN, SPLIT>(e, i + 1, cell_start[cb + c + 1], 0.f, 0.f, 0.f);
+    scan_range<ECH>(e, i + 1, cell_start[cb + c + 1], 0.f, 0.f, 0.f);
     {
       const int q = cb + (cz * ny + cy) * nx + xp;
-      scan_range<ECH, SCREEN, SPLIT>(e, cell_start[q], cell_start[q + 1], I.csf[0], 0.f, 0.f);
+      scan_range<ECH>(e, cell_start[q], cell_start[q + 1], I.csf[0], 0.f, 0.f);
     }
     // layer y, z+1: three x cells
     {
       const int row = cb + (zp * ny + cy) * nx;
-      scan_range<ECH, SCREEN, SPLIT>(e, cell_start[row + xm], cell_start[row + xm + 1], -I.csf[0], 0.f, I.csf[2]);
-      scan_range<ECH, SCREEN, SPLIT>(e, cell_start[row + cx], cell_start[row + cx + 1], 0.f, 0.f, I.csf[2]);
-      scan_range<ECH, SCREEN, SPLIT>(e, cell_start[row + xp], cell_start[row + xp + 1], I.csf[0], 0.f, I.csf[2]);
+      scan_range<ECH>(e, cell_start[row + xm], cell_start[row + xm + 1], -I.csf[0], 0.f, I.csf[2]);
+      scan_range<ECH>(e, cell_start[row + cx], cell_start[row + cx + 1], 0.f, 0.f, I.csf[2]);
+      scan_range<ECH>(e, cell_start[row + xp], cell_start[row + xp + 1], I.csf[0], 0.f, I.csf[2]);
     }
     // layer y+1: 3x3 cells, or across y = L_y the 4 x cells covering the
     // image range shifted by the Lees-Edwards offset
@@ -297,11 +229,10 @@ k_enumerate(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ s
         const int q = cb + (qz * ny + qy) * nx + qx;
         float cxo, cyo, czo;
         stencil_shift(I, ox, 1, oz, le ? 1 : 0, fsh, offr, cxo, cyo, czo);
-        scan_range<ECH, SCREEN, SPLIT>(e, cell_start[q], cell_start[q + 1], cxo, cyo, czo);
+        scan_range<ECH>(e, cell_start[q], cell_start[q + 1], cxo, cyo, czo);
       }
     }
   }
-  if (SPLIT && i < n) close_row(e);
   finish_rows(g, s, L, bw_count, scan_status, st, e, i, tile * (kThreads / 32) + (threadIdx.x >> 5));
 }
 
@@ -319,7 +250,7 @@ __global__ void __launch_bounds__(kThreads, 8)
 k_enumerate_classes(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sgk, StateBuf s,
                     const float4* __restrict__ posf, const int* __restrict__ cellid,
                     const int* __restrict__ cell_start, ListBuf L, int* __restrict__ bw_count,
-                    unsigned long long* scan_status, int* scan_ticket, DevStatus* st) {
+                    unsigned long long* scan_status, int* scan_ticket, DevStatus* st, EnumCut q) {
   if (dev_err(st)) return;
   __shared__ int s_tile;
   if (threadIdx.x == 0) s_tile = atomicAdd(scan_ticket, 1);
@@ -334,7 +265,7 @@ k_enumerate_classes(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __rest
     const int inst = s.inst[i];
     const InstGeo& I = ig[inst];
     const StepGeo sg = sgk[inst];
-    enum_init(e, g, I, s, posf, i, sg.off, L.list + (int64_t)i * g.Ms, g.reach);
+    enum_init(e, g, I, s, posf, i, sg.off, L.list + (int64_t)i * g.Ms, g.reach, q);
     const int fsh = sg.fsh;
     const float offr = sg.offr_hi;
     const int nx = I.nc[0], ny = I.nc[1], nz = I.nc[2];
@@ -343,7 +274,7 @@ k_enumerate_classes(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __rest
     const int c = (cellid[i] - I.cell_base) % layer;
     const int cx = c % nx, cy = (c / nx) % ny, cz = c / (nx * ny);
     // own bin, partners after i
-    scan_range<ECH, false>(e, i + 1, cell_start[cellid[i] + 1], 0.f, 0.f, 0.f);
+    scan_range<ECH>(e, i + 1, cell_start[cellid[i] + 1], 0.f, 0.f, 0.f);
     for (int c2 = cls; c2 >= 0; --c2) {
       const int R = g.rtab[cls][c2];
       const bool half = c2 == cls;
@@ -389,7 +320,7 @@ k_enumerate_classes(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __rest
                   } while (j >= kend);
                   stencil_shift(I, ox + k, oy, oz, le, fsh, offr, cxo, cyo, czo);
                 }
-                scan_range<ECH, false>(e, j, j + 1, cxo, cyo, czo);
+                scan_range<ECH>(e, j, j + 1, cxo, cyo, czo);
               }
             }
             ox += m;
@@ -400,42 +331,497 @@ k_enumerate_classes(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __rest
   }
   finish_rows(g, s, L, bw_count, scan_status, st, e, i, tile * (kThreads / 32) + (threadIdx.x >> 5));
 }
+
+// Exact decision of (i, j) (out of line: about one candidate in a thousand).
+__device__ __noinline__ bool decide_exact(const Geo& g, const InstGeo& I, const StateBuf& s, double off, int i,
+                                          int j) {
+  const int n = g.n;
+  return exact_is_pair(g, I, off, s.x[i], s.x[n + i], s.x[2 * n + i], s.a[i], s.x[j], s.x[n + j], s.x[2 * n + j],
+                       s.a[j]);
+}
+
+// ------------------------------------------------------------------------
+// Segment walk.  One block per segment: seg consecutive x cells of one row of
+// cells, as many as hold about 26 particles (one cell on dense grids, then
+// shared by several blocks), a lane per owner.  The half stencil of the
+// segment is five rows of adjacent cells, each one or (across x = L_x) two
+// pieces of the sorted order: its own row from the segment on, the z+1 row and
+// the three rows of layer y+1 (across y = L_y one x cell more, shifted by the
+// Lees-Edwards offset).  A warp takes one of them: it reads the cell offsets,
+// stages the particles in shared memory relative to the segment's origin,
+// kTile at a time, and each lane runs over its own cells' part of them.
+//
+// What bounds it is the issue slots (2.4 to 2.9 instructions a cycle and SM):
+// a candidate is loaded once for 32 owners instead of once for each, and costs
+// a lane 11 instructions, one of them a shared load; the set-up of a block is
+// worth half a pass of 32 owners.  Against the walk by owner with the same
+// screen (one box, mixed precision, with the row pass): Table 5 with the 4 a0
+// range (128 per cell, 2.9M pairs) 312 -> 179 us, 1M log-uniform [1, 10] (7.1
+// per cell) 220 -> 199, the 100k packing with the 1 a0 range (4.1 per cell) 40
+// -> 38.  On sparse grids the set-up does not pay: 100k (1.7 per cell) 28
+// against 37 us, a batch of 64 (1.8) 106 against 202.
+//
+// The decision: u = r^2 - s^2 in FP32, its sign bit shifted into a mask, 32
+// candidates at a time without a branch, with the smallest |u| beside it.  A
+// lane whose smallest |u| lies within the margin (1e-4 cell^2; positions up
+// to 31 cells from the origin round to 2e-6 cell, u near the cutoff to
+// 1e-5 cell^2) takes those candidates again with the exact FP64 predicate.  A
+// box narrower than twice the stencil (img) takes every candidate again, and
+// separations beyond half the box exactly too.
+//
+// An owner's row lists the pairs of the five rows of cells in turn, ascending
+// within each (tile by tile on dense grids): the warps exchange the owners'
+// counts and write their own part.  SPLIT (pairs listed beyond the lubrication
+// range, with electro-chemical forces): pairs within the lubrication range by
+// an FP32 test go to the row's front, the others to its back from the end;
+// k_rows closes the row up.
+// ------------------------------------------------------------------------
+template <bool ECH, bool SPLIT, bool ONE>
+__global__ void __launch_bounds__(32 * kRows, 6)
+k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I1, const InstGeo* __restrict__ ig,
+            const StepGeo* __restrict__ sgk, const __grid_constant__ StateBuf s, const float4* __restrict__ posf,
+            const int* __restrict__ cellid, const int* __restrict__ cell_start, int* __restrict__ list,
+            int* __restrict__ count, int* __restrict__ nnear, const int* __restrict__ blk_inst, DevStatus* st,
+            EnumCut q) {
+  __shared__ float4 s_c[kRows][kTile + 4];
+  __shared__ int s_j[kRows][kTile];
+  __shared__ int s_off[kRows][32];
+  __shared__ int s_len[kRows];
+  __shared__ int s_cnt[2][kRows][32];      // pairs of each owner in each row (near ones << 16: SPLIT)
+  __shared__ int4 s_par[kRows];            // rows: bin of their x = 0, x of their first cell, cells, image across y
+  __shared__ int s_seg[4];                 // first bin, cells, part, first owner
+  if (dev_err(st)) return;
+  const int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
+  const int inst = ONE ? 0 : blk_inst[blockIdx.x];
+  const InstGeo& I = ONE ? I1 : ig[inst];
+  const StepGeo sg = sgk[inst];
+  const int nx = I.nc[0], ny = I.nc[1], nz = I.nc[2];
+  if (r == 0) {
+    // the first warp finds the segment, a lane for each of its rows
+    unsigned item = blockIdx.x - (ONE ? 0 : I.enum_blk);
+    const int seg = I.enum_seg, subs = I.enum_subs;
+    int sub = 0;
+    if (subs > 1) {
+      const unsigned h = item / (unsigned)subs;
+      sub = (int)(item - h * subs);
+      item = h;
+    }
+    const int row = (int)(item / (unsigned)I.enum_hx);
+    const int x0 = ((int)item - row * I.enum_hx) * seg;
+    const int cz = row / ny, cy = row - cz * ny;
+    const int bxe = min(seg, nx - x0);
+    const bool img = lane >= 2 && cy == ny - 1;
+    int xf = lane == 0 ? x0 : (img ? wrapi(x0 - 2 - sg.fsh, nx) : x0 - 1);
+    if (xf < 0) xf += nx;
+    const int qy = lane < 2 ? cy : (cy == ny - 1 ? 0 : cy + 1);
+    int qz = lane == 0 ? cz : (lane == 1 ? cz + 1 : cz + lane - 3);
+    qz = qz < 0 ? nz - 1 : (qz == nz ? 0 : qz);
+    if (lane < kRows)
+      s_par[lane] = make_int4(I.cell_base + (qz * ny + qy) * nx, xf, bxe + (lane == 0 ? 1 : (img ? 3 : 2)), img);
+    if (lane == 0) {
+      s_seg[0] = I.cell_base + row * nx + x0;
+      s_seg[1] = bxe;
+      s_seg[2] = sub + 1 < subs ? sub : -1 - sub;
+    }
+  }
+  __syncthreads();
+  // the warp's row: w cells from x = xf on, of the row of cells at rc
+  const int4 par = s_par[r];
+  const int rc = par.x, xf = par.y, w = par.z;
+  const bool le = par.w != 0;
+  // lane k: the boundary before its cell k, as a place in the row's sequence;
+  // place p is particle first + p, or beyond x = L_x (p >= n1) first + wrap + p
+  const int xk = xf + min(lane, w);
+  int b = cell_start[rc + (xk <= nx ? xk : xk - nx)];
+  const int first = __shfl_sync(0xffffffffu, b, 0);
+  int n1 = INT_MAX, wrap = 0;
+  if (xf + w > nx) {
+    const int row0 = cell_start[rc];
+    n1 = cell_start[rc + nx] - first;
+    wrap = row0 - n1 - first;
+    b = xk <= nx ? b - first : b - row0 + n1;
+  } else {
+    b -= first;
+  }
+  s_off[r][lane] = b;
+  const int len = __shfl_sync(0xffffffffu, b, w);
+  if (lane == 0) {
+    s_len[r] = len;
+    if (r == 0) s_seg[3] = first;
+  }
+  __syncthreads();
+  const int c0 = s_seg[0], part = s_seg[2], hs = s_seg[3], he = hs + s_off[0][s_seg[1]];
+  const int o_beg = hs + 32 * (part < 0 ? -1 - part : part), o_end = part < 0 ? he : min(o_beg + 32, he);
+  const int most = max(max(max(s_len[0], s_len[1]), max(s_len[2], s_len[3])), s_len[4]);
+  const float kx0 = r == 0 ? 0.f : (le ? -2.f : -1.f), sx = le ? sg.offr_hi : 0.f;
+  const float sy = r < 2 ? 0.f : I.csf[1];
+  const float sz = r == 0 ? 0.f : (r == 1 ? I.csf[2] : (float)(r - 3) * I.csf[2]);
+  // separations stay below half the box when it is wider than twice the
+  // stencil's reach (two cells, three across y = L_y; plus one cell of slack)
+  const bool img = nx < 7 || ny < 5 || nz < 5;
+  const float m2 = I.r2_margin;
+  int buf = 0, band = 0;
+  for (int o0 = o_beg; o0 < o_end; o0 += 32) {
+    // the lane's owner and its part [lo, hi) of the row
+    const int i = o0 + lane;
+    const bool in = i < o_end;
+    float px = 0.f, py = 0.f, pz = 0.f, pa = 0.f, sa = 0.f;
+    int lo = 0, hi = 0;
+    if (in) {
+      const float4 p = posf[i];
+      const int kx = cellid[i] - c0;
+      px = fmaf((float)kx, I.csf[0], p.x);
+      py = p.y;
+      pz = p.z;
+      pa = p.w;
+      sa = fmaf(p.w, q.sc, q.sd);
+      lo = r == 0 ? i - hs + 1 : s_off[r][kx];
+      hi = s_off[r][kx + (r == 0 ? 2 : (le ? 4 : 3))];
+    }
+    int* rw = list + (int64_t)i * g.Ms;
+    int pairs = 0, near = 0;    // of the owner, in the tiles so far
+    for (int t0 = 0; t0 < most; t0 += kTile) {
+      const int t1 = min(t0 + kTile, len);
+      if (o0 == o_beg || most > kTile) {     // (a single tile stays for the next owners)
+        __syncwarp();
+        for (int p = t0 + lane; p < t1; p += 32) {
+          const int j = first + p + (p < n1 ? 0 : wrap);
+          const float4 c = __ldg(posf + j);
+          int kc = __ldg(cellid + j) - rc - xf;
+          if (kc < 0) kc += nx;
+          s_c[r][p - t0] = make_float4(c.x + fmaf((float)kc + kx0, I.csf[0], sx), c.y + sy, c.z + sz, c.w);
+          s_j[r][p - t0] = j;
+        }
+        __syncwarp();
+      }
+      const int a = max(lo, t0) - t0, z = min(hi, t1) - t0;
+      unsigned hit[kTile / 32];
+#pragma unroll
+      for (int h = 0; h < kTile / 32; ++h) {
+        const int m = min(32, z - a - 32 * h);
+        hit[h] = 0u;
+        if (m <= 0) continue;
+        const float4* __restrict__ c = &s_c[r][a + 32 * h];
+        float least = __int_as_float(0x7f800000);
+        int n = 0;
+        do {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const float4 pj = c[n + u];   // up to three past the end: masked off below
+            const float dx = pj.x - px, dy = pj.y - py, dz = pj.z - pz;
+            float sv = fmaf(pj.w, q.sc, sa);
+            if (ECH) sv = fmaxf(sv, pj.w + (pa + q.de));
+            const float t = fmaf(-sv, sv, fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
+            hit[h] = __funnelshift_l(__float_as_uint(t), hit[h], 1);
+            least = fminf(least, fabsf(t));
+          }
+          n += 4;
+        } while (n < m);
+        hit[h] <<= 32 - n;                          // candidate b at bit 31 - b
+        const unsigned all = ~(m < 32 ? 0xffffffffu >> m : 0u);
+        hit[h] &= all;
+        if (least <= m2 || img) {
+          for (unsigned left = all; left;) {
+            const int e = __clz(left);
+            const unsigned bit = 0x80000000u >> e;
+            left &= ~bit;
+            const float4 pj = c[e];
+            const float dx = pj.x - px, dy = pj.y - py, dz = pj.z - pz;
+            float sv = fmaf(pj.w, q.sc, sa);
+            if (ECH) sv = fmaxf(sv, pj.w + (pa + q.de));
+            const float t = fmaf(-sv, sv, fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
+            if (!(fabsf(t) > m2) ||
+                (img && (fabsf(dx) > I.halfLf[0] || fabsf(dy) > I.halfLf[1] || fabsf(dz) > I.halfLf[2]))) {
+              ++band;
+              if (decide_exact(g, I, s, sg.off, i, s_j[r][a + 32 * h + e])) hit[h] |= bit;
+              else hit[h] &= ~bit;
+            }
+          }
+        }
+      }
+      int mine = 0;
+      unsigned nrm[kTile / 32];
+#pragma unroll
+      for (int h = 0; h < kTile / 32; ++h) {
+        mine += __popc(hit[h]);
+        nrm[h] = 0u;
+        if (SPLIT) {
+          for (unsigned left = hit[h]; left;) {
+            const int e = __clz(left);
+            left &= ~(0x80000000u >> e);
+            const float4 pj = s_c[r][a + 32 * h + e];
+            const float dx = pj.x - px, dy = pj.y - py, dz = pj.z - pz;
+            const float sl = fmaf(pa + pj.w, q.lc, q.ld);
+            if (fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < sl * sl) nrm[h] |= 0x80000000u >> e;
+          }
+          mine += __popc(nrm[h]) << 16;
+        }
+      }
+      s_cnt[buf][r][lane] = mine;
+      __syncthreads();
+      int at = 0, tot = 0;
+#pragma unroll
+      for (int v = 0; v < kRows; ++v) {
+        if (v == r) at = tot;
+        tot += s_cnt[buf][v][lane];
+      }
+      buf ^= 1;
+      // the warp's part of the owner's row
+      int kn = SPLIT ? near + (at >> 16) : pairs + at, kf = SPLIT ? pairs - near + (at & 0xffff) - (at >> 16) : 0;
+#pragma unroll
+      for (int h = 0; h < kTile / 32; ++h)
+        for (unsigned left = hit[h]; left;) {
+          const int e = __clz(left);
+          const unsigned bit = 0x80000000u >> e;
+          left &= ~bit;
+          const int j = s_j[r][a + 32 * h + e];
+          if (SPLIT) {
+            if (kn + kf < g.M) rw[nrm[h] & bit ? kn : g.M - 1 - kf] = j;
+            if (nrm[h] & bit) ++kn; else ++kf;
+          } else {
+            if (kn < g.M) rw[kn] = j;
+            ++kn;
+          }
+        }
+      pairs += SPLIT ? tot & 0xffff : tot;
+      near += SPLIT ? tot >> 16 : 0;
+    }
+    if (r == 0 && in) {
+      count[i] = pairs;
+      if (SPLIT) nnear[i] = near;
+    }
+  }
+  if (__any_sync(0xffffffffu, band != 0)) {
+    band = __reduce_add_sync(0xffffffffu, band);
+    if (lane == 0) atomicAdd(&st->w[ST_BAND], band);
+  }
+}
+
+// Row pass: row lengths, counters, the id <-> row maps, the exclusive scan of
+// the row lengths (decoupled look-back over tiles of TILE owners) and the
+// compact pair arrays (owner and partner of every pair in owner order, the
+// order the pair kernel deals them out in), written by the block together,
+// coalesced; the first pairs are read while the first warp looks back.  SPLIT
+// rows are closed up in place here: the far block [M - far, M) moves down
+// behind the near one, ascending, every entry read before any write reaches
+// it (a source lies beyond its destination by the gap).  A kernel of its own:
+// with the look-back at the end of the search every block held its place
+// until the slowest before it was done (a third of the kernel at 1M).
+// TILE: 256 owners, or 64 where rows are long (a block's pairs are what its
+// time goes with).
+template <bool SPLIT, int TILE>
+__global__ void __launch_bounds__(kRowThreads)
+k_rows(int n, int M, int Ms, int64_t pcap, const int* __restrict__ ids, const __grid_constant__ ListBuf L,
+       const int* __restrict__ nnear, int* __restrict__ bw_count, unsigned long long* scan_status, int* scan_ticket,
+       DevStatus* st) {
+  constexpr int kAhead = 4;                  // pairs a thread reads before the offsets are known
+  __shared__ int s_tile, s_prefix;
+  __shared__ int s_warp[kRowThreads / 32];
+  __shared__ int s_ex[TILE + 1], s_near[SPLIT ? TILE : 1];
+  // (a block that saw an error takes no ticket: no tile waits for it)
+  if (threadIdx.x == 0) s_tile = dev_err(st) ? -1 : atomicAdd(scan_ticket, 1);
+  __syncthreads();
+  const int tile = s_tile, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (tile < 0) return;
+  const int i0 = tile * TILE, i = i0 + threadIdx.x;
+  const bool own = threadIdx.x < TILE && i < n;
+  const int cnt = own ? L.count[i] : 0;
+  const int v = min(cnt, M);
+  if (SPLIT && own) s_near[threadIdx.x] = min(nnear[i], v);
+  int incl = v;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += t;
+  }
+  if (lane == 31) s_warp[wid] = incl;
+  __syncthreads();
+  int before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < kRowThreads / 32; ++w) {
+    if (w < wid) before += s_warp[w];
+    total += s_warp[w];
+  }
+  if (threadIdx.x < TILE) s_ex[threadIdx.x] = before + incl - v;
+  if (threadIdx.x == 0) s_ex[TILE] = total;
+  __syncthreads();
+  // pair t of the tile: its owner (the last whose row starts at or before t)
+  // and its place there
+  auto find = [&](int t, int& o, int& k, int& src) {
+    o = 0;
+#pragma unroll
+    for (int step = TILE / 2; step >= 1; step >>= 1)
+      if (s_ex[o + step] <= t) o += step;
+    k = t - s_ex[o];
+    src = k;
+    if (SPLIT && k >= s_near[o]) src = M - (s_ex[o + 1] - s_ex[o]) + k;
+  };
+  int aj[kAhead], ao[kAhead], ak[kAhead];
+#pragma unroll
+  for (int r = 0; r < kAhead; ++r) {
+    const int t = threadIdx.x + r * kRowThreads;
+    aj[r] = -1;
+    ao[r] = 0;
+    ak[r] = -1;
+    if (t < total) {
+      int k, src;
+      find(t, ao[r], k, src);
+      aj[r] = L.list[(int64_t)(i0 + ao[r]) * Ms + src];
+      if (src != k) ak[r] = k;
+    }
+  }
+  if (wid == 0) {
+    const int prefix = lookback_warp(scan_status, tile, total, st);
+    if (lane == 0) {
+      s_prefix = prefix;
+      if (i0 + TILE >= n) L.start[n] = prefix + total;
+    }
+  }
+  const int wmax = __reduce_max_sync(0xffffffffu, cnt);
+  if (lane == 0 && wmax > *(volatile int*)&st->w[ST_MAXROW]) atomicMax(&st->w[ST_MAXROW], wmax);
+  if (own) {
+    if (cnt > M) {
+      L.count[i] = M;
+      set_err(st, DSS_ERR_CAPACITY);
+    }
+    bw_count[i] = 0;
+    const int id = ids[i];
+    L.slot_of_id[id] = i;
+    L.id_of_slot[i] = id;
+  }
+  __syncthreads();
+  const int base = s_prefix;
+  if (own) L.start[i] = base + before + incl - v;
+#pragma unroll
+  for (int r = 0; r < kAhead; ++r) {
+    const int t = threadIdx.x + r * kRowThreads;
+    if (t < total) {
+      if (base + t < pcap) {
+        L.pj[base + t] = aj[r];
+        L.pown[base + t] = i0 + ao[r];
+      }
+      if (SPLIT && ak[r] >= 0) L.list[(int64_t)(i0 + ao[r]) * Ms + ak[r]] = aj[r];
+    }
+  }
+  for (int t0 = kAhead * kRowThreads; t0 < total; t0 += kRowThreads) {
+    const int t = t0 + threadIdx.x;
+    int o = 0, k = 0, src = 0, j = 0;
+    if (t < total) {
+      find(t, o, k, src);
+      j = L.list[(int64_t)(i0 + o) * Ms + src];
+    }
+    if (SPLIT) __syncthreads();
+    if (t < total) {
+      if (base + t < pcap) {
+        L.pj[base + t] = j;
+        L.pown[base + t] = i0 + o;
+      }
+      if (SPLIT && src != k) L.list[(int64_t)(i0 + o) * Ms + k] = j;
+    }
+  }
+}
 }  // namespace
 
-int enum_tiles_for(int n) { return (n + kThreads - 1) / kThreads; }
-int enum_scan_tiles_for(int n) { return enum_tiles_for(n) * (kThreads / 32); }
+int enum_scan_tiles_for(int n) { return (n + kThreads - 1) / kThreads * (kThreads / 32); }
+
+// Expected passes of 32 owners over a segment of mean owners (Poisson counts).
+static double seg_passes(double mean) {
+  double e = 0.0, p = std::exp(-mean);   // p: probability of exactly k owners
+  for (int k = 1; k <= 4 * (int)mean + 64; ++k) {
+    p *= mean / k;
+    e += p * ((k + 31) / 32);
+  }
+  return e;
+}
+
+// The enumeration's kernel and launch for the current grid.  Grids of fewer
+// than four particles a cell, and of size classes, are walked by owner (the
+// two searches meet between 1.8 and 4.1 per cell, see k_enumerate_seg).
+// Segments are cut so that the cost per owner is smallest: a block's set-up is
+// worth about half a pass of 32 owners.  Cells of more than 26 particles are
+// shared by as many blocks as hold their average and a quarter more.  Per
+// instance: the segment's cells, the segments of a row of cells, the blocks of
+// a segment, the first block.  Returns the number of blocks (and their
+// instances, when asked for).
+int64_t enum_plan(dss_handle* h, std::vector<int>* blk_inst) {
+  h->enum_walk = h->g.nclass > 1 || h->tune_enum_unr == 1 ||
+                 (h->tune_enum_unr == 0 && h->n < 4 * (int64_t)h->g.ncell);
+  int64_t blk = 0;
+  if (blk_inst) blk_inst->clear();
+  for (int k = 0; k < h->K; ++k) {
+    InstGeo& I = h->ig_host[k];
+    const double per = (double)h->inst_n[k] / (double)I.ncell;
+    const int nx = I.nc[0];
+    int hx = nx;
+    I.enum_subs = 1;
+    if (per > 26.0) {
+      I.enum_subs = (int)std::min(std::ceil(1.25 * per / 32.0), 1024.0);
+    } else {
+      // (a row of the stencil holds each cell once: seg + 3 cells across
+      // y = L_y; and a row of it fits one tile)
+      double best = INFINITY;
+      for (int seg = 1; seg <= std::min(kSegMax, nx - 3) && (seg == 1 || per * (seg + 2) < 0.9 * kTile); ++seg) {
+        const int q = (nx + seg - 1) / seg;
+        const double mean = per * nx / q, cost = (0.5 + seg_passes(mean)) / mean;
+        if (cost < best) {
+          best = cost;
+          hx = q;
+        }
+      }
+    }
+    I.enum_hx = hx;
+    I.enum_seg = (nx + hx - 1) / hx;
+    I.enum_blk = (int)blk;
+    const int64_t items = (int64_t)hx * I.nc[1] * I.nc[2] * I.enum_subs;
+    if (blk_inst && !h->enum_walk) blk_inst->insert(blk_inst->end(), (size_t)items, k);
+    blk += items;
+  }
+  if (h->enum_walk) blk = (h->n + kThreads - 1) / kThreads;
+  h->enum_blocks = blk;
+  return blk;
+}
 
 void launch_enumerate(dss_handle* h, int stbuf, int dst_list, int adv) {
-  const int n = (int)h->n;
+  (void)adv;
   ListBuf& L = h->lb[dst_list];
+  const Geo& g = h->g;
   prof_mark(h, 4);
-  // the pair-mean lubrication cutoff and the electro-chemical range combine
-  // by a maximum, which only that case needs in the candidate test
-  const bool ech = h->g.de > 0.0 && h->g.mode == 0;
-  auto kc = ech ? k_enumerate_classes<true> : k_enumerate_classes<false>;
-  // cells holding many particles (long ranges, large radius ratios)
-  const bool crowded = h->tune_enum_unr ? h->tune_enum_unr == 4 : h->n >= 8 * (int64_t)h->g.ncell;
-  // with electro-chemical forces over crowded cells (long ranges) most
-  // listed pairs lie beyond the lubrication range: rows put the others
+  // FP32 cutoffs.  The electro-chemical range beats the pair-mean lubrication
+  // cutoff for every pair when it beats the largest; only between the two do
+  // both enter the candidate test.
+  EnumCut q;
+  const bool mean = g.mode == 0, wide = g.de > 0.0 && g.de >= g.delta * h->a_max;
+  q.sc = mean && !wide ? 1.0f + 0.5f * (float)g.delta : 1.0f;
+  q.sd = mean ? (wide ? (float)g.de : 0.0f) : (float)(g.delta * g.a0 > g.de ? g.delta * g.a0 : g.de);
+  q.lc = mean ? 1.0f + 0.5f * (float)g.delta : 1.0f;
+  q.ld = mean ? 0.0f : (float)(g.delta * g.a0);
+  q.de = (float)g.de;
+  const bool ech = g.de > 0.0 && mean && !wide;
+  // with electro-chemical forces over cells of many particles (long ranges)
+  // most listed pairs lie beyond the lubrication range: rows put the others
   // first, so that the pair kernel's warps meet runs of pairs without
   // lubrication (short rows gain less than the reordering costs)
-  const bool split = h->g.de > 0.0 && crowded;
-  // cells of three or more particles on average (the 1M log-uniform
-  // packing: 7.5; Table 5: 24) take the screened candidate loop; under two
-  // per cell (the 100k packing: 1.7) the plain loop is faster
-  const bool screen = crowded || (!h->tune_enum_unr && h->n >= 3 * (int64_t)h->g.ncell);
-  auto k1 = ech ? (split ? k_enumerate<true, true, true> : k_enumerate<true, false, false>)
-                : split  ? k_enumerate<false, true, true>
-                : screen ? k_enumerate<false, true, false>
-                         : k_enumerate<false, false, false>;
-  if (h->g.nclass > 1)
-    kc<<<enum_tiles_for(n), kThreads, 0, h->stream>>>(
-        h->g, h->ig, h->sg, h->st[stbuf], h->posf, h->cellid, h->cell_start, L, h->bw_count,
-        h->scan_status + h->scan_tiles_max, h->scan_ticket + 1, h->status);
-  else
-    k1<<<enum_tiles_for(n), kThreads, 0, h->stream>>>(
-        h->g, h->ig, h->sg, h->st[stbuf], h->posf, h->cellid, h->cell_start, L, h->bw_count,
-        h->scan_status + h->scan_tiles_max, h->scan_ticket + 1, h->status, adv);
+  const bool split = g.de > 0.0 && !h->enum_walk && h->n >= 8 * (int64_t)g.ncell;
+  const unsigned blocks = (unsigned)h->enum_blocks;
+  unsigned long long* status = h->scan_status + h->scan_tiles_max;
+  int* ticket = h->scan_ticket + 1;
+  if (h->enum_walk) {
+    auto kw = g.nclass > 1 ? (ech ? k_enumerate_classes<true> : k_enumerate_classes<false>)
+                           : (ech ? k_enumerate<true> : k_enumerate<false>);
+    kw<<<blocks, kThreads, 0, h->stream>>>(g, h->ig, h->sg, h->st[stbuf], h->posf, h->cellid, h->cell_start, L,
+                                           h->bw_count, status, ticket, h->status, q);
+  } else {
+    const bool one = h->K == 1;
+    auto ks = ech ? (split ? (one ? k_enumerate_seg<true, true, true> : k_enumerate_seg<true, true, false>)
+                           : (one ? k_enumerate_seg<true, false, true> : k_enumerate_seg<true, false, false>))
+                  : (split ? (one ? k_enumerate_seg<false, true, true> : k_enumerate_seg<false, true, false>)
+                           : (one ? k_enumerate_seg<false, false, true> : k_enumerate_seg<false, false, false>));
+    ks<<<blocks, 32 * kRows, 0, h->stream>>>(g, h->ig_host[0], h->ig, h->sg, h->st[stbuf], h->posf, h->cellid,
+                                             h->cell_start, L.list, L.count, h->offs, h->enum_inst, h->status, q);
+    const int tile = split ? 64 : 256;
+    auto kr = split ? k_rows<true, 64> : k_rows<false, 256>;
+    kr<<<((int)h->n + tile - 1) / tile, kRowThreads, 0, h->stream>>>((int)h->n, g.M, g.Ms, g.pcap, h->st[stbuf].id, L,
+                                                                      h->offs, h->bw_count, status, ticket, h->status);
+  }
   h->last_list = dst_list;
-  h->compact_ok[dst_list] = L.pown != nullptr;
 }

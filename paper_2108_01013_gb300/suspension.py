@@ -285,8 +285,8 @@ class Suspension:
 
     def autotune_kernels(self, trial_steps: int = 20):
         """Time the kernel shapes (pair-kernel blocks per SM 3 or 4; the
-        enumeration's candidate loop 1: plain, 4: screened with four loads
-        ahead), keep the fastest, restore the state.  Returns
+        enumeration's search 1: walked by owner, 4: staged by segments of
+        cells), keep the fastest, restore the state.  Returns
         ((blocks, loop), {(blocks, loop): ms/step})."""
         ms = np.zeros(4)
         ch = np.zeros(2, dtype=np.int32)

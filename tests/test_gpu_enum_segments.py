@@ -1,0 +1,122 @@
+"""The staged search over crowded cells (a block per segment of cells, rows
+scanned in a pass of their own) against the CPU oracle's brute force, where it
+can go wrong: boxes of 4 to 9 cells (every candidate exact below 7, the
+shifted row as wide as the box, segments ending at the box edge), cells of
+more owners than a warp holds and rows of more candidates than one tile,
+batched instances of different grids, rows that overflow, pair arrays that
+grow after the search."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    import oracle
+    import paper_2108_01013_gb300 as dss
+    from paper_2108_01013_gb300 import synth
+    oracle.build()
+    dss.build()
+    synth.build()
+    return dict(oracle=oracle, dss=dss, synth=synth)
+
+
+def _handle(env, g, cells, nstep=0, **kw):
+    """A handle whose grid has the given number of cells per axis."""
+    p = env["dss"].default_params(g["box"], cell_size=g["box"][0] / cells * (1.0 - 1e-12), **kw)
+    z = np.zeros_like(g["x"])
+    return env["dss"].Suspension(g["x"], g["a"], g["box"], p, ids=g["ids"], nstep=nstep, alpha_lin=z, alpha_ang=z)
+
+
+def _want(env, g, nstep, **kw):
+    po = env["oracle"].make_params(g["box"], **kw)
+    return env["oracle"].pairs_bruteforce(g["x"], g["a"], g["ids"], po, env["oracle"].le_offset(po, nstep))
+
+
+@pytest.mark.parametrize("n,cells", [(600, 4), (1200, 5), (2500, 6), (2600, 7), (4500, 9), (5000, 4), (9000, 5)])
+@pytest.mark.parametrize("nstep", [0, 777, 54321])
+def test_segment_pairs_bit_exact(env, n, cells, nstep):
+    g = env["synth"].small(n, 0.50, 900 + n)
+    kw = dict(shear_rate=1.3, dt=1e-3)
+    s = _handle(env, g, cells, nstep, **kw)
+    assert s.counters()["ncell"] == (cells,) * 3 and n >= 4 * cells ** 3
+    s.neighbour_build()
+    np.testing.assert_array_equal(s.pairs(), _want(env, g, nstep, **kw))
+    c = s.counters()
+    rows = np.bincount(_want(env, g, nstep, **kw).reshape(-1), minlength=n)
+    assert 0 < c["max_row"] <= rows.max()
+    s.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("forces", ["contact", "far"])
+def test_segment_forces_as_on_sparse_grid(env, precision, forces):
+    """The same forces on the grid that is walked owner by owner.  The rows
+    differ in their order alone: the sums of at most 60 pair terms differ by
+    less than 60 roundings of the particle's largest (FP64 2^-52, mixed 2^-23),
+    taken relative to the largest force of the packing."""
+    g = env["synth"].small(4000, 0.50, 77)
+    kw = dict(shear_rate=1.0, precision=precision)
+    if forces == "far":      # listed beyond the lubrication range: rows in two parts
+        kw.update(f_er=10.0, lambda_d=0.05, delta_lub=0.1)
+    out = []
+    for cells in (5, int(g["box"][0] / (2.8 + (1.0 if forces == "far" else 0.07) + 1e-6))):
+        s = _handle(env, g, cells, 31, **kw)
+        F, T = s.forces()
+        out.append((F.cpu().numpy(), T.cpu().numpy(), s.pairs()))
+        s.close()
+    np.testing.assert_array_equal(out[0][2], out[1][2])
+    tol = 60 * (2.0 ** -52 if precision == "fp64" else 2.0 ** -23)
+    for a, b in zip(out[0][:2], out[1][:2]):
+        assert np.abs(a - b).max() <= tol * np.abs(b).max()
+
+
+def test_segment_batch(env):
+    """Instances of 343 to 1728 cells' worth of different boxes in one launch."""
+    dss, orc = env["dss"], env["oracle"]
+    gs = [env["synth"].small(n, phi, 60 + n) for n, phi in [(3000, 0.5), (900, 0.42), (5200, 0.55), (2048, 0.48)]]
+    off = np.concatenate([[0], np.cumsum([g["a"].shape[0] for g in gs])])
+    rates = [0.5, 3.0, 1.0, 20.0]
+    p = dss.default_params(cell_size=gs[1]["box"][0] / 4.0 * (1.0 - 1e-12), dt=1e-3)
+    x = np.concatenate([g["x"] for g in gs], axis=1)
+    z = np.zeros_like(x)
+    b = dss.Batch(x, np.concatenate([g["a"] for g in gs]), np.diff(off), [g["box"] for g in gs], rates, p, nstep=333,
+                  alpha_lin=z, alpha_ang=z)
+    b.neighbour_build()
+    want = []
+    for k, g in enumerate(gs):
+        po = orc.make_params(g["box"], shear_rate=rates[k], dt=1e-3)
+        want.append(orc.pairs_bruteforce(g["x"], g["a"], g["ids"], po, orc.le_offset(po, 333)) + off[k])
+    np.testing.assert_array_equal(b.pairs(), np.concatenate(want))
+    b.close()
+
+
+@pytest.mark.parametrize("cells", [5, 0])
+def test_pair_arrays_that_grow_after_the_search(env, cells):
+    """A force evaluation whose pairs exceed the pair arrays lists them again:
+    the same bits as with room from the start."""
+    g = env["synth"].small(2000, 0.52, 5)
+    cells = cells or int(g["box"][0] / 2.871)
+    out = []
+    for cap in (1, 32):
+        s = _handle(env, g, cells, 3, pair_capacity=cap)
+        F, T = s.forces()
+        out.append((F.cpu().numpy(), T.cpu().numpy(), s.pairs(), s.counters()["band_checks"]))
+        s.step(3)
+        out[-1] += (s.state()["x"].cpu().numpy(),)
+        s.close()
+    for a, b in zip(*out):
+        np.testing.assert_array_equal(a, b)
+
+
+def test_segment_row_overflow_is_reported(env):
+    g = env["synth"].small(3000, 0.55, 9)
+    s = _handle(env, g, 5, 0, capacity_M=2)
+    with pytest.raises(env["dss"].DssError) as e:
+        s.neighbour_build()
+    assert e.value.code == -3
+    s.close()
