@@ -410,7 +410,7 @@ k_adj_tape_pairs(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restric
     t.pj[p] = j;
     double dx, dy, dz;
     int sy;
-    min_image(I, off, xi, yi, zi, s.x[j], s.x[n + j], s.x[2 * n + j], dx, dy, dz, sy);
+    min_image<false>(I, off, xi, yi, zi, s.x[j], s.x[n + j], s.x[2 * n + j], dx, dy, dz, sy);
     const double rr = exact_dist(dx, dy, dz);
     int pold = -1;
     double xo[3] = {0.0, 0.0, 0.0}, ro[3] = {0.0, 0.0, 0.0};
@@ -514,7 +514,7 @@ k_adj_pairs(Geo g, const InstGeo* __restrict__ ig, AdjTape t, const double* __re
     const int i = t.op[p], j = t.pj[p];
     PairIn in;
     int sy;
-    min_image(I, t.sg->off, t.x[i], t.x[n + i], t.x[2 * n + i], t.x[j], t.x[n + j], t.x[2 * n + j],
+    min_image<false>(I, t.sg->off, t.x[i], t.x[n + i], t.x[2 * n + i], t.x[j], t.x[n + j], t.x[2 * n + j],
               in.r[0], in.r[1], in.r[2], sy);
     in.sy = sy;
     in.yi = t.x[n + i];

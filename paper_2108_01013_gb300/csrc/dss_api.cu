@@ -732,6 +732,7 @@ int create_handle(dss_handle** out, const dss_params* p, int K, const int64_t* n
   g.hdt2 = g.hdt * p->dt;
   g.k6 = 6.0 * DSS_PI * p->eta0;
   g.k8 = 8.0 * DSS_PI * p->eta0;
+  g.mu_kt = p->mu / p->kt;
   g.f.kn = (float)p->kn;
   g.f.kt = (float)p->kt;
   g.f.mu_kt = (float)(p->mu / p->kt);

@@ -140,7 +140,7 @@ __device__ __forceinline__ F3 tangf(F3 n, F3 v) { return v - dotf(n, v) * n; }
 // records as they are stored.
 template <typename R>
 struct PairRes {
-  R F[3], Ti[3], Tj[3], Fc[3], Fl[3], r[3];
+  R F[3], Ti[3], Tj[3], Fl[3], r[3];
   Xi4 xrec, rrec;
   int contact;
 };
@@ -167,15 +167,15 @@ __device__ __forceinline__ PairRes<double> pair_eval_fp64(const Geo& g, const In
   const double sgn = idi < idj ? 1.0 : -1.0;
   double xo[3] = {0.0, 0.0, 0.0}, ro[3] = {0.0, 0.0, 0.0};
   const double rr = exact_dist(dx, dy, dz);
-  if (__dsub_rn(rr, __dadd_rn(ai, aj)) < 0.0) {
+  if (__double2hiint(__dsub_rn(rr, __dadd_rn(ai, aj))) < 0) {
     history_lookup<EXT>(g, H, hr, i, j, idi, idj, xo, ro);
     xo[0] *= sgn; xo[1] *= sgn; xo[2] *= sgn;
   }
-  const double Om = -0.5 * I.gdot;
+  const double hg = 0.5 * I.gdot;
   V3 Vi = v3(ui.x - I.gdot * yi, ui.y, ui.z);
   V3 Vj = v3(uj.x - I.gdot * yj, uj.y, uj.z);
-  V3 Wi = v3(wi.x, wi.y, wi.z - Om);
-  V3 Wj = v3(wj.x, wj.y, wj.z - Om);
+  V3 Wi = v3(wi.x, wi.y, wi.z + hg);
+  V3 Wj = v3(wj.x, wj.y, wj.z + hg);
   double rate = I.gdot;
   if (EXT && g.wave) {
     // the wave of Eq. 17 at each centre: V and W relative to the local flow,
@@ -187,15 +187,14 @@ __device__ __forceinline__ PairRes<double> pair_eval_fp64(const Geo& g, const In
     Wj.z += 0.5 * qj.y;
     rate = I.gdot + 0.5 * (qi.y + qj.y);
   }
-  const V3 du = v3(uj.x + sy * I.gdot * I.L[1] - ui.x, uj.y - ui.y, uj.z - ui.z);
-  const PairParams<double> pp{g.kn, g.kt, I.gn, g.mu, g.delta};
-  const PairModelOut<double> o = pair_model<double, EXT>(g, I, pp, r, rr, ai, aj, Vi, Vj, Wi, Wj, du, wi, wj,
-                                                    v3(xo[0], xo[1], xo[2]), v3(ro[0], ro[1], ro[2]), rate);
+  V3 du = v3(uj.x - ui.x, uj.y - ui.y, uj.z - ui.z);
+  if (sy != 0) du.x += sy > 0 ? I.gdot * I.L[1] : -(I.gdot * I.L[1]);
+  const PairModelOut o = pair_model<EXT>(g, I.gn, r, rr, ai, aj, Vi, Vj, Wi, Wj, du, wi, wj,
+                                         v3(xo[0], xo[1], xo[2]), v3(ro[0], ro[1], ro[2]), rate);
   PairRes<double> q;
   q.F[0] = o.F.x; q.F[1] = o.F.y; q.F[2] = o.F.z;
   q.Ti[0] = o.Ti.x; q.Ti[1] = o.Ti.y; q.Ti[2] = o.Ti.z;
   q.Tj[0] = o.Tj.x; q.Tj[1] = o.Tj.y; q.Tj[2] = o.Tj.z;
-  q.Fc[0] = o.Fc.x; q.Fc[1] = o.Fc.y; q.Fc[2] = o.Fc.z;
   q.Fl[0] = o.Fl.x; q.Fl[1] = o.Fl.y; q.Fl[2] = o.Fl.z;
   q.r[0] = dx; q.r[1] = dy; q.r[2] = dz;
   q.xrec = Xi4{sgn * o.xi.x, sgn * o.xi.y, sgn * o.xi.z, o.contact ? 1.0 : 0.0};
@@ -232,24 +231,34 @@ __device__ __forceinline__ PairRes<float> pair_eval_mixed(const Geo& g, const In
   int wy = ((cj >> 10) & 1023) - ((ci >> 10) & 1023);
   const int le = wy < -R ? 1 : (wy > R ? -1 : 0);
   wy += le * ny;
-  int wx = (cj & 1023) - (ci & 1023) + le * sg.fsh;
-  wx %= nx;
-  if (wx < 0) wx += nx;
-  // the image row spans x offsets -R-1..R (above) or -R..R+1 (below)
-  if (le == -1 ? 2 * wx > nx : 2 * wx >= nx) wx -= nx;
+  int wx = (cj & 1023) - (ci & 1023);
+  if (le != 0) {
+    wx = (wx + le * sg.fsh) % nx;
+    if (wx < 0) wx += nx;
+    // the image row spans x offsets -R-1..R (above) or -R..R+1 (below)
+    if (le == -1 ? 2 * wx > nx : 2 * wx >= nx) wx -= nx;
+  } else if (wx > R) {
+    wx -= nx;
+  } else if (wx < -R) {
+    wx += nx;
+  }
   int wz = (cj >> 20) - (ci >> 20);
   if (wz > R) wz -= nz; else if (wz < -R) wz += nz;
-  FF cx = cell_shift(wx, I.csf[0], I.cs_lo[0]);
+  // the low words' difference (below 2^-23 cell) goes into the shift's low
+  // word; the sums need an error relative to the cell and to S^2, not to
+  // their own (cancelled) value
+  FF cx = cell_shift(wx, I.csf[0], I.cs_lo[0]), cy = cell_shift(wy, I.csf[1], I.cs_lo[1]),
+     cz = cell_shift(wz, I.csf[2], I.cs_lo[2]);
   if (le == 1) cx = ff_add(cx, FF{sg.offr_hi, sg.offr_lo});
   else if (le == -1) cx = ff_add(cx, FF{-sg.offr_hi, -sg.offr_lo});
-  const FF dxf = ff_add(two_sum(pj.x, -pi.x), ff_add(cx, FF{lj.x - li.x, 0.f}));
-  const FF dyf = ff_add(two_sum(pj.y, -pi.y),
-                        ff_add(cell_shift(wy, I.csf[1], I.cs_lo[1]), FF{lj.y - li.y, 0.f}));
-  const FF dzf = ff_add(two_sum(pj.z, -pi.z),
-                        ff_add(cell_shift(wz, I.csf[2], I.cs_lo[2]), FF{lj.z - li.z, 0.f}));
-  const FF Sff = ff_add(FF{pi.w, li.w}, FF{pj.w, lj.w});
-  const FF r2ff = ff_add(ff_add(ff_sqr(dxf), ff_sqr(dyf)), ff_sqr(dzf));
-  const FF numff = ff_add(r2ff, ff_neg(ff_sqr(Sff)));          // r^2 - S^2, ~44 bits
+  cx.lo += lj.x - li.x;
+  cy.lo += lj.y - li.y;
+  cz.lo += lj.z - li.z;
+  const FF dxf = ff_add_abs(two_sum(pj.x, -pi.x), cx), dyf = ff_add_abs(two_sum(pj.y, -pi.y), cy),
+           dzf = ff_add_abs(two_sum(pj.z, -pi.z), cz);
+  const FF Sff = ff_add_abs(FF{pi.w, li.w}, FF{pj.w, lj.w});
+  const FF r2ff = ff_add_abs(ff_add_abs(ff_sqr(dxf), ff_sqr(dyf)), ff_sqr(dzf));
+  const FF numff = ff_add_abs(r2ff, ff_neg(ff_sqr(Sff)));      // r^2 - S^2 to ~2^-45 S^2
   const float num = numff.hi + numff.lo;
   const float r2 = r2ff.hi + r2ff.lo;
   const float ir = rsqrtf(r2);
@@ -391,38 +400,29 @@ __device__ __forceinline__ PairRes<float> pair_eval_mixed(const Geo& g, const In
   // pairs are all beyond it skips the block)
   F3 Fl = f3(0.0f, 0.0f, 0.0f), Tli = Fl, Tlj = Fl;
   if (lub_on) {
-    const float iS = __fdividef(1.0f, S), iS2 = iS * iS, iS3 = iS2 * iS;
+    const float iS = __fdividef(1.0f, S);
     float ds = 2.0f * d * iS;
     ds = ds > 0.0f ? ds : 0.0f;
     const float dd = ds + g.f.eps;
     const float X = __fdividef(1.0f, dd);
     const float Y = -__logf(dd);
-    const float A = Ai, B = Bj, AB = A * B;
-    const float xa = X * 2.0f * AB * AB * iS3;
-    const float ya = Y * (4.0f / 15.0f) * AB * (2.0f * A * A + AB + 2.0f * B * B) * iS3;
-    const float ybi = -Y * (2.0f / 15.0f) * A * AB * (4.0f * A + B) * iS2;
-    const float ybj = -Y * (2.0f / 15.0f) * AB * B * (A + 4.0f * B) * iS2;
-    const float yci = Y * (8.0f / 15.0f) * A * A * AB * iS;
-    const float ycj = Y * (8.0f / 15.0f) * AB * B * B * iS;
-    const float ycx = Y * (2.0f / 15.0f) * AB * AB * iS;
-    const float xg = X * 2.0f * AB * AB * iS2;
-    const float yg = Y * (1.0f / 15.0f) * AB * (4.0f - 6.0f * AB * iS2);
-    const float yhi = Y * iS2 * ((2.0f / 15.0f) * A * A * AB * (2.0f * A - B) + (1.0f / 15.0f) * AB * AB * (7.0f * A + B));
-    const float yhj = Y * iS2 * ((1.0f / 15.0f) * AB * AB * (A + 7.0f * B) + (2.0f / 15.0f) * AB * B * B * (2.0f * B - A));
-    const F3 dV = Vi - Vj;
-    const float nV = dotf(nn, dV);
-    const F3 fr = (xa * nV) * nn + ya * tangf(nn, dV) + ybi * crossf(nn, Wi) + ybj * crossf(nn, Wj);
+    // the closed form of dss_pair_model.cuh
+    const float A = Ai, B = Bj, AB = A * B, h = AB * iS, hb = h * iS;
+    const float xa = ((2.0f * k6) * X) * (h * hb);
+    const float y2 = ((2.0f / 15.0f) * k6) * Y, yb = y2 * hb, yh = y2 * h;
+    const float ya = (2.0f * yb) * (2.0f * S - 3.0f * h);
+    const float ybi = -(yb * A) * (3.0f * A + S), ybj = -(yb * B) * (3.0f * B + S);
+    const float yci = (4.0f * yh) * (A * A), ycj = (4.0f * yh) * (B * B), ycx = yh * AB;
     // strain of the shear rate acting on the pair (the wave of Eq. 17: the
     // mean of the two centres' local rates)
     const float rate = (EXT && g.wave) ? gd + 0.5f * (vi4.w + vj4.w) : gd;
-    const F3 twoEn = f3(rate * nn.y, rate * nn.x, 0.0f);
-    const float Pn = rate * nn.x * nn.y;
-    const F3 Qn = twoEn - (2.0f * Pn) * nn;
-    const F3 nperp = crossf(nn, twoEn);
-    Fl = k6 * (((xg * Pn) * nn + yg * Qn) - fr);
-    const F3 ndV = crossf(nn, dV);
-    Tli = k6 * (ybi * ndV - (yci * tangf(nn, Wi) + ycx * tangf(nn, Wj)) + yhi * nperp);
-    Tlj = k6 * (ybj * ndV - (ycx * tangf(nn, Wi) + ycj * tangf(nn, Wj)) + yhj * nperp);
+    const float e = 0.5f * S * rate;
+    const F3 G = f3((Vi.x - Vj.x) - e * nn.y, (Vi.y - Vj.y) - e * nn.x, Vi.z - Vj.z);
+    const float nG = dotf(nn, G), fn = (ya - xa) * nG;
+    const F3 nW = crossf(nn, ybi * Wi + ybj * Wj), nxG = crossf(nn, G);
+    Fl = f3(fn * nn.x - ya * G.x - nW.x, fn * nn.y - ya * G.y - nW.y, fn * nn.z - ya * G.z - nW.z);
+    Tli = ybi * nxG - tangf(nn, yci * Wi + ycx * Wj);
+    Tlj = ybj * nxG - tangf(nn, ycx * Wi + ycj * Wj);
     if (g.f.taper > 0.0f) {
       // differentiable cutoff: smoothstep over the last fraction w of the range
       const float dl = g.mode == 1 ? g.f.delta_a0 : g.f.delta * 0.5f * S;
@@ -446,7 +446,6 @@ __device__ __forceinline__ PairRes<float> pair_eval_mixed(const Geo& g, const In
   q.F[0] = F.x; q.F[1] = F.y; q.F[2] = F.z;
   q.Ti[0] = Ti.x; q.Ti[1] = Ti.y; q.Ti[2] = Ti.z;
   q.Tj[0] = Tj.x; q.Tj[1] = Tj.y; q.Tj[2] = Tj.z;
-  q.Fc[0] = Fc.x; q.Fc[1] = Fc.y; q.Fc[2] = Fc.z;
   q.Fl[0] = Fl.x; q.Fl[1] = Fl.y; q.Fl[2] = Fl.z;
   q.r[0] = r.x; q.r[1] = r.y; q.r[2] = r.z;
   return q;
@@ -492,11 +491,12 @@ __device__ __forceinline__ void store_record(double* b, double a0, double a1, do
 // Per pair after its evaluation: the partner's share (-F and its torque)
 // written to slot `slot` of the partner's row (taken by the caller with an
 // atomic on the row's count) with the owner's index, the stretch records,
-// the contact count and the stresslet of Eq. 9 (S^C = r (x) F^C,
-// S^L = sym(r (x) F^L), F on the owner) added to the thread's sum.
+// the contact count and the stresslet of Eq. 9, S = r (x) F^C + sym(r (x) F^L)
+// = r (x) F - (1/2)(r (x) F^L - F^L (x) r), F on the owner: r (x) F and the
+// three components of r x F^L added to the thread's sums (12 values).
 template <typename R, bool EXT>
 __device__ __forceinline__ void pair_commit(const Geo& g, const PairRes<R>& q, int i, int j, int p, ListBuf& W,
-                                            int slot, R* __restrict__ bw, DevStatus* st, R Sx[9],
+                                            int slot, R* __restrict__ bw, DevStatus* st, R Sx[12],
                                             int& ncont) {
   if (slot < g.M) {
     R* b = bw + ((int64_t)j * g.M + slot) * kSlot;
@@ -510,8 +510,18 @@ __device__ __forceinline__ void pair_commit(const Geo& g, const PairRes<R>& q, i
 #pragma unroll
   for (int a = 0; a < 3; ++a)
 #pragma unroll
-    for (int b2 = 0; b2 < 3; ++b2)
-      Sx[3 * a + b2] += q.r[a] * q.Fc[b2] + R(0.5) * (q.r[a] * q.Fl[b2] + q.r[b2] * q.Fl[a]);
+    for (int b2 = 0; b2 < 3; ++b2) Sx[3 * a + b2] += q.r[a] * q.F[b2];
+  Sx[9] += q.r[1] * q.Fl[2] - q.r[2] * q.Fl[1];
+  Sx[10] += q.r[2] * q.Fl[0] - q.r[0] * q.Fl[2];
+  Sx[11] += q.r[0] * q.Fl[1] - q.r[1] * q.Fl[0];
+}
+// The nine stresslet components from the twelve sums.
+template <typename R>
+__device__ __forceinline__ void stresslet(R S[12]) {
+  const R x = R(0.5) * S[9], y = R(0.5) * S[10], z = R(0.5) * S[11];
+  S[1] -= z; S[3] += z;
+  S[2] += y; S[6] -= y;
+  S[5] -= x; S[7] += x;
 }
 
 // Number of values per warp-boundary slot of the pair-balanced kernel: force
@@ -527,6 +537,7 @@ __device__ __forceinline__ void owner_scan(int lane, int seg, R v[NV]) {
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
     const int so = __shfl_up_sync(0xffffffffu, seg, d);
+    if (!__any_sync(0xffffffffu, lane >= d && so == seg)) break;   // no longer runs in this warp
 #pragma unroll
     for (int c = 0; c < NV; ++c) {
       const R u = __shfl_up_sync(0xffffffffu, v[c], d);
@@ -635,12 +646,17 @@ k_pairs_pb(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sg
     }
     return;
   }
-  R Sx[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+  R Sx[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
   int ncont = 0;
   const int lane = threadIdx.x & 31;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
   const int npw = (P + 31) >> 5;
+  // Consecutive warps of pairs go to one block (they share particles in L1);
+  // in FP64, when there are fewer than warps, they are spread over the blocks:
+  // 2,300 pairs on ten SMs ran eight warps on each SM's two FP64 lanes (47 us,
+  // spread 27)
+  const int gw = MIXED || npw > nw ? (blockIdx.x * blockDim.x + threadIdx.x) >> 5
+                                   : (int)((threadIdx.x >> 5) * gridDim.x + blockIdx.x);
   for (int pw = gw; pw < npw; pw += nw) {
     const int p = pw * 32 + lane;
     const bool valid = p < P;
@@ -666,8 +682,9 @@ k_pairs_pb(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sg
       v[0] = q.F[0]; v[1] = q.F[1]; v[2] = q.F[2];
       v[3] = q.Ti[0]; v[4] = q.Ti[1]; v[5] = q.Ti[2];
       if constexpr (PERS) {
-        R Sp[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+        R Sp[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
         pair_commit<R, EXT>(g, q, i, j, p, W, slot, bw, st, Sp, ncont);
+        stresslet(Sp);
 #pragma unroll
         for (int c = 0; c < 9; ++c) v[6 + c] = Sp[c];
       } else {
@@ -708,6 +725,7 @@ k_pairs_pb(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sg
         ew0 += (10.0 / 3.0) * DSS_PI * g.eta0 * a * a * a * s.wv[il].y;
       }
     }
+    stresslet(Sx);
     stress_partials<MIXED, EXT>(Sx, ew0, ncont, spart, st);
   }
 }
@@ -974,6 +992,14 @@ __device__ __forceinline__ void warp_sum_row(const R* __restrict__ row, int cc, 
   }
 }
 
+// a / b from r = 1/b rounded: the quotient estimate a r corrected by its exact
+// remainder (Markstein): the rounded quotient, three operations instead of a
+// division's ten on GB300's narrow FP64 pipe.
+__device__ __forceinline__ double div_by(double a, double b, double r) {
+  const double q = a * r;
+  return fma(fma(-q, b, a), r, q);
+}
+
 // Total force and torque on particle j (its own pair sum, its partner
 // records, Stokes drag), then the accelerations and, in a step, the velocity
 // half-kick of Eq. 15d.  Returns true when the sums are not finite (the
@@ -1140,13 +1166,15 @@ __device__ __forceinline__ bool gather_one(const Geo& g, const InstGeo* __restri
       aw[c] = T[c] * iIr;
     }
   } else {
-    // FP64: F/m and T/I as IEEE divisions, m and I formed left to right
+    // FP64: F/m and T/I, m and I formed left to right; one IEEE reciprocal
+    // each, the quotients corrected by their remainders (div_by)
     const double m = __dmul_rn(__dmul_rn(__dmul_rn(__dmul_rn(4.0 / 3.0 * DSS_PI, g.rho), a), a), a);
     const double I = __dmul_rn(__dmul_rn(__dmul_rn(0.4, m), a), a);
+    const double im = __drcp_rn(m), iI = __drcp_rn(I);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      al[c] = __ddiv_rn(F[c], m);
-      aw[c] = __ddiv_rn(T[c], I);
+      al[c] = div_by(F[c], m, im);
+      aw[c] = div_by(T[c], I, iI);
     }
   }
 #pragma unroll

@@ -62,6 +62,7 @@ struct Geo {
   double hdt, hdt2;   // dt/2 and (dt/2) dt, each rounded once
   double k6;          // 6 pi eta0
   double k8;          // 8 pi eta0
+  double mu_kt;       // mu / k_t
   double taper;       // lubrication taper width w (0: hard cutoff)
   double f_er, lambda_d, hamaker, vdw_eps;   // electro-chemical forces (Eq. 6-7)
   double de;          // their range as a surface distance (0: off)
@@ -135,10 +136,22 @@ __device__ __forceinline__ double pair_delta(const Geo& g, double ai, double aj)
   return g.de > dl ? g.de : dl;
 }
 
+// |v| > L for L > 0 and any v but NaN (which passes), on the bit patterns.
+__device__ __forceinline__ bool abs_gt(double v, double L) {
+  return (__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFll) > __double_as_longlong(L);
+}
+// The nearest image of a separation beyond half the box (out of line: a branch
+// turned into predicated instructions would still issue to the FP64 pipe).
+static __device__ __noinline__ double image_slow(double v, double L, double invL) {
+  return __dsub_rn(v, __dmul_rn(L, rint(__dmul_rn(v, invL))));
+}
+
 // Minimum-image separation r = x_j - x_i under Lees-Edwards conditions,
 // spelled out operation by operation (no contraction) so that the neighbour
 // decision is the same bit pattern on every path.  sy: image shift in y
-// (-1: image one box below, +1: above).
+// (-1: image one box below, +1: above).  CALL: the rare image counts called
+// out of line (not from kernels that hold their state across the call).
+template <bool CALL = true>
 __device__ __forceinline__ void min_image(const InstGeo& g, double off, double xi, double yi,
                                           double zi, double xj, double yj, double zj,
                                           double& dx, double& dy, double& dz, int& sy) {
@@ -146,20 +159,30 @@ __device__ __forceinline__ void min_image(const InstGeo& g, double off, double x
   dy = __dsub_rn(yj, yi);
   dz = __dsub_rn(zj, zi);
   sy = 0;
-  if (dy > g.halfL[1]) {
-    dy = __dsub_rn(dy, g.L[1]);
-    dx = __dsub_rn(dx, off);
-    sy = -1;
-  } else if (dy < -g.halfL[1]) {
-    dy = __dadd_rn(dy, g.L[1]);
-    dx = __dadd_rn(dx, off);
-    sy = 1;
+  // nearly every pair lies within half the box along each axis: nothing to
+  // shift.  The tests compare bit patterns (FP64 compares go through GB300's
+  // narrow FP64 pipe).
+  if (abs_gt(dy, g.halfL[1])) {
+    if (__double2hiint(dy) >= 0) {
+      dy = __dsub_rn(dy, g.L[1]);
+      dx = __dsub_rn(dx, off);
+      sy = -1;
+    } else {
+      dy = __dadd_rn(dy, g.L[1]);
+      dx = __dadd_rn(dx, off);
+      sy = 1;
+    }
   }
   // image count rint(dx / L) taken as rint(dx * (1/L)): the two differ only
   // when dx is within rounding of +-L/2, where both images lie at least
   // L/2 >= 1.5 cells away, beyond any pair's cutoff, so no decision changes
-  dx = __dsub_rn(dx, __dmul_rn(g.L[0], rint(__dmul_rn(dx, g.invL[0]))));
-  dz = __dsub_rn(dz, __dmul_rn(g.L[2], rint(__dmul_rn(dz, g.invL[2]))));
+  if constexpr (CALL) {
+    if (abs_gt(dx, g.halfL[0])) dx = image_slow(dx, g.L[0], g.invL[0]);
+    if (abs_gt(dz, g.halfL[2])) dz = image_slow(dz, g.L[2], g.invL[2]);
+  } else {
+    dx = __dsub_rn(dx, __dmul_rn(g.L[0], rint(__dmul_rn(dx, g.invL[0]))));
+    dz = __dsub_rn(dz, __dmul_rn(g.L[2], rint(__dmul_rn(dz, g.invL[2]))));
+  }
 }
 
 // Centre distance |r| with the operations of the plain FP64 evaluation
@@ -430,6 +453,12 @@ __device__ __forceinline__ FF ff_add_f(FF a, float b) {
 __device__ __forceinline__ FF ff_mul_f(FF a, float b) {
   const float p = a.hi * b;
   return fast_two_sum(p, fmaf(a.hi, b, -p) + a.lo * b);
+}
+// a + b with an error of about 2^-47 (|a| + |b|): where a sum of magnitudes
+// bounds what is needed, not the (cancelled) result
+__device__ __forceinline__ FF ff_add_abs(FF a, FF b) {
+  const FF s = two_sum(a.hi, b.hi);
+  return fast_two_sum(s.hi, s.lo + (a.lo + b.lo));
 }
 // w whole cells of edge (cs_hi + cs_lo) as a double-float: the product of
 // the FP32 words is made exact with Dekker's TwoProduct (w cs_hi needs more
