@@ -651,13 +651,16 @@ k_pairs_pb(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sg
   const int lane = threadIdx.x & 31;
   const int nw = (gridDim.x * blockDim.x) >> 5;
   const int npw = (P + 31) >> 5;
-  // Consecutive warps of pairs go to one block (they share particles in L1);
-  // in FP64, when there are fewer than warps, they are spread over the blocks:
-  // 2,300 pairs on ten SMs ran eight warps on each SM's two FP64 lanes (47 us,
-  // spread 27)
-  const int gw = MIXED || npw > nw ? (blockIdx.x * blockDim.x + threadIdx.x) >> 5
-                                   : (int)((threadIdx.x >> 5) * gridDim.x + blockIdx.x);
-  for (int pw = gw; pw < npw; pw += nw) {
+  // Rounds of one warp of pairs per warp of the grid, consecutive ones to one
+  // block (they share particles in L1).  FP64 spreads the last, partial round
+  // over the blocks: an SM's time goes with its warps there, and eight more on
+  // some of the SMs than on the others cost 20 of 263 us a step at 267k pairs,
+  // 18 of 153 at 115k, and 20 of 85 at 2,300, which ran on ten SMs.  (In mixed
+  // precision, bound by latency, it gave nothing.)
+  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int spread = (int)((threadIdx.x >> 5) * gridDim.x + blockIdx.x);
+  for (int pw = !MIXED && npw < nw ? spread : gw, next = nw; pw < npw;
+       pw = MIXED ? pw + nw : next + (npw - next < nw ? spread : gw), next += nw) {
     const int p = pw * 32 + lane;
     const bool valid = p < P;
     const int i = valid ? W.pown[p] : -1;
