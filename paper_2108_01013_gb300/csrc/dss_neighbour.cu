@@ -178,6 +178,7 @@ k_enumerate(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ s
             const float4* __restrict__ posf, const int* __restrict__ cellid,
             const int* __restrict__ cell_start, ListBuf L, int* __restrict__ bw_count,
             unsigned long long* scan_status, int* scan_ticket, DevStatus* st, EnumCut q) {
+  dep_wait();
   if (dev_err(st)) return;
   __shared__ int s_tile;
   if (threadIdx.x == 0) s_tile = atomicAdd(scan_ticket, 1);
@@ -251,6 +252,7 @@ k_enumerate_classes(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __rest
                     const float4* __restrict__ posf, const int* __restrict__ cellid,
                     const int* __restrict__ cell_start, ListBuf L, int* __restrict__ bw_count,
                     unsigned long long* scan_status, int* scan_ticket, DevStatus* st, EnumCut q) {
+  dep_wait();
   if (dev_err(st)) return;
   __shared__ int s_tile;
   if (threadIdx.x == 0) s_tile = atomicAdd(scan_ticket, 1);
@@ -383,6 +385,7 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
             const int* __restrict__ cellid, const int* __restrict__ cell_start, int* __restrict__ list,
             int* __restrict__ count, int* __restrict__ nnear, const int* __restrict__ blk_inst, DevStatus* st,
             EnumCut q) {
+  dep_wait();
   __shared__ float4 s_c[kRows][kTile + 4];
   __shared__ int s_j[kRows][kTile];
   __shared__ int s_off[kRows][32];
@@ -614,6 +617,7 @@ __global__ void __launch_bounds__(kRowThreads)
 k_rows(int n, int M, int Ms, int64_t pcap, const int* __restrict__ ids, const __grid_constant__ ListBuf L,
        const int* __restrict__ nnear, int* __restrict__ bw_count, unsigned long long* scan_status, int* scan_ticket,
        DevStatus* st) {
+  dep_wait();
   constexpr int kAhead = 4;                  // pairs a thread reads before the offsets are known
   __shared__ int s_tile, s_prefix;
   __shared__ int s_warp[kRowThreads / 32];
@@ -812,7 +816,7 @@ void launch_enumerate(dss_handle* h, int stbuf, int dst_list, int adv) {
   if (h->enum_walk) {
     auto kw = g.nclass > 1 ? (ech ? k_enumerate_classes<true> : k_enumerate_classes<false>)
                            : (ech ? k_enumerate<true> : k_enumerate<false>);
-    kw<<<blocks, kThreads, 0, h->stream>>>(g, h->ig, h->sg, h->st[stbuf], h->posf, h->cellid, h->cell_start, L,
+    launch_dep(kw, blocks, kThreads, h->stream, g, h->ig, h->sg, h->st[stbuf], h->posf, h->cellid, h->cell_start, L,
                                            h->bw_count, status, ticket, h->status, q);
   } else {
     const bool one = h->K == 1;
@@ -820,11 +824,11 @@ void launch_enumerate(dss_handle* h, int stbuf, int dst_list, int adv) {
                            : (one ? k_enumerate_seg<true, false, true> : k_enumerate_seg<true, false, false>))
                   : (split ? (one ? k_enumerate_seg<false, true, true> : k_enumerate_seg<false, true, false>)
                            : (one ? k_enumerate_seg<false, false, true> : k_enumerate_seg<false, false, false>));
-    ks<<<blocks, 32 * kRows, 0, h->stream>>>(g, h->ig_host[0], h->ig, h->sg, h->st[stbuf], h->posf, h->cellid,
+    launch_dep(ks, blocks, 32 * kRows, h->stream, g, h->ig_host[0], h->ig, h->sg, h->st[stbuf], h->posf, h->cellid,
                                              h->cell_start, L.list, L.count, h->offs, h->enum_inst, h->status, q);
     const int tile = split ? 64 : 256;
     auto kr = split ? k_rows<true, 64> : k_rows<false, 256>;
-    kr<<<((int)h->n + tile - 1) / tile, kRowThreads, 0, h->stream>>>((int)h->n, g.M, g.Ms, g.pcap, h->st[stbuf].id, L,
+    launch_dep(kr, ((int)h->n + tile - 1) / tile, kRowThreads, h->stream, (int)h->n, g.M, g.Ms, g.pcap, h->st[stbuf].id, L,
                                                                       h->offs, h->bw_count, status, ticket, h->status);
   }
   h->last_list = dst_list;
