@@ -48,7 +48,7 @@ void free_buffers(dss_handle* h) {
   h->pred = nullptr;
   dfree(h->xc); dfree(h->mark);
   h->xc = nullptr; h->mark = nullptr; h->marked = false;
-  dfree(h->cell_count); dfree(h->cell_start); dfree(h->tmp); dfree(h->spart);
+  dfree(h->cell_count); dfree(h->cell_ids); h->cell_ids = nullptr; dfree(h->cell_start); dfree(h->tmp); dfree(h->spart);
   dfree(h->own); dfree(h->bw_count); dfree(h->bw_rec); dfree(h->carry); dfree(h->own_s);
   h->own = nullptr; h->bw_count = nullptr; h->bw_rec = nullptr; h->carry = nullptr; h->own_s = nullptr;
   h->pb_blocks = 0;
@@ -208,6 +208,13 @@ int alloc_buffers(dss_handle* h) {
       (r = dalloc(h, &h->scan_ticket, 2)))
     return r;
   CK(cudaMemsetAsync(h->cell_count, 0, sizeof(int) * h->g.ncell, h->stream));
+  {
+    // rows of ids: four times the average cell and twelve more (random
+    // packings stay within), shorter on grids of mostly empty cells
+    const double per = (double)n / (double)h->g.ncell;
+    h->cell_cap = per < 0.1 ? 4 : (per < 0.5 ? 8 : ((int)std::min(4.0 * per, 1e6) + 12 + 3) & ~3);
+    if ((r = dalloc(h, &h->cell_ids, (size_t)h->g.ncell * h->cell_cap))) return r;
+  }
   h->pcap = 0;
   int per = h->p.pair_capacity > 0 ? h->p.pair_capacity : 16;
   if ((r = alloc_pair_buffers(h, std::max<int64_t>((int64_t)n * per, 1024), false))) return r;
@@ -215,8 +222,30 @@ int alloc_buffers(dss_handle* h) {
   return DSS_OK;
 }
 
+// Longer rows of ids after an operation that met a fuller cell.
+int grow_cells(dss_handle* h) {
+  CK(cudaStreamSynchronize(h->stream));
+  const int cap = (h->status_host->w[ST_CELL] + h->status_host->w[ST_CELL] / 2 + 3) & ~3;
+  int* ids = nullptr;
+  int r = dalloc(h, &ids, (size_t)h->g.ncell * cap);
+  if (r) {
+    cudaGetLastError();
+    return DSS_OK;   // the short rows still serve
+  }
+  dfree(h->cell_ids);
+  h->bytes -= (int64_t)(sizeof(int) * (size_t)h->g.ncell * h->cell_cap);
+  h->cell_ids = ids;
+  h->cell_cap = cap;
+  drop_graphs(h);
+  return DSS_OK;
+}
+
 // Orders the library's stream after everything queued on the caller's stream.
 int enter(dss_handle* h) {
+  if (h->sized && h->status_host->w[ST_CELL] > h->cell_cap) {
+    const int r = grow_cells(h);
+    if (r) return r;
+  }
   if (!h->own_stream) return DSS_OK;
   CK(cudaEventRecord(h->ev_enter, h->user_stream));
   CK(cudaStreamWaitEvent(h->stream, h->ev_enter, 0));
@@ -318,6 +347,7 @@ __global__ void k_set_nstep(DevStatus* st, long long nstep) {
   st->w[ST_NSTEP_HI] = (int)(nstep >> 32);
   st->w[ST_STEPS] = 0;
   st->w[ST_ERR] = 0;
+  st->w[ST_CELL] = 0;
 }
 
 __global__ void k_iota(int n, int* __restrict__ v) {
@@ -720,6 +750,7 @@ int create_handle(dss_handle** out, const dss_params* p, int K, const int64_t* n
     return DSS_ERR_CUDA;
   }
   cudaMemsetAsync(h->status, 0, sizeof(DevStatus), h->stream);
+  memset(h->status_host, 0, sizeof(DevStatus));
   Geo& g = h->g;
   g.n = (int)total;
   g.K = K;

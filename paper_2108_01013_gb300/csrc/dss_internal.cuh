@@ -25,6 +25,7 @@ enum {
   ST_NSTEP_LO = 6,   // time step counter (64 bit, lo/hi)
   ST_NSTEP_HI = 7,
   ST_BADPOS = 8,     // set_state: positions outside the box
+  ST_CELL = 10,      // a cell of more particles than its row of ids holds (0: none so far)
   ST_IDORDER = 9,    // 1 after dss_load_state: the committed state is not in the history's row order
   ST_WORDS = 16
 };
@@ -665,6 +666,8 @@ struct dss_handle {
   int* key;          // n
   int* offs;         // n
   int* cell_count;   // ncell
+  int* cell_ids;     // ncell rows of cell_cap ids (a multiple of four)
+  int cell_cap;
   int* cell_start;   // ncell+1
   int* tmp;          // n
   // lists: hist = committed (history source), work = being built
