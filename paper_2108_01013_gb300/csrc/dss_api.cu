@@ -265,6 +265,8 @@ int sync_status(dss_handle* h) {
 }
 
 int clear_err(dss_handle* h) {
+  // (a step that failed in its corrector may have begun the next histogram)
+  if (h->sized) CK(cudaMemsetAsync(h->cell_count, 0, sizeof(int) * h->g.ncell, h->stream));
   CK(cudaMemsetAsync(&h->status->w[ST_ERR], 0, sizeof(int), h->stream));
   return DSS_OK;
 }
@@ -444,16 +446,28 @@ __global__ void k_history_out(Geo g, ListBuf L, long long* __restrict__ keys,
 
 // The operation sequences.  stbuf/list indices follow the handle's
 // committed (cur, hist) pair; "w" is the scratch side.
-void seq_sort_enum(dss_handle* h, bool predict, int adv) {
+void seq_sort_enum(dss_handle* h, bool predict, int adv, bool keyed = false) {
   const int w = 1 - h->cur;
-  launch_sort(h, predict, h->cur, w);
+  launch_sort(h, predict, h->cur, w, keyed);
   launch_enumerate(h, w, 1 - h->hist, adv);
 }
 
-void seq_step(dss_handle* h) {
+// Whether the steps of a run hand the next one's first part to their corrector:
+// up to 1600 particles per SM, where the kernels wait on latency.  Beyond, the
+// corrector is bound by memory and the predictor by the FP64 pipe, and each
+// does better in its own kernel (1M 466 us a step apart, 470 together); so do
+// the long partner rows of electro-chemical ranges over crowded cells (Table 5
+// 521, 526).
+bool chain_steps(const dss_handle* h) {
+  return h->n <= 1600 * (int64_t)h->sms && !(h->g.de > 0.0 && h->n >= 8 * (int64_t)h->g.ncell);
+}
+
+// A step; keyed: the step before it ran its first part, next: this one runs
+// that of the step after it.
+void seq_step(dss_handle* h, bool keyed = false, bool next = false) {
   const int w = 1 - h->cur;
-  seq_sort_enum(h, true, 1);
-  launch_forces(h, w, 1 - h->hist, h->hist, 1, G_STEP, nullptr, nullptr);
+  seq_sort_enum(h, true, 1, keyed);
+  launch_forces(h, w, 1 - h->hist, h->hist, 1, G_STEP, nullptr, nullptr, next);
 }
 
 int capture_step(dss_handle* h, int key) {
@@ -479,10 +493,11 @@ int capture_multi(dss_handle* h, int key) {
   h->cur = key >> 1;
   h->hist = key & 1;
   cudaGraph_t graph;
+  const bool chain = chain_steps(h);
   CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
   h->capturing = true;
   for (int k = 0; k < DSS_MULTI_STEPS; ++k) {
-    seq_step(h);
+    seq_step(h, chain && k > 0, chain && k + 1 < DSS_MULTI_STEPS);
     h->cur = 1 - h->cur;
     h->hist = 1 - h->hist;
   }

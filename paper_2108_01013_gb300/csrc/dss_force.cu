@@ -24,8 +24,8 @@
 //   finish adds them to the running sums and commits the step.
 #include <climits>
 
-#include "dss_internal.cuh"
 #include "dss_pair_model.cuh"
+#include "dss_predict.cuh"
 
 namespace {
 constexpr int kPairThreads = 256;
@@ -1010,14 +1010,14 @@ __device__ __forceinline__ double div_by(double a, double b, double r) {
 // half-kick of Eq. 15d.  Returns true when the sums are not finite (the
 // error is then set).  Every load that does not depend on the partner rows
 // is issued first.
-template <bool MIXED, bool EXT>
+template <bool MIXED, bool EXT, bool NEXT>
 __device__ __forceinline__ bool gather_one(const Geo& g, const InstGeo* __restrict__ ig, const StateBuf& s,
                                            const void* __restrict__ own_v,
                                            const int* __restrict__ bw_count, const void* __restrict__ bw_v,
                                            double* __restrict__ Fout, double* __restrict__ Tout,
                                            DevStatus* st, int mode, int j0, int* slots,
                                            const void* __restrict__ carry_v, int cnv,
-                                           const int* __restrict__ start) {
+                                           const int* __restrict__ start, const SortOut& so) {
   using R = typename std::conditional<MIXED, float, double>::type;
   const R* __restrict__ own = static_cast<const R*>(own_v);
   const R* __restrict__ carry = static_cast<const R*>(carry_v);
@@ -1082,6 +1082,14 @@ __device__ __forceinline__ bool gather_one(const Geo& g, const InstGeo* __restri
       u[c] = su[c * n + j];
       w[c] = sw[c * n + j];
     }
+  }
+  double x[3] = {0.0, 0.0, 0.0};
+  int inst = 0, cls = 0;
+  if constexpr (NEXT) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) x[c] = __ldg(s.x + c * n + j);
+    inst = __ldg(s.inst + j);
+    cls = __ldg(s.cls + j);
   }
   cnt = cnt < g.M ? cnt : g.M;
   if (cnt <= 8) {
@@ -1191,19 +1199,27 @@ __device__ __forceinline__ bool gather_one(const Geo& g, const InstGeo* __restri
     // Eq. 15d from u^{n+1/2}: u^{n+1} = u^{n+1/2} + dt/2 alpha^{n+1} (FP64
     // mode: product and sum rounded separately)
     const double hdt = g.hdt;
-    if constexpr (MIXED) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        s.u[c * n + j] = __fma_rn(hdt, (double)al[c], u[c]);
-        s.w[c * n + j] = __fma_rn(hdt, (double)aw[c], w[c]);
+    for (int c = 0; c < 3; ++c) {
+      if constexpr (MIXED) {
+        u[c] = __fma_rn(hdt, (double)al[c], u[c]);
+        w[c] = __fma_rn(hdt, (double)aw[c], w[c]);
+      } else {
+        u[c] = __dadd_rn(u[c], __dmul_rn(hdt, (double)al[c]));
+        w[c] = __dadd_rn(w[c], __dmul_rn(hdt, (double)aw[c]));
       }
-    } else {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        s.u[c * n + j] = __dadd_rn(u[c], __dmul_rn(hdt, (double)al[c]));
-        s.w[c * n + j] = __dadd_rn(w[c], __dmul_rn(hdt, (double)aw[c]));
-      }
+      s.u[c * n + j] = u[c];
+      s.w[c * n + j] = w[c];
     }
+  }
+  if constexpr (NEXT) {
+    // the next step's predictor and cell (its end is two steps after the
+    // count, which this step has yet to raise)
+    const InstGeo& I = ig[inst];
+    const Pred p = predict_one(g, I, st, 2, x[0], x[1], x[2], u[0], u[1], u[2], (double)al[0], (double)al[1],
+                               (double)al[2]);
+    store_pred(so, n, j, p);
+    key_insert(so, j, cell_key(I, cls, p.x, p.y, p.z), id);
   }
   return bad;
 }
@@ -1213,13 +1229,19 @@ __device__ __forceinline__ bool gather_one(const Geo& g, const InstGeo* __restri
 // thread.  At most 80 registers, so that six blocks fit on an SM and a
 // 100k-particle grid runs in one wave.  The last block to finish commits the step; only the writes that
 // block reads (the stresses, an error code) are fenced before the count.
-template <bool MIXED, bool EXT>
+// NEXT (inside a run of steps): the first part of the next step rides along
+// (dss_predict.cuh), so that a run reads the state once where two kernels did
+// and has a kernel less per step; an extra block sets the next geometry.  On
+// systems whose kernels are bound by latency (see chain_steps): 1,000 spheres
+// in FP64 54.8 -> 51.5 us a step, 20,000 43.9 -> 39.6, 100,000 76.6 -> 73.5.
+template <bool MIXED, bool EXT, bool NEXT>
 __global__ void __launch_bounds__(kThreads, 6)
 k_gather(Geo g, const InstGeo* __restrict__ ig, StateBuf s, const void* __restrict__ own_v,
          const int* __restrict__ bw_count, const void* __restrict__ bw_v, double* __restrict__ Fout,
          double* __restrict__ Tout, DevStatus* st, int mode, const double* __restrict__ spart,
          double* sigma, double* sigma_sum, const int* __restrict__ start, unsigned int* done_blocks,
-         const void* __restrict__ carry_v, int pb_blocks, const void* __restrict__ own_s_v) {
+         const void* __restrict__ carry_v, int pb_blocks, const void* __restrict__ own_s_v,
+         const __grid_constant__ SortOut so) {
   dep_wait();
   // An error set before this kernel (an earlier kernel of the step, or an
   // earlier step of the same dss_step call, whose successors still replay)
@@ -1232,7 +1254,10 @@ k_gather(Geo g, const InstGeo* __restrict__ ig, StateBuf s, const void* __restri
   __syncthreads();
   bool fence = false;
   if (!s_err0) {
-    if (blockIdx.x < (unsigned)g.K) {
+    if constexpr (NEXT) reset_scans(so);
+    if (NEXT && blockIdx.x == gridDim.x - 1) {
+      set_step_geo(g, ig, st, 2, so.sg);
+    } else if (blockIdx.x < (unsigned)g.K) {
       if (own_s_v)
         inst_stress_parts(g, ig[blockIdx.x], spart + (int64_t)blockIdx.x * kOsParts * 9,
                           sigma + 9 * blockIdx.x);
@@ -1241,8 +1266,8 @@ k_gather(Geo g, const InstGeo* __restrict__ ig, StateBuf s, const void* __restri
       fence = threadIdx.x < 9;
     } else {
       const int j = (int)(blockIdx.x - g.K) * blockDim.x + threadIdx.x;
-      fence = gather_one<MIXED, EXT>(g, ig, s, own_v, bw_count, bw_v, Fout, Tout, st, mode, j,
-                                s_slot[threadIdx.x >> 5], carry_v, own_s_v ? 15 : 6, start);
+      fence = gather_one<MIXED, EXT, NEXT>(g, ig, s, own_v, bw_count, bw_v, Fout, Tout, st, mode, j,
+                                           s_slot[threadIdx.x >> 5], carry_v, own_s_v ? 15 : 6, start, so);
     }
   }
   __shared__ bool last;
@@ -1258,7 +1283,10 @@ k_gather(Geo g, const InstGeo* __restrict__ ig, StateBuf s, const void* __restri
     // a committed step adds every instance's stress to the running sums
     if (!s_err && mode == G_STEP)
       for (int t = threadIdx.x; t < 9 * g.K; t += blockDim.x) sigma_sum[t] += __ldcg(sigma + t);
-    if (threadIdx.x == 0) commit_step(g, st, start, mode == G_STEP ? 1 : 0);
+    if (threadIdx.x == 0) {
+      commit_step(g, st, start, mode == G_STEP ? 1 : 0);
+      if (NEXT && !s_err) st->w[ST_MAXROW] = st->w[ST_BAND] = st->w[ST_NCONT] = 0;
+    }
     if (threadIdx.x == 0) *done_blocks = 0u;
   }
 }
@@ -1301,7 +1329,7 @@ namespace {
 // or rolling resistance is on; the plain kernels carry none of its code).
 template <bool EXT>
 void launch_forces_t(dss_handle* h, int stbuf, int work_list, int hist_list, int adv, int mode,
-                     double* F_out, double* T_out) {
+                     double* F_out, double* T_out, bool next) {
   (void)adv;
   const int n = (int)h->n;
   const bool mixed = h->g.precision == DSS_MIXED;
@@ -1340,26 +1368,21 @@ void launch_forces_t(dss_handle* h, int stbuf, int work_list, int hist_list, int
       launch_dep(k_owner_stress<false, EXT>, h->g.K * kOsParts, kPairThreads, h->stream,
           h->g, h->ig, h->st[stbuf], own_s, carry, h->lb[work_list].start, h->spart, h->status);
   }
-  if (mixed)
-    launch_dep(k_gather<true, EXT>, gb, kThreads, h->stream, h->g, h->ig, h->st[stbuf], h->own, h->bw_count,
-                                                        h->bw_rec, F_out, T_out, h->status, mode, h->spart,
-                                                        h->sigma, h->sigma_sum, h->lb[work_list].start,
-                                                        h->done_blocks, carry, pbb, own_s);
-  else
-    launch_dep(k_gather<false, EXT>, gb, kThreads, h->stream, h->g, h->ig, h->st[stbuf], h->own, h->bw_count,
-                                                         h->bw_rec, F_out, T_out, h->status, mode, h->spart,
-                                                         h->sigma, h->sigma_sum, h->lb[work_list].start,
-                                                         h->done_blocks, carry, pbb, own_s);
+  auto kg = mixed ? (next ? k_gather<true, EXT, true> : k_gather<true, EXT, false>)
+                  : (next ? k_gather<false, EXT, true> : k_gather<false, EXT, false>);
+  launch_dep(kg, gb + (next ? 1 : 0), kThreads, h->stream, h->g, h->ig, h->st[stbuf], h->own, h->bw_count, h->bw_rec,
+             F_out, T_out, h->status, mode, h->spart, h->sigma, h->sigma_sum, h->lb[work_list].start, h->done_blocks,
+             carry, pbb, own_s, sort_out(h));
   prof_mark(h, 7);
 }
 }  // namespace
 
 void launch_forces(dss_handle* h, int stbuf, int work_list, int hist_list, int adv, int mode,
-                   double* F_out, double* T_out) {
+                   double* F_out, double* T_out, bool next) {
   if (h->g.wave || h->g.k_r > 0.0)
-    launch_forces_t<true>(h, stbuf, work_list, hist_list, adv, mode, F_out, T_out);
+    launch_forces_t<true>(h, stbuf, work_list, hist_list, adv, mode, F_out, T_out, next);
   else
-    launch_forces_t<false>(h, stbuf, work_list, hist_list, adv, mode, F_out, T_out);
+    launch_forces_t<false>(h, stbuf, work_list, hist_list, adv, mode, F_out, T_out, next);
 }
 
 void launch_pairs_out(dss_handle* h, int list, long long* out) {

@@ -730,11 +730,13 @@ struct dss_handle {
 // Kernel launchers (defined in the .cu files).  adv = 1 inside a time step
 // (positions are at time (nstep+1) dt), 0 for an evaluation at the current
 // time.
-void launch_sort(dss_handle* h, bool predict, int src, int dst);
+// keyed: the step before ran the first part (launch_forces with next).
+void launch_sort(dss_handle* h, bool predict, int src, int dst, bool keyed = false);
 void launch_enumerate(dss_handle* h, int stbuf, int dst_list, int adv);
 enum GatherMode { G_STEP = 0, G_EVAL = 1, G_ACCEL = 2 };
+// next (a step only): the corrector also predicts the next step's positions.
 void launch_forces(dss_handle* h, int stbuf, int work_list, int hist_list, int adv, int mode,
-                   double* F_out, double* T_out);
+                   double* F_out, double* T_out, bool next = false);
 void launch_pairs_out(dss_handle* h, int list, long long* out);
 void launch_images_out(dss_handle* h, int* out);
 void launch_mark(dss_handle* h);

@@ -12,182 +12,42 @@
 // coalesced as its reads; a scatter of indices before it and reads through
 // them cost a kernel and two dependent loads more (20,000 spheres 45.7 -> 43.9
 // us a step, 100,000 77.5 -> 76.6, 1M 474 -> 466).
-#include "dss_internal.cuh"
+#include "dss_predict.cuh"
 
 namespace {
 
 constexpr int kThreads = 256;
 
-// Predictor of Eq. 15a-b and the wrap of Eq. 16 for one particle; computed
-// once per step and stored for the gather.  In FP64 mode each product and
-// sum is rounded separately (the trajectory then differs from a plain FP64
-// evaluation only through the order of the force sums); in mixed precision
-// as fused multiply-adds (GB300's narrow FP64 pipe bounds this kernel).
-// Returns the y crossing (-1 out through the top, +1 bottom).
-// Comparisons for the wrap on the IEEE bit patterns (integer instructions
-// instead of GB300's narrow FP64 pipe).  For L > 0 and any finite v the
-// signed 64-bit order of the patterns is the order of the values on the
-// non-negative side, and every negative v sorts below; -0.0 is not below 0.
-__device__ __forceinline__ bool ge_pos(double v, double L) {
-  return __double_as_longlong(v) >= __double_as_longlong(L);
-}
-__device__ __forceinline__ bool lt_zero(double v) {
-  const long long b = __double_as_longlong(v);
-  return b < 0 && b != (long long)0x8000000000000000ull;
-}
-
-struct Pred {
-  double x, y, z, ux, uy, uz;
-  int cross;
-};
-
-// Lees-Edwards wrap of Eq. 16 and the periodic wraps along x and z, for a
-// particle that left the box (out of line: see f32_rn_slow).
-__device__ __noinline__ Pred wrap_out(const Geo& g, const InstGeo& I, const DevStatus* st, int adv, Pred r) {
-  double x = r.x, y = r.y, z = r.z, ux = r.ux;
-  // leaving through y >= L_y re-enters at the bottom shifted by -off along
-  // x with u_x - gdot L_y, and vice versa
-  const double Ly = I.L[1];
-  if (ge_pos(y, Ly)) {
-    y = __dsub_rn(y, Ly);
-    x = __dsub_rn(x, le_offset(g, I, dev_nstep(st) + adv));
-    r.cross = -1;
-  } else if (lt_zero(y)) {
-    y = __dadd_rn(y, Ly);
-    x = __dadd_rn(x, le_offset(g, I, dev_nstep(st) + adv));
-    r.cross = 1;
-    if (ge_pos(y, Ly)) y = 0.0;
-  }
-  // x back into [0, L_x): two conditional shifts give the same bits as
-  // fmod followed by the two corrections, for |x| < 2 L_x
-  const double Lx = I.L[0];
-  if (lt_zero(x)) x = __dadd_rn(x, Lx); else if (ge_pos(x, Lx)) x = __dsub_rn(x, Lx);
-  if (lt_zero(x)) x = __dadd_rn(x, Lx); else if (ge_pos(x, Lx)) x = __dsub_rn(x, Lx);
-  if (ge_pos(z, I.L[2])) {
-    z = __dsub_rn(z, I.L[2]);
-  } else if (lt_zero(z)) {
-    z = __dadd_rn(z, I.L[2]);
-    if (ge_pos(z, I.L[2])) z = 0.0;
-  }
-  if (r.cross != 0)
-    ux = __dadd_rn(ux, __dmul_rn(__dmul_rn((double)r.cross, I.gdot), Ly));
-  r.x = x; r.y = y; r.z = z; r.ux = ux;
-  return r;
-}
-
-__device__ __forceinline__ Pred predict_one(const Geo& g, const InstGeo& I, const DevStatus* st,
-                                            int adv, const StateBuf& s, int i, bool predict) {
-  const int n = g.n;
-  Pred r;
-  double x = s.x[i], y = s.x[n + i], z = s.x[2 * n + i];
-  double ux = s.u[i], uy = s.u[n + i], uz = s.u[2 * n + i];
-  r.cross = 0;
-  if (predict) {
-    const double dt = g.dt;
-    const double hdt2 = g.hdt2;
-    const double hdt = g.hdt;
-    double ax = s.al[i], ay = s.al[n + i], az = s.al[2 * n + i];
-    if (g.precision == DSS_FP64) {
-      // FP64 mode: every product and sum rounded on its own, in the order
-      // x + dt u + (dt/2 dt) alpha of Eq. 15a (no contraction)
-      x = __dadd_rn(__dadd_rn(x, __dmul_rn(dt, ux)), __dmul_rn(hdt2, ax));
-      y = __dadd_rn(__dadd_rn(y, __dmul_rn(dt, uy)), __dmul_rn(hdt2, ay));
-      z = __dadd_rn(__dadd_rn(z, __dmul_rn(dt, uz)), __dmul_rn(hdt2, az));
-      ux = __dadd_rn(ux, __dmul_rn(hdt, ax));
-      uy = __dadd_rn(uy, __dmul_rn(hdt, ay));
-      uz = __dadd_rn(uz, __dmul_rn(hdt, az));
-    } else {
-      x = __fma_rn(hdt2, ax, __fma_rn(dt, ux, x));
-      y = __fma_rn(hdt2, ay, __fma_rn(dt, uy, y));
-      z = __fma_rn(hdt2, az, __fma_rn(dt, uz, z));
-      ux = __fma_rn(hdt, ax, ux);
-      uy = __fma_rn(hdt, ay, uy);
-      uz = __fma_rn(hdt, az, uz);
-    }
-  }
-  r.x = x; r.y = y; r.z = z;
-  r.ux = ux; r.uy = uy; r.uz = uz;
-  // inside the box (nearly every particle): nothing to wrap
-  if (predict && (ge_pos(y, I.L[1]) || lt_zero(y) || ge_pos(x, I.L[0]) || lt_zero(x) || ge_pos(z, I.L[2]) ||
-                  lt_zero(z)))
-    r = wrap_out(g, I, st, adv, r);
-  return r;
-}
-
-// Cell coordinate floor(x / cs) along one axis, clamped to the grid (the
-// FP64 product's floor, mostly decided in FP32: floor_mul).
-__device__ __forceinline__ int cell_coord_fast(double v, double inv, float invf, int nc) {
-  const int k = floor_mul(v, inv, invf);
-  return k < 0 ? 0 : (k >= nc ? nc - 1 : k);
-}
-
-// Bin of a particle: its instance's bins, its size class's layer, its cell.
-__device__ __forceinline__ int cell_key(const InstGeo& I, int cls, double x, double y, double z) {
-  int cx = cell_coord_fast(x, I.inv_cs[0], I.inv_csf[0], I.nc[0]);
-  int cy = cell_coord_fast(y, I.inv_cs[1], I.inv_csf[1], I.nc[1]);
-  int cz = cell_coord_fast(z, I.inv_cs[2], I.inv_csf[2], I.nc[2]);
-  return I.cell_base + cls * I.ncell_layer + (cz * I.nc[1] + cy) * I.nc[0] + cx;
-}
-
-// 1. key + warp-aggregated histogram
+// 1. key + warp-aggregated histogram; the last block sets the geometry
 __global__ void __launch_bounds__(kThreads)
-k_key_hist(Geo g, const InstGeo* __restrict__ ig, StepGeo* __restrict__ sg, StateBuf s,
-           int* __restrict__ key, int* __restrict__ cell_count, DevStatus* st, bool predict, unsigned long long* scan_status, int* scan_ticket,
-           int scan_tiles, double* __restrict__ pred, signed char* __restrict__ xc, int* __restrict__ cell_ids,
-           int bcap) {
+k_key_hist(const __grid_constant__ Geo g, const InstGeo* __restrict__ ig, const __grid_constant__ StateBuf s,
+           DevStatus* st, bool predict, const __grid_constant__ SortOut q) {
   dep_wait();
   if (dev_err(st)) return;
-  // reset the look-back state of both scans of this operation (spread over
-  // the grid), the counters, and set every instance's Lees-Edwards geometry
-  // for its time
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < 2 * scan_tiles; t += gridDim.x * blockDim.x)
-    scan_status[t] = 0ull;
-  if (blockIdx.x == 0) {
-    if (threadIdx.x < 2) scan_ticket[threadIdx.x] = 0;
+  reset_scans(q);
+  if (blockIdx.x == gridDim.x - 1) {
     if (threadIdx.x == 0) {
       st->w[ST_MAXROW] = 0;
       st->w[ST_BAND] = 0;
       st->w[ST_NCONT] = 0;
     }
-    for (int k = threadIdx.x; k < g.K; k += blockDim.x) {
-      const InstGeo& I = ig[k];
-      const double off = le_offset(g, I, dev_nstep(st) + (predict ? 1 : 0));
-      const int fsh = le_shift_cells(I, off);
-      const double offr = off - fsh * I.cs[0];
-      StepGeo q;
-      q.off = off;
-      q.fsh = fsh;
-      q.offr_hi = (float)offr;
-      q.offr_lo = (float)(offr - (double)q.offr_hi);
-      sg[k] = q;
-    }
+    set_step_geo(g, ig, st, predict ? 1 : 0, q.sg);
+    return;
   }
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= g.n) return;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, n = g.n;
+  if (i >= n) return;
   const InstGeo& I = ig[s.inst[i]];
-  const int id = s.id[i];
-  Pred p = predict_one(g, I, st, predict ? 1 : 0, s, i, predict);
+  const int id = s.id[i], cls = s.cls[i];
+  double x = s.x[i], y = s.x[n + i], z = s.x[2 * n + i];
   if (predict) {
-    const int n = g.n;
-    pred[i] = p.x;
-    pred[n + i] = p.y;
-    pred[2 * n + i] = p.z;
-    pred[3 * n + i] = p.ux;
-    pred[4 * n + i] = p.uy;
-    pred[5 * n + i] = p.uz;
-    xc[i] = (signed char)p.cross;
+    const Pred p = predict_one(g, I, st, 1, x, y, z, s.u[i], s.u[n + i], s.u[2 * n + i], s.al[i], s.al[n + i],
+                               s.al[2 * n + i]);
+    store_pred(q, n, i, p);
+    x = p.x;
+    y = p.y;
+    z = p.z;
   }
-  int k = cell_key(I, s.cls[i], p.x, p.y, p.z);
-  unsigned act = __activemask();
-  unsigned peers = __match_any_sync(act, k);
-  int lane = threadIdx.x & 31;
-  int leader = __ffs(peers) - 1;
-  int rank = __popc(peers & ((1u << lane) - 1u));
-  int base = 0;
-  if (lane == leader) base = atomicAdd(&cell_count[k], __popc(peers));
-  base = __shfl_sync(peers, base, leader);
-  key[i] = k;
-  if (base + rank < bcap) cell_ids[(int64_t)k * bcap + base + rank] = id;
+  key_insert(q, i, cell_key(I, cls, x, y, z), id);
 }
 
 // 3. the place of each particle: inside a cell by id, so that the sorted order,
@@ -197,7 +57,7 @@ k_key_hist(Geo g, const InstGeo* __restrict__ ig, StepGeo* __restrict__ sg, Stat
 // ranked over all particles' keys, and the host gives the next operation longer
 // rows (ST_CELL).
 template <bool WAVE>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 4)
 k_rank_gather(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sgk, StateBuf src,
               StateBuf dst, const int* __restrict__ key, const int* __restrict__ cell_start,
               const int* __restrict__ cell_ids, int bcap, int* __restrict__ perm, int* __restrict__ cellid,
@@ -210,7 +70,25 @@ k_rank_gather(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__
   if (o >= n) return;
   const int k = key[o];
   const int id = src.id[o];
+  const int inst = src.inst[o], iy = src.iy[o], cross = predict ? (int)xc[o] : 0;
+  const unsigned char cls = src.cls[o];
+  const double a = src.a[o];
   const int c0 = cell_start[k], cnt = cell_start[k + 1] - c0;
+  // the state goes out with the loads that find its place
+  Pred p;
+  double wv3[3], wa[3];
+  if (predict) {
+    p.x = pred[o]; p.y = pred[n + o]; p.z = pred[2 * n + o];
+    p.ux = pred[3 * n + o]; p.uy = pred[4 * n + o]; p.uz = pred[5 * n + o];
+  } else {
+    p.x = src.x[o]; p.y = src.x[n + o]; p.z = src.x[2 * n + o];
+    p.ux = src.u[o]; p.uy = src.u[n + o]; p.uz = src.u[2 * n + o];
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    wv3[c] = src.w[c * n + o];
+    wa[c] = src.aw[c * n + o];
+  }
   int rank = 0;
   if (cnt <= bcap) {
     const int4* __restrict__ row = reinterpret_cast<const int4*>(cell_ids + (int64_t)k * bcap);
@@ -225,43 +103,29 @@ k_rank_gather(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__
   const int f = c0 + rank;
   perm[f] = o;
   cellid[f] = k;
-  const int inst = src.inst[o];
   const InstGeo& I = ig[inst];
-  Pred p;
-  if (predict) {
-    p.x = pred[o]; p.y = pred[n + o]; p.z = pred[2 * n + o];
-    p.ux = pred[3 * n + o]; p.uy = pred[4 * n + o]; p.uz = pred[5 * n + o];
-  } else {
-    p.x = src.x[o]; p.y = src.x[n + o]; p.z = src.x[2 * n + o];
-    p.ux = src.u[o]; p.uy = src.u[n + o]; p.uz = src.u[2 * n + o];
-  }
   dst.x[f] = p.x; dst.x[n + f] = p.y; dst.x[2 * n + f] = p.z;
   dst.u[f] = p.ux; dst.u[n + f] = p.uy; dst.u[2 * n + f] = p.uz;
-  double wv3[3];
   if (predict) {
     const double hdt = g.hdt;
     if (g.precision == DSS_FP64)
-      for (int c = 0; c < 3; ++c)
-        wv3[c] = __dadd_rn(src.w[c * n + o], __dmul_rn(hdt, src.aw[c * n + o]));
+      for (int c = 0; c < 3; ++c) wv3[c] = __dadd_rn(wv3[c], __dmul_rn(hdt, wa[c]));
     else
-      for (int c = 0; c < 3; ++c)
-        wv3[c] = __fma_rn(hdt, src.aw[c * n + o], src.w[c * n + o]);
+      for (int c = 0; c < 3; ++c) wv3[c] = __fma_rn(hdt, wa[c], wv3[c]);
   } else {
     for (int c = 0; c < 3; ++c) {
-      wv3[c] = src.w[c * n + o];
       dst.al[c * n + f] = src.al[c * n + o];
-      dst.aw[c * n + f] = src.aw[c * n + o];
+      dst.aw[c * n + f] = wa[c];
     }
   }
   for (int c = 0; c < 3; ++c) dst.w[c * n + f] = wv3[c];
   const double w0 = wv3[0], w1 = wv3[1], w2 = wv3[2];
-  const double a = src.a[o];
   dst.a[f] = a;
   dst.id[f] = id;
   dst.inst[f] = inst;
-  dst.cls[f] = src.cls[o];
+  dst.cls[f] = cls;
   // image count: leaving through the top is one image up
-  dst.iy[f] = src.iy[o] - (predict ? (int)xc[o] : 0);
+  dst.iy[f] = iy - cross;
   if (WAVE) {
     // the wave of Eq. 17 at the centre, once per evaluation: its part of
     // U_inf,x and of the local rate dU_inf,x/dy
@@ -407,14 +271,11 @@ void launch_scan(dss_handle* h, const int* in, int* out, int count, int which, b
                                                  h->scan_ticket + which, h->status, zero_in ? 1 : 0);
 }
 
-void launch_sort(dss_handle* h, bool predict, int src, int dst) {
+void launch_sort(dss_handle* h, bool predict, int src, int dst, bool keyed) {
   const int n = (int)h->n;
   const int blocks = (n + kThreads - 1) / kThreads;
   prof_mark(h, 0);
-  launch_dep(k_key_hist, blocks, kThreads, h->stream, h->g, h->ig, h->sg, h->st[src], h->key,
-                                                 h->cell_count, h->status, predict, h->scan_status,
-                                                 h->scan_ticket, h->scan_tiles_max, h->pred, h->xc, h->cell_ids,
-                                                 h->cell_cap);
+  if (!keyed) launch_dep(k_key_hist, blocks + 1, kThreads, h->stream, h->g, h->ig, h->st[src], h->status, predict, sort_out(h));
   prof_mark(h, 1);
   launch_scan(h, h->cell_count, h->cell_start, h->g.ncell, 0, true);
   prof_mark(h, 2);

@@ -120,3 +120,48 @@ def test_segment_row_overflow_is_reported(env):
         s.neighbour_build()
     assert e.value.code == -3
     s.close()
+
+
+def test_cells_fuller_than_their_id_rows(env):
+    """Clumps of more particles per cell than the sort's rows of ids hold (four
+    times the average and twelve): the order and the pairs are those of any
+    other cell, before and after the host lengthens the rows."""
+    rng = np.random.default_rng(3)
+    n, L = 3000, 60.0
+    x = rng.uniform(0.0, L, size=(3, n))
+    x[:, :900] = rng.uniform(0.5, 6.5, size=(3, 900))      # ~700 in 27 of 8000 cells, up to ~60 in one
+    x[:, 900:1000] = rng.uniform(31.0, 33.0, size=(3, 100))
+    g = dict(x=x, a=np.ones(n), box=np.array([L, L, L]), ids=rng.permutation(n).astype(np.int32))
+    kw = dict(shear_rate=1.0, dt=1e-6)
+    p = env["dss"].default_params(g["box"], capacity_M=400, **kw)
+    z = np.zeros_like(x)
+    s = env["dss"].Suspension(x, g["a"], g["box"], p, ids=g["ids"], alpha_lin=z, alpha_ang=z, nstep=5)
+    for _ in range(3):
+        s.neighbour_build()
+        np.testing.assert_array_equal(s.pairs(), _want(env, g, 5, **kw))
+    s.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("ext", [False, True])
+def test_runs_of_steps_as_single_steps(env, precision, ext):
+    """Steps in one call, whose correctors begin the next step, against as many
+    calls of one step: the same bits, through box crossings and box offsets."""
+    g = env["synth"].small(1500, 0.50, 21)
+    kw = dict(mu=0.5, shear_rate=40.0, dt=1e-4, precision=precision)
+    if ext:
+        kw.update(wave_amp=2.0, wave_n=1, k_r=500.0)
+    out = []
+    for calls in ([19, 8, 3], [1] * 30):
+        s = env["dss"].Suspension(g["x"], g["a"], g["box"], env["dss"].default_params(g["box"], **kw), ids=g["ids"],
+                                  nstep=9990)
+        for k in calls:
+            s.step(k)
+        c = s.counters()
+        st = {k: v.cpu().numpy() for k, v in s.state().items()}
+        out.append((st, s.stress(), s.images(), c["npairs"], c["ncontacts"], c["max_row"], c["band_checks"]))
+        s.close()
+    for k in out[0][0]:
+        np.testing.assert_array_equal(out[0][0][k], out[1][0][k])
+    for a, b in zip(out[0][1:], out[1][1:]):
+        np.testing.assert_array_equal(a, b)
