@@ -82,12 +82,11 @@ void free_buffers(dss_handle* h) {
 }
 
 void drop_graphs(dss_handle* h) {
-  for (int k = 0; k < 4; ++k) {
-    if (h->graph_ok[k]) cudaGraphExecDestroy(h->step_graph[k]);
-    h->graph_ok[k] = false;
-    if (h->multi_ok[k]) cudaGraphExecDestroy(h->multi_graph[k]);
-    h->multi_ok[k] = false;
-  }
+  for (int g = 0; g < DSS_GRAPHS; ++g)
+    for (int k = 0; k < 4; ++k) {
+      if (h->graph_ok[g][k]) cudaGraphExecDestroy(h->step_graph[g][k]);
+      h->graph_ok[g][k] = false;
+    }
 }
 
 // Pair-capacity dependent buffers: per-pair records, stretch, contact flags,
@@ -340,6 +339,13 @@ const void* device_view(const void* p) {
   return nullptr;
 }
 
+bool is_device(const void* p) {
+  cudaPointerAttributes at;
+  const bool dev = cudaPointerGetAttributes(&at, p) == cudaSuccess && at.type == cudaMemoryTypeDevice;
+  cudaGetLastError();
+  return dev;
+}
+
 // Tile 1 of a look-back whose tile 0 never publishes: the wait must give up.
 __global__ void k_selftest_wait(unsigned long long* status, DevStatus* st) {
   lookback_warp(status, 1, 0, st);
@@ -472,34 +478,19 @@ void seq_step(dss_handle* h, bool keyed = false, bool next = false) {
   launch_forces(h, w, 1 - h->hist, h->hist, 1, G_STEP, nullptr, nullptr, next);
 }
 
-int capture_step(dss_handle* h, int key) {
-  cudaGraph_t graph;
-  CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-  h->capturing = true;
-  seq_step(h);
-  h->capturing = false;
-  cudaError_t e = cudaStreamEndCapture(h->stream, &graph);
-  if (e != cudaSuccess) return DSS_ERR_CUDA;
-  e = cudaGraphInstantiate(&h->step_graph[key], graph, 0);
-  cudaGraphDestroy(graph);
-  if (e != cudaSuccess) return DSS_ERR_CUDA;
-  h->graph_ok[key] = true;
-  return DSS_OK;
-}
-
-// DSS_MULTI_STEPS steps in one graph, starting with the buffers in the
-// roles (cur, hist) of key; each step's kernels skip after an earlier
-// failure exactly as in separate launches.
-int capture_multi(dss_handle* h, int key) {
-  const int cur0 = h->cur, hist0 = h->hist;
+// 2^g steps in one graph, starting with the buffers in the roles (cur, hist)
+// of key; each step's kernels skip after an earlier failure exactly as in
+// separate launches.
+int capture_steps(dss_handle* h, int g, int key) {
+  const int cur0 = h->cur, hist0 = h->hist, steps = 1 << g;
   h->cur = key >> 1;
   h->hist = key & 1;
   cudaGraph_t graph;
   const bool chain = chain_steps(h);
   CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
   h->capturing = true;
-  for (int k = 0; k < DSS_MULTI_STEPS; ++k) {
-    seq_step(h, chain && k > 0, chain && k + 1 < DSS_MULTI_STEPS);
+  for (int k = 0; k < steps; ++k) {
+    seq_step(h, chain && k > 0, chain && k + 1 < steps);
     h->cur = 1 - h->cur;
     h->hist = 1 - h->hist;
   }
@@ -508,10 +499,10 @@ int capture_multi(dss_handle* h, int key) {
   h->hist = hist0;
   cudaError_t e = cudaStreamEndCapture(h->stream, &graph);
   if (e != cudaSuccess) return DSS_ERR_CUDA;
-  e = cudaGraphInstantiate(&h->multi_graph[key], graph, 0);
+  e = cudaGraphInstantiate(&h->step_graph[g][key], graph, 0);
   cudaGraphDestroy(graph);
   if (e != cudaSuccess) return DSS_ERR_CUDA;
-  h->multi_ok[key] = true;
+  h->graph_ok[g][key] = true;
   return DSS_OK;
 }
 
@@ -1062,10 +1053,7 @@ int get_state_enqueue(dss_handle* h, double* const out[5]) {
   for (int k = 0; k < 5; ++k) {
     direct.d[k] = staged.d[k] = views.d[k] = nullptr;
     if (!out[k]) continue;
-    cudaPointerAttributes at;
-    const bool is_dev = cudaPointerGetAttributes(&at, out[k]) == cudaSuccess && at.type == cudaMemoryTypeDevice;
-    cudaGetLastError();
-    if (is_dev) {
+    if (is_device(out[k])) {
       direct.d[k] = out[k];
     } else {
       staged.d[k] = h->stage + (size_t)k * 3 * n;
@@ -1154,19 +1142,29 @@ int dss_force_eval(dss_handle* h, double* F, double* T) {
   if (!h) return DSS_ERR_ARG;
   if (!h->have_state) return DSS_ERR_STATE;
   ENTER(h);
-  const int n = (int)h->n;
+  const size_t b3 = sizeof(double) * 3 * (size_t)h->n;
+  // (device outputs are written by the kernel itself)
+  double* const Fd = F && !is_device(F) ? h->io3 : F;
+  double* const Td = T && !is_device(T) ? h->io3b : T;
+  const int list = 1 - h->hist;
   seq_sort_enum(h, false, 0);
   h->cur = 1 - h->cur;
-  int rc = ensure_pair_capacity(h, 1 - h->hist);
-  if (rc) return rc;
-  launch_forces(h, h->cur, 1 - h->hist, h->hist, 0, G_EVAL, F ? h->io3 : nullptr,
-                T ? h->io3b : nullptr);
+  launch_forces(h, h->cur, list, h->hist, 0, G_EVAL, Fd, Td);
   CK(cudaGetLastError());
-  if (F) CK(cudaMemcpyAsync(F, h->io3, sizeof(double) * 3 * n, cudaMemcpyDefault, h->stream));
-  if (T) CK(cudaMemcpyAsync(T, h->io3b, sizeof(double) * 3 * n, cudaMemcpyDefault, h->stream));
   int r = sync_status(h);
   if (r) return r;
+  if (status_error(h) == DSS_ERR_CAPACITY && h->status_host->w[ST_NPAIRS] > h->pcap) {
+    // more pairs than the pair arrays hold: grow them, list and evaluate again
+    clear_err(h);
+    if ((r = ensure_pair_capacity(h, list))) return r;
+    launch_forces(h, h->cur, list, h->hist, 0, G_EVAL, Fd, Td);
+    CK(cudaGetLastError());
+    if ((r = sync_status(h))) return r;
+  }
   if ((r = status_error(h))) { clear_err(h); return r; }
+  if (Fd != F) CK(cudaMemcpyAsync(F, Fd, b3, cudaMemcpyDefault, h->stream));
+  if (Td != T) CK(cudaMemcpyAsync(T, Td, b3, cudaMemcpyDefault, h->stream));
+  if (Fd != F || Td != T) CK(cudaStreamSynchronize(h->stream));
   return DSS_OK;
 }
 
@@ -1188,38 +1186,27 @@ int step_launch(dss_handle* h, int64_t remaining, StepRun& run) {
   run.steps0 = h->status_host->w[ST_STEPS];
   run.cur0 = h->cur;
   run.hist0 = h->hist;
-  int c = run.cur0, hs = run.hist0;
-  for (int64_t k = 0; k < remaining; ++k) {
-    if (!h->graph_ok[c * 2 + hs]) {
-      h->cur = c;
-      h->hist = hs;
-      r = capture_step(h, c * 2 + hs);
-      if (r) return r;
-    }
-    c = 1 - c;
-    hs = 1 - hs;
-  }
-  c = run.cur0;
-  hs = run.hist0;
-  // runs of DSS_MULTI_STEPS steps go out as one graph launch (not while
-  // profiling, which times each step's kernels)
-  const int64_t multi = h->profiling ? 0 : remaining / DSS_MULTI_STEPS;
-  if (multi > 0 && !h->multi_ok[c * 2 + hs]) {
-    r = capture_multi(h, c * 2 + hs);
-    if (r) return r;
+  // the fewest graphs (the boundary between two costs about 5 us, that between
+  // two steps of one graph none): runs of 8 steps, then one each of 4, 2 and 1
+  // as they are needed; single steps while profiling, which times each one's
+  // kernels.  Even runs leave the buffers in their roles.
+  const int top = h->profiling ? 0 : DSS_GRAPHS - 1;
+  int key = run.cur0 * 2 + run.hist0;
+  int64_t count[DSS_GRAPHS];
+  int64_t left = remaining;
+  for (int g = top; g >= 0; --g) {
+    count[g] = left >> g;
+    left -= count[g] << g;
+    if (count[g] > 0 && !h->graph_ok[g][key] && (r = capture_steps(h, g, key))) return r;
+    if (g == 0 && count[0] > 1 && !h->graph_ok[0][3 - key] && (r = capture_steps(h, 0, 3 - key))) return r;
   }
   CK(cudaEventRecord(h->step_ev[0], h->stream));
-  for (int64_t k = 0; k < multi; ++k) CK(cudaGraphLaunch(h->multi_graph[c * 2 + hs], h->stream));
-  for (int64_t k = multi * DSS_MULTI_STEPS; k < remaining; ++k) {
-    const int key = c * 2 + hs;
-    CK(cudaGraphLaunch(h->step_graph[key], h->stream));
-    if (h->profiling) {
-      r = accumulate_profile(h);
-      if (r) return r;
+  for (int g = top; g >= 0; --g)
+    for (int64_t k = 0; k < count[g]; ++k) {
+      CK(cudaGraphLaunch(h->step_graph[g][key], h->stream));
+      if (h->profiling && (r = accumulate_profile(h))) return r;
+      if (g == 0) key = 3 - key;
     }
-    c = 1 - c;
-    hs = 1 - hs;
-  }
   CK(cudaEventRecord(h->step_ev[1], h->stream));
   return DSS_OK;
 }

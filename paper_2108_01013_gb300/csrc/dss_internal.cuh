@@ -12,7 +12,7 @@
 
 #define DSS_PI 3.14159265358979323846
 #define DSS_PROF_KERNELS 7
-#define DSS_MULTI_STEPS 8
+#define DSS_GRAPHS 4
 
 // Device status word layout (int32 slots in DevStatus::w).
 enum {
@@ -705,13 +705,10 @@ struct dss_handle {
   double* stage;     // 15n: staging of the five state vectors for host transfers
   int* io_id;        // n
   int last_list;     // list written by the last enumeration
-  // graphs: one per (cur, hist) combination
-  cudaGraphExec_t step_graph[4];
-  bool graph_ok[4];
-  // DSS_MULTI_STEPS consecutive steps in one graph (an even count: the
-  // buffers are back in their roles after it), one per (cur, hist) start
-  cudaGraphExec_t multi_graph[4];
-  bool multi_ok[4];
+  // graphs of 1, 2, 4 and 8 steps (log2 of the steps), one per (cur, hist)
+  // combination they start from; captured when first needed
+  cudaGraphExec_t step_graph[DSS_GRAPHS][4];
+  bool graph_ok[DSS_GRAPHS][4];
   // kernel shapes chosen by dss_autotune_kernels (0: the built-in rule):
   // resident pair blocks per SM the register budget is cut for (3 or 4), and
   // the enumeration's search (1: walked by owner, 4: staged by segments)
