@@ -37,7 +37,7 @@ void free_buffers(dss_handle* h) {
     dfree(s.x); dfree(s.u); dfree(s.w); dfree(s.al); dfree(s.aw); dfree(s.a); dfree(s.id); dfree(s.inst);
     dfree(s.cls);
     dfree(s.iy);
-    dfree(s.vf); dfree(s.wf); dfree(s.posl); dfree(s.cellc); dfree(s.wv);
+    dfree(s.rec); dfree(s.wvf); dfree(s.wv);
     memset(&s, 0, sizeof(s));
     ListBuf& L = h->lb[b];
     dfree(L.count); dfree(L.list); dfree(L.start); dfree(L.xi); dfree(L.xr); dfree(L.slot_of_id);
@@ -160,8 +160,7 @@ int alloc_buffers(dss_handle* h) {
         (r = dalloc(h, &s.iy, n)))
       return r;
     if (h->p.precision == DSS_MIXED &&
-        ((r = dalloc(h, &s.vf, n)) || (r = dalloc(h, &s.wf, n)) || (r = dalloc(h, &s.posl, n)) ||
-         (r = dalloc(h, &s.cellc, n))))
+        ((r = dalloc(h, &s.rec, 2 * n)) || (h->g.wave && (r = dalloc(h, &s.wvf, n)))))
       return r;
     if (h->g.wave && (r = dalloc(h, &s.wv, n))) return r;
     ListBuf& L = h->lb[b];

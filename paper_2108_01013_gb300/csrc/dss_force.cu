@@ -213,18 +213,20 @@ __device__ __forceinline__ PairRes<double> pair_eval_fp64(const Geo& g, const In
 template <bool EXT>
 __device__ __forceinline__ PairRes<float> pair_eval_mixed(const Geo& g, const InstGeo& I, const StateBuf& s,
                                                          const ListBuf& H, const HistRef& hr,
-                                                         const StepGeo& sg,
-                                                         const float4* __restrict__ posf, int i, int j) {
+                                                         const StepGeo& sg, int i, int j) {
   const float gd = I.gdot_f;
   const float k6 = g.f.k6;
   // double-float separation from cell-local hi/lo words and the cell offset
   // (listed pairs are at most `reach` cells apart along y and z; a pair whose
   // rows differ by more crosses y = L_y, its image shifted by +-off along x)
-  const float4 pi = posf[i], pj = posf[j], li = s.posl[i], lj = s.posl[j];
-  const int ci = s.cellc[i], cj = s.cellc[j];
+  const Rec8 gi = load_rec(s.rec + rec_geometry(i)), gj = load_rec(s.rec + rec_geometry(j));
+  const Rec8 mi = load_rec(s.rec + rec_motion(i)), mj = load_rec(s.rec + rec_motion(j));
+  const F3 pi = f3(gi.v[0], gi.v[1], gi.v[2]), pj = f3(gj.v[0], gj.v[1], gj.v[2]);
+  const F3 li = f3(gi.v[4], gi.v[5], gi.v[6]), lj = f3(gj.v[4], gj.v[5], gj.v[6]);
+  const int ci = __float_as_int(mi.v[6]), cj = __float_as_int(mj.v[6]);
   // the ids and the probe of the committed rows go out with the state loads
   // (their latency hides behind the geometry; the probe is used by contacts)
-  const int idi = s.id[i], idj = s.id[j];
+  const int idi = __float_as_int(mi.v[7]), idj = __float_as_int(mj.v[7]);
   const HistProbe pr = hist_probe(g, H, hr, i, j, idi, idj);
   const int nx = I.nc[0], ny = I.nc[1], nz = I.nc[2];
   const int R = g.reach;
@@ -256,7 +258,7 @@ __device__ __forceinline__ PairRes<float> pair_eval_mixed(const Geo& g, const In
   cz.lo += lj.z - li.z;
   const FF dxf = ff_add_abs(two_sum(pj.x, -pi.x), cx), dyf = ff_add_abs(two_sum(pj.y, -pi.y), cy),
            dzf = ff_add_abs(two_sum(pj.z, -pi.z), cz);
-  const FF Sff = ff_add_abs(FF{pi.w, li.w}, FF{pj.w, lj.w});
+  const FF Sff = ff_add_abs(FF{gi.v[3], gi.v[7]}, FF{gj.v[3], gj.v[7]});
   const FF r2ff = ff_add_abs(ff_add_abs(ff_sqr(dxf), ff_sqr(dyf)), ff_sqr(dzf));
   const FF numff = ff_add_abs(r2ff, ff_neg(ff_sqr(Sff)));      // r^2 - S^2 to ~2^-45 S^2
   const float num = numff.hi + numff.lo;
@@ -267,10 +269,15 @@ __device__ __forceinline__ PairRes<float> pair_eval_mixed(const Geo& g, const In
   const float d = __fdividef(num, rr + S);
   const F3 r = f3(dxf.hi + dxf.lo, dyf.hi + dyf.lo, dzf.hi + dzf.lo);
   const F3 nn = ir * r;
-  const float4 vi4 = s.vf[i], vj4 = s.vf[j], wi4 = s.wf[i], wj4 = s.wf[j];
-  const F3 Vi = f3(vi4.x, vi4.y, vi4.z), Vj = f3(vj4.x, vj4.y, vj4.z);
-  const F3 Wi = f3(wi4.x, wi4.y, wi4.z), Wj = f3(wj4.x, wj4.y, wj4.z);
-  const float Ai = pi.w + li.w, Bj = pj.w + lj.w;
+  const F3 Vi = f3(mi.v[0], mi.v[1], mi.v[2]), Vj = f3(mj.v[0], mj.v[1], mj.v[2]);
+  const F3 Wi = f3(mi.v[3], mi.v[4], mi.v[5]), Wj = f3(mj.v[3], mj.v[4], mj.v[5]);
+  const float Ai = gi.v[3] + gi.v[7], Bj = gj.v[3] + gj.v[7];
+  // the wave at the centres: its part of the local rate and of U_inf,x
+  float2 qi = make_float2(0.f, 0.f), qj = qi;
+  if (EXT && g.wave) {
+    qi = s.wvf[i];
+    qj = s.wvf[j];
+  }
   PairRes<float> q;
   // ---- contact, Eq. 4-5: the flag here, the forces after the lubrication
   F3 Fc = f3(0, 0, 0), nxf = f3(0, 0, 0), Tr = f3(0, 0, 0);
@@ -309,9 +316,9 @@ __device__ __forceinline__ PairRes<float> pair_eval_mixed(const Geo& g, const In
     F3 du = (Vj - Vi) + f3(gd * r.y, 0.f, 0.f);
     F3 wi = f3(Wi.x, Wi.y, Wi.z - 0.5f * gd), wj = f3(Wj.x, Wj.y, Wj.z - 0.5f * gd);
     if (EXT && g.wave) {
-      du.x += wj4.w - wi4.w;
-      wi.z -= 0.5f * vi4.w;
-      wj.z -= 0.5f * vj4.w;
+      du.x += qj.y - qi.y;
+      wi.z -= 0.5f * qi.x;
+      wj.z -= 0.5f * qj.x;
     }
     const float fn = g.f.kn * d + I.gn_f * dotf(nn, du);
     const F3 ut = tangf(nn, du - crossf(Ai * wi + Bj * wj, nn));
@@ -415,7 +422,7 @@ __device__ __forceinline__ PairRes<float> pair_eval_mixed(const Geo& g, const In
     const float yci = (4.0f * yh) * (A * A), ycj = (4.0f * yh) * (B * B), ycx = yh * AB;
     // strain of the shear rate acting on the pair (the wave of Eq. 17: the
     // mean of the two centres' local rates)
-    const float rate = (EXT && g.wave) ? gd + 0.5f * (vi4.w + vj4.w) : gd;
+    const float rate = (EXT && g.wave) ? gd + 0.5f * (qi.x + qj.x) : gd;
     const float e = 0.5f * S * rate;
     const F3 G = f3((Vi.x - Vj.x) - e * nn.y, (Vi.y - Vj.y) - e * nn.x, Vi.z - Vj.z);
     const float nG = dotf(nn, G), fn = (ya - xa) * nG;
@@ -626,7 +633,7 @@ __device__ __forceinline__ void stress_partials(
 template <bool MIXED, int MINB, bool EXT, bool PERS>
 __global__ void __launch_bounds__(kPairThreads, MINB)
 k_pairs_pb(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sgk, StateBuf s, ListBuf W,
-           ListBuf H, const float4* __restrict__ posf, void* __restrict__ own_v, void* __restrict__ own_s_v,
+           ListBuf H, void* __restrict__ own_v, void* __restrict__ own_s_v,
            void* __restrict__ carry_v, int* __restrict__ bw_count, void* __restrict__ bw_v,
            double* __restrict__ spart, DevStatus* st, const int* __restrict__ perm) {
   dep_wait();
@@ -681,7 +688,7 @@ k_pairs_pb(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sg
       const InstGeo& I = ig[inst];
       const StepGeo sg = sgk[inst];
       PairRes<R> q;
-      if constexpr (MIXED) q = pair_eval_mixed<EXT>(g, I, s, H, hr, sg, posf, i, j);
+      if constexpr (MIXED) q = pair_eval_mixed<EXT>(g, I, s, H, hr, sg, i, j);
       else q = pair_eval_fp64<EXT>(g, I, s, H, hr, sg.off, i, j);
       v[0] = q.F[0]; v[1] = q.F[1]; v[2] = q.F[2];
       v[3] = q.Ti[0]; v[4] = q.Ti[1]; v[5] = q.Ti[2];
@@ -1066,8 +1073,10 @@ __device__ __forceinline__ bool gather_one(const Geo& g, const InstGeo* __restri
   double yj = 0.0, gd = 0.0, fx = 0.0;
   double2 wq = make_double2(0.0, 0.0);
   if constexpr (MIXED) {
-    v4 = __ldg(s.vf + j);
-    w4 = __ldg(s.wf + j);
+    const Rec8 m = load_rec(s.rec + rec_motion(j));
+    v4 = make_float4(m.v[0], m.v[1], m.v[2], 0.f);
+    w4 = make_float4(m.v[3], m.v[4], m.v[5], 0.f);
+    if (EXT && g.wave) w4.w = __ldg(s.wvf + j).y;
   } else {
     yj = __ldg(s.x + n + j);
     gd = __ldg(&ig[__ldg(s.inst + j)].gdot);
@@ -1342,7 +1351,7 @@ void launch_forces_t(dss_handle* h, int stbuf, int work_list, int hist_list, int
   const bool pb4 = mixed && !pers && h->tune_pairs_minb == 4;
   const int pbg = pb4 ? 4 * h->sms : h->pb_blocks;
 #define DSS_PB_ARGS                                                                                     \
-  h->g, h->ig, h->sg, h->st[stbuf], h->lb[work_list], h->lb[hist_list], h->posf, h->own, h->own_s,    \
+  h->g, h->ig, h->sg, h->st[stbuf], h->lb[work_list], h->lb[hist_list], h->own, h->own_s,             \
       h->carry, h->bw_count, h->bw_rec, h->spart, h->status, h->perm
   if (pb4)
     launch_dep(k_pairs_pb<true, 4, EXT, false>, pbg, kPairThreads, h->stream, DSS_PB_ARGS);

@@ -505,6 +505,33 @@ __device__ __forceinline__ FF ff_sqr(FF a) {
 // ------------------------------------------------------------------------
 // Host-side handle
 // ------------------------------------------------------------------------
+// Eight FP32 words: one sector, one load or store instruction.
+struct __align__(32) Rec8 {
+  float v[8];
+};
+// A particle's two records.  Geometry: cell-local position and radius as
+// double-floats, high words x, y, z, a, then the low words.  Motion: velocity
+// relative to U_inf, angular velocity relative to Omega_inf, cell coordinates
+// packed cx | cy << 10 | cz << 20, id.  A pair reads two sectors of each
+// particle instead of the half of six and an eighth of two (four float4 and
+// two int arrays): the pair kernel of a batch of 64 110 -> 102 us, of 1M 115 ->
+// 108, of 100k, whose arrays sit in the L2, 26.5 both.
+__host__ __device__ constexpr int64_t rec_geometry(int64_t i) { return 2 * i; }
+__host__ __device__ constexpr int64_t rec_motion(int64_t i) { return 2 * i + 1; }
+__device__ __forceinline__ Rec8 load_rec(const Rec8* p) {
+  Rec8 r;
+  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3]), "=f"(r.v[4]), "=f"(r.v[5]), "=f"(r.v[6]),
+        "=f"(r.v[7])
+      : "l"(p));
+  return r;
+}
+__device__ __forceinline__ void store_rec(Rec8* p, const Rec8& r) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(r.v[0]), "f"(r.v[1]),
+               "f"(r.v[2]), "f"(r.v[3]), "f"(r.v[4]), "f"(r.v[5]), "f"(r.v[6]), "f"(r.v[7])
+               : "memory");
+}
+
 struct StateBuf {
   double* x;    // 3n positions
   double* u;    // 3n velocity (u^{n+1/2} after the sort of a step)
@@ -516,13 +543,10 @@ struct StateBuf {
   int* inst;    // n instance index
   unsigned char* cls;  // n size class (stencil reach), see Geo::rtab
   int* iy;      // n Lees-Edwards image count along y since the state was set (unwrapped y = y + iy L_y)
-  float4* vf;   // n, mixed precision: FP32 velocity relative to U_inf (xyz); with the wave
-                //    of Eq. 17, w = U k cos(k y) (the wave's part of the local rate)
-  float4* wf;   // n, mixed precision: FP32 angular velocity relative to Omega_inf (xyz); with
-                //    the wave, w = U sin(k y) (the wave's part of U_inf,x)
+  Rec8* rec;    // 2n, mixed precision: what the FP32 pair arithmetic reads of a particle
+                // (rec_geometry, rec_motion)
+  float2* wvf;  // n, mixed precision with the wave: FP32 copy of wv, (U k cos(k y), U sin(k y))
   double2* wv;  // n, wave of Eq. 17 on: (U sin(k y), U k cos(k y)) at the centre
-  float4* posl; // n, mixed precision: low words of the cell-local position and radius
-  int* cellc;   // n, mixed precision: cell coordinates packed cx | cy << 10 | cz << 20
 };
 
 // Tangential stretch of one listed pair and its contact flag (one 32-byte

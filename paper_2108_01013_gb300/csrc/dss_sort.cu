@@ -126,6 +126,9 @@ k_rank_gather(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__
   dst.cls[f] = cls;
   // image count: leaving through the top is one image up
   dst.iy[f] = iy - cross;
+  // FP32 copies relative to the ambient flow for the FP32 pair arithmetic:
+  // u - U_inf(x) and w - Omega_inf are O(gdot a), free of O(gdot L) terms
+  Rec8 mv;
   if (WAVE) {
     // the wave of Eq. 17 at the centre, once per evaluation: its part of
     // U_inf,x and of the local rate dU_inf,x/dy
@@ -134,14 +137,13 @@ k_rank_gather(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__
     const double ws = g.wave_amp * sn, wc = g.wave_amp * I.wave_k * cs;
     dst.wv[f] = make_double2(ws, wc);
     if (g.precision == DSS_MIXED) {
-      dst.vf[f] = make_float4(f32_rn(p.ux - I.gdot * p.y - ws), f32_rn(p.uy), f32_rn(p.uz), f32_rn(wc));
-      dst.wf[f] = make_float4(f32_rn(w0), f32_rn(w1), f32_rn(w2 + 0.5 * (I.gdot + wc)), f32_rn(ws));
+      dst.wvf[f] = make_float2(f32_rn(wc), f32_rn(ws));
+      mv = Rec8{f32_rn(p.ux - I.gdot * p.y - ws), f32_rn(p.uy), f32_rn(p.uz), f32_rn(w0), f32_rn(w1),
+                f32_rn(w2 + 0.5 * (I.gdot + wc))};
     }
   } else if (g.precision == DSS_MIXED) {
-    // FP32 copies relative to the ambient flow for the FP32 pair arithmetic:
-    // u - U_inf(x) and w - Omega_inf are O(gdot a), free of O(gdot L) terms
-    dst.vf[f] = make_float4(f32_rn(p.ux - I.gdot * p.y), f32_rn(p.uy), f32_rn(p.uz), 0.f);
-    dst.wf[f] = make_float4(f32_rn(w0), f32_rn(w1), f32_rn(w2 + 0.5 * I.gdot), 0.f);
+    mv = Rec8{f32_rn(p.ux - I.gdot * p.y), f32_rn(p.uy), f32_rn(p.uz), f32_rn(w0), f32_rn(w1),
+              f32_rn(w2 + 0.5 * I.gdot)};
   }
   // cell-local position (FP32 for the enumeration prefilter; in mixed
   // precision also the low words, for double-float pair geometry)
@@ -161,8 +163,10 @@ k_rank_gather(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__
   f32_split(a, pf.w, pl.w);
   posf[f] = pf;
   if (g.precision == DSS_MIXED) {
-    dst.posl[f] = pl;
-    dst.cellc[f] = cx | (cy << 10) | (cz << 20);
+    mv.v[6] = __int_as_float(cx | (cy << 10) | (cz << 20));
+    mv.v[7] = __int_as_float(id);
+    store_rec(dst.rec + rec_geometry(f), Rec8{pf.x, pf.y, pf.z, pf.w, pl.x, pl.y, pl.z, pl.w});
+    store_rec(dst.rec + rec_motion(f), mv);
   }
   (void)sgk;
 }
