@@ -16,10 +16,9 @@
 //   records of its row taken in increasing owner index (a fixed order, so the
 //   result is bitwise reproducible; rows of 9 to 24 FP32 records and longer
 //   FP64 rows are summed by the whole warp, ranks counted and placed, then a
-//   fixed reduction; longer FP32 rows by their own thread in 64-bit fixed
+//   fixed reduction; longer FP32 rows by eight lanes each in 64-bit fixed
 //   point, whose sum does not depend on the order), Stokes drag (Eq. A1) and
-//   the corrector
-//   of Eq. 15d.  K leading blocks reduce each instance's bulk stress of
+//   the corrector of Eq. 15d.  K leading blocks reduce each instance's bulk stress of
 //   Eq. 8 from the pair blocks' partials; the last block of the gather to
 //   finish adds them to the running sums and commits the step.
 #include <climits>
@@ -224,8 +223,8 @@ __device__ __forceinline__ PairRes<float> pair_eval_mixed(const Geo& g, const In
   const F3 pi = f3(gi.v[0], gi.v[1], gi.v[2]), pj = f3(gj.v[0], gj.v[1], gj.v[2]);
   const F3 li = f3(gi.v[4], gi.v[5], gi.v[6]), lj = f3(gj.v[4], gj.v[5], gj.v[6]);
   const int ci = __float_as_int(mi.v[6]), cj = __float_as_int(mj.v[6]);
-  // the ids and the probe of the committed rows go out with the state loads
-  // (their latency hides behind the geometry; the probe is used by contacts)
+  // the probe of the committed rows goes out with the state loads (its latency
+  // hides behind the geometry; it is used by contacts)
   const int idi = __float_as_int(mi.v[7]), idj = __float_as_int(mj.v[7]);
   const HistProbe pr = hist_probe(g, H, hr, i, j, idi, idj);
   const int nx = I.nc[0], ny = I.nc[1], nz = I.nc[2];
@@ -905,65 +904,78 @@ __device__ __forceinline__ long long fx_of(float v, int e, int bits) {
   return u < 0 ? -m : m;
 }
 
-// A row of more than 8 FP32 records (mixed precision), summed by its own
-// thread in 64-bit fixed point.  Per component the largest exponent e of the
-// row fixes the unit 2^(e - 126 - bits), bits = 62 - ceil(log2(cc + 1)), so
-// that every record is an integer below 2^bits and the row's sum stays below
-// 2^62 (a first pass finds e, a second adds; four records in flight per
-// thread).  Integer addition is
-// associative: the total is a function of the set of records alone, whatever
-// their order in the row, so no ranking and no help from the other lanes is
-// needed.  It is exact up to the dropped bits below 2^-(bits - 24) of each
-// record relative to the row's largest (more accurate than an FP32 running
-// sum).  A non-finite record makes the total NaN.
-__device__ __forceinline__ void row_sum_fixed(const float* __restrict__ row, int cc, float tot[6]) {
-  int e[6] = {0, 0, 0, 0, 0, 0};
-  bool bad = false;
-  int k = 0;
-  for (; k + 4 <= cc; k += 4) {
-    float b[4][8];
+// acc 2^k in FP32 (k in [-190, 80]; two factors of a power of two each).
+__device__ __forceinline__ float fx_float(long long acc, int k) {
+  const int h = k >> 1;
+  return __ll2float_rn(acc) * __int_as_float((h + 127) << 23) * __int_as_float((k - h + 127) << 23);
+}
+
+// The long rows (more than kRankedMax FP32 records) of a warp's particles
+// (mask), four at a time, eight lanes to a row, in 64-bit fixed point.  Per
+// component the largest exponent e of the row fixes the unit 2^(e - 126 -
+// bits), bits = 62 - ceil(log2(cc + 1)), so that every record is an integer
+// below 2^bits and the row's sum stays below 2^62 (a first pass finds e, a
+// second, from L1, adds).  Integer addition is associative: the total is a
+// function of the set of records alone, whatever their order in the row and
+// the lanes, so no ranking is needed.  It is exact up to the dropped bits below
+// 2^-(bits - 24) of each record relative to the row's largest (more accurate
+// than an FP32 running sum).  A non-finite record makes the total NaN.  j, cnt:
+// the lane's particle and its records; F, T: the lane's sums.
+// Neighbouring lanes read neighbouring sectors, and a warp's work is the sum of
+// its rows, not 32 times the longest: the corrector of Table 5 (45 records a
+// row, up to 216) 160 us with a thread to a row, 90 so.  On rows of 9 to 24
+// records the ranked sum of the whole warp is faster (100k with the 1 a0 range
+// 26 against 36 us).
+__device__ __forceinline__ void group_sum_rows(const float* __restrict__ bw, int M, unsigned mask, int j, int cnt,
+                                               float F[3], float T[3]) {
+  const int lane = threadIdx.x & 31, sub = lane & 7, grp = lane >> 3;
+  while (mask) {
+    int src[4];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) load_record(row + (k + t) * kSlot, b[t]);
+    for (int q = 0; q < 4; ++q) {
+      src[q] = mask ? __ffs(mask) - 1 : -1;
+      mask &= mask - 1u;
+    }
+    const int mine = grp == 0 ? src[0] : (grp == 1 ? src[1] : (grp == 2 ? src[2] : src[3]));
+    const int jj = __shfl_sync(0xffffffffu, j, mine & 31), c0 = __shfl_sync(0xffffffffu, cnt, mine & 31);
+    const int cc = mine < 0 ? 0 : c0;
+    const Rec8* row = reinterpret_cast<const Rec8*>(bw + (int64_t)jj * M * kSlot);
+    int e[6] = {0, 0, 0, 0, 0, 0};   // largest exponent bits, in place
+    for (int k = sub; k < cc; k += 8) {
+      const Rec8 b = load_rec(row + k);
 #pragma unroll
-    for (int t = 0; t < 4; ++t)
-#pragma unroll
-      for (int c = 0; c < 6; ++c) {
-        const int ev = (__float_as_int(b[t][c]) >> 23) & 0xff;
-        e[c] = max(e[c], ev);
-        bad |= ev == 0xff;
-      }
-  }
-  for (; k < cc; ++k) {
-    float b[8];
-    load_record(row + k * kSlot, b);
+      for (int c = 0; c < 6; ++c) e[c] = max(e[c], __float_as_int(b.v[c]) & 0x7f800000);
+    }
+    bool bad = false;
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
-      const int ev = (__float_as_int(b[c]) >> 23) & 0xff;
-      e[c] = max(e[c], ev);
-      bad |= ev == 0xff;
+#pragma unroll
+      for (int d = 4; d > 0; d >>= 1) e[c] = max(e[c], __shfl_xor_sync(0xffffffffu, e[c], d));
+      e[c] >>= 23;
+      bad |= e[c] == 0xff;
+    }
+    const int bits = 62 - (32 - __clz(cc));
+    long long acc[6] = {0, 0, 0, 0, 0, 0};
+    for (int k = sub; k < cc; k += 8) {
+      const Rec8 b = load_rec(row + k);
+#pragma unroll
+      for (int c = 0; c < 6; ++c) acc[c] += fx_of(b.v[c], e[c], bits);
+    }
+    // each row's total to its own lane
+    const int from = lane == src[1] ? 8 : (lane == src[2] ? 16 : (lane == src[3] ? 24 : 0));
+    const bool take = lane == src[0] || lane == src[1] || lane == src[2] || lane == src[3];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+#pragma unroll
+      for (int d = 4; d > 0; d >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], d);
+      float t = bad ? __int_as_float(0x7fc00000) : fx_float(acc[c], e[c] - 126 - bits);
+      t = __shfl_sync(0xffffffffu, t, from);
+      if (take) {
+        if (c < 3) F[c] += t;
+        else T[c - 3] += t;
+      }
     }
   }
-  const int bits = 62 - (32 - __clz(cc));
-  long long acc[6] = {0, 0, 0, 0, 0, 0};
-  k = 0;
-  for (; k + 4 <= cc; k += 4) {
-    float b[4][8];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) load_record(row + (k + t) * kSlot, b[t]);
-#pragma unroll
-    for (int t = 0; t < 4; ++t)
-#pragma unroll
-      for (int c = 0; c < 6; ++c) acc[c] += fx_of(b[t][c], e[c], bits);
-  }
-  for (; k < cc; ++k) {
-    float b[8];
-    load_record(row + k * kSlot, b);
-#pragma unroll
-    for (int c = 0; c < 6; ++c) acc[c] += fx_of(b[c], e[c], bits);
-  }
-#pragma unroll
-  for (int c = 0; c < 6; ++c)
-    tot[c] = bad ? __int_as_float(0x7fc00000) : (float)ldexp((double)acc[c], e[c] - 126 - bits);
 }
 
 // A row of more than 8 records, summed by the whole warp: each record's rank
@@ -1101,19 +1113,10 @@ __device__ __forceinline__ bool gather_one(const Geo& g, const InstGeo* __restri
     cls = __ldg(s.cls + j);
   }
   cnt = cnt < g.M ? cnt : g.M;
-  if (cnt <= 8) {
-    sum_records<R>(bw + (int64_t)j * g.M * kSlot, cnt, F, T);
-  } else if constexpr (MIXED) {
-    if (cnt > kRankedMax) {
-      // long FP32 rows: each thread its own, in fixed point
-      float tot[6];
-      row_sum_fixed(bw + (int64_t)j * g.M * kSlot, cnt, tot);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        F[c] += tot[c];
-        T[c] += tot[3 + c];
-      }
-    }
+  if (cnt <= 8) sum_records<R>(bw + (int64_t)j * g.M * kSlot, cnt, F, T);
+  if constexpr (MIXED) {
+    const unsigned lng = __ballot_sync(0xffffffffu, cnt > kRankedMax);
+    if (lng) group_sum_rows(bw, g.M, lng, j, cnt, F, T);
   }
   {
     // rows of 9..kRankedMax FP32 records, and every longer FP64 row: the
@@ -1257,12 +1260,13 @@ k_gather(Geo g, const InstGeo* __restrict__ ig, StateBuf s, const void* __restri
   // means this step is void: touch no state, since the buffer this step
   // would write can be the committed one.  Every block still reaches the
   // counter below.
-  __shared__ int s_err0;
-  __shared__ int s_slot[kThreads / 32][kHeavyWin];
-  if (threadIdx.x == 0) s_err0 = dev_err(st);
-  __syncthreads();
+  __shared__ int s_slot[kThreads / 32][MIXED ? 32 : kHeavyWin];
+  // (the stress blocks meet at barriers and decide together; elsewhere a warp
+  // for itself)
+  bool err0 = dev_err(st) != 0;
+  if (blockIdx.x < (unsigned)g.K) err0 = __syncthreads_or(err0) != 0;
   bool fence = false;
-  if (!s_err0) {
+  if (!err0) {
     if constexpr (NEXT) reset_scans(so);
     if (NEXT && blockIdx.x == gridDim.x - 1) {
       set_step_geo(g, ig, st, 2, so.sg);
