@@ -48,7 +48,7 @@ void free_buffers(dss_handle* h) {
   h->pred = nullptr;
   dfree(h->xc); dfree(h->mark);
   h->xc = nullptr; h->mark = nullptr; h->marked = false;
-  dfree(h->cell_count); dfree(h->cell_ids); h->cell_ids = nullptr; dfree(h->cell_start); dfree(h->tmp); dfree(h->spart);
+  dfree(h->cell_count); dfree(h->tile_count); h->tile_count = nullptr; dfree(h->cell_ids); h->cell_ids = nullptr; dfree(h->cell_start); dfree(h->tmp); dfree(h->spart);
   dfree(h->own); dfree(h->bw_count); dfree(h->bw_rec); dfree(h->carry); dfree(h->own_s);
   h->own = nullptr; h->bw_count = nullptr; h->bw_rec = nullptr; h->carry = nullptr; h->own_s = nullptr;
   h->pb_blocks = 0;
@@ -172,7 +172,7 @@ int alloc_buffers(dss_handle* h) {
   if ((r = dalloc(h, &h->posf, n)) || (r = dalloc(h, &h->cellid, n)) || (r = dalloc(h, &h->perm, n)) ||
       (r = dalloc(h, &h->pred, 6 * n)) || (r = dalloc(h, &h->xc, n)) ||
       (r = dalloc(h, &h->key, n)) || (r = dalloc(h, &h->offs, n)) ||
-      (r = dalloc(h, &h->cell_count, (size_t)h->g.ncell)) ||
+      (r = dalloc(h, &h->cell_count, (size_t)h->g.ncell)) || (r = dalloc(h, &h->tile_count, (size_t)kTileCopies * kScanTiles)) ||
       (r = dalloc(h, &h->cell_start, (size_t)h->g.ncell + 1)) || (r = dalloc(h, &h->tmp, n)) ||
       (r = dalloc(h, &h->io3, 3 * n)) || (r = dalloc(h, &h->io3b, 3 * n)) ||
       (r = dalloc(h, &h->stage, 15 * n)) ||
@@ -206,6 +206,7 @@ int alloc_buffers(dss_handle* h) {
       (r = dalloc(h, &h->scan_ticket, 2)))
     return r;
   CK(cudaMemsetAsync(h->cell_count, 0, sizeof(int) * h->g.ncell, h->stream));
+  CK(cudaMemsetAsync(h->tile_count, 0, sizeof(int) * kTileCopies * kScanTiles, h->stream));
   {
     // rows of ids: four times the average cell and twelve more (random
     // packings stay within), shorter on grids of mostly empty cells
@@ -264,7 +265,10 @@ int sync_status(dss_handle* h) {
 
 int clear_err(dss_handle* h) {
   // (a step that failed in its corrector may have begun the next histogram)
-  if (h->sized) CK(cudaMemsetAsync(h->cell_count, 0, sizeof(int) * h->g.ncell, h->stream));
+  if (h->sized) {
+    CK(cudaMemsetAsync(h->cell_count, 0, sizeof(int) * h->g.ncell, h->stream));
+    CK(cudaMemsetAsync(h->tile_count, 0, sizeof(int) * kTileCopies * kScanTiles, h->stream));
+  }
   CK(cudaMemsetAsync(&h->status->w[ST_ERR], 0, sizeof(int), h->stream));
   return DSS_OK;
 }

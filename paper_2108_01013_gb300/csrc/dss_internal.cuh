@@ -14,6 +14,12 @@
 #define DSS_PROF_KERNELS 7
 #define DSS_GRAPHS 4
 
+// Bins a block of the cell scan takes, and the most blocks whose totals the
+// histogram keeps itself.
+constexpr int kScanTile = 2048;
+constexpr int kScanTiles = 128;
+constexpr int kTileCopies = 8;
+
 // Device status word layout (int32 slots in DevStatus::w).
 enum {
   ST_ERR = 0,        // first error code seen (0 = none); later kernels early-exit
@@ -690,6 +696,7 @@ struct dss_handle {
   int* key;          // n
   int* offs;         // n
   int* cell_count;   // ncell
+  int* tile_count;   // kTileCopies x kScanTiles: counts of kScanTile bins each (grids of up to kScanTiles of them)
   int* cell_ids;     // ncell rows of cell_cap ids (a multiple of four)
   int cell_cap;
   int* cell_start;   // ncell+1
@@ -766,7 +773,6 @@ void launch_clusters(dss_handle* h, int* parent, int* minid, int* count, int* la
 void launch_phi_profile(dss_handle* h, int nbins, double a_split, const double* unit, unsigned long long* acc);
 int pair_grid_blocks(const dss_handle* h);
 int pair_pb_blocks(const dss_handle* h);
-void launch_scan(dss_handle* h, const int* in, int* out, int count, int which, bool zero_in);
 int scan_tiles_for(int count);
 int64_t enum_plan(dss_handle* h, std::vector<int>* blk_inst);
 double echem_range(const dss_params* p);

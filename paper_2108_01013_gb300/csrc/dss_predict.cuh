@@ -9,7 +9,8 @@
 // What the sort's first kernel writes.
 struct SortOut {
   int* key;                 // cell of each particle (source order)
-  int* cell_count;          // histogram of the keys (cleared by the scan)
+  int* cell_count;          // histogram of the keys (cleared behind the scan)
+  int* tile_count;          // its sums over the scan's tiles (null: too many)
   int* cell_ids;            // per cell a row of bcap ids
   int bcap;
   double* pred;             // 6n: predicted position and velocity
@@ -21,8 +22,17 @@ struct SortOut {
 };
 
 inline SortOut sort_out(const dss_handle* h) {
-  return SortOut{h->key,  h->cell_count, h->cell_ids,    h->cell_cap,           h->pred,
-                 h->xc,   h->scan_status, h->scan_ticket, 2 * h->scan_tiles_max, h->sg};
+  return SortOut{h->key,
+                 h->cell_count,
+                 scan_tiles_for(h->g.ncell) <= kScanTiles ? h->tile_count : nullptr,
+                 h->cell_ids,
+                 h->cell_cap,
+                 h->pred,
+                 h->xc,
+                 h->scan_status,
+                 h->scan_ticket,
+                 2 * h->scan_tiles_max,
+                 h->sg};
 }
 
 // Predictor of Eq. 15a-b and the wrap of Eq. 16 for one particle; computed
@@ -142,6 +152,19 @@ __device__ __forceinline__ void key_insert(const SortOut& q, int i, int k, int i
   const int rank = __popc(peers & ((1u << lane) - 1u));
   int base = 0;
   if (lane == leader) base = atomicAdd(&q.cell_count[k], __popc(peers));
+  if (q.tile_count) {
+    // mostly one tile a warp: neighbours in memory are neighbours in space, and
+    // for that the sums are kept in copies (one copy: 1M 32 -> 47 us)
+    const int t = k / kScanTile;
+    int one;
+    int* const tc = q.tile_count + (blockIdx.x % kTileCopies) * kScanTiles;
+    __match_all_sync(act, t, &one);
+    if (one) {
+      if (lane == __ffs(act) - 1) atomicAdd(&tc[t], __popc(act));
+    } else if (lane == leader) {
+      atomicAdd(&tc[t], __popc(peers));
+    }
+  }
   base = __shfl_sync(peers, base, leader) + rank;
   q.key[i] = k;
   if (base < q.bcap) q.cell_ids[(int64_t)k * q.bcap + base] = id;

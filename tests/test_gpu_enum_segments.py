@@ -165,3 +165,27 @@ def test_runs_of_steps_as_single_steps(env, precision, ext):
         np.testing.assert_array_equal(out[0][0][k], out[1][0][k])
     for a, b in zip(out[0][1:], out[1][1:]):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("cells", [(16, 16, 8), (17, 11, 11), (12, 13, 13), (64, 64, 63), (64, 64, 64), (65, 64, 64)])
+def test_cell_scan_at_tile_edges(env, cells):
+    """Grids of one scan tile of 2048 cells exactly, a little more and less, of
+    128 tiles (the most whose sums the histogram keeps) and of one row more:
+    every search, also one behind another, finds the brute force's pairs."""
+    rng = np.random.default_rng(sum(cells))
+    box = 3.0 * np.array(cells, dtype=np.float64)
+    x = rng.uniform(0.0, 1.0, size=(3, 1500)) * box[:, None]
+    d = rng.normal(size=(3, 1500))
+    x = np.concatenate([x, (x + 2.03 * d / np.linalg.norm(d, axis=0)) % box[:, None]], axis=1)
+    n = x.shape[1]
+    g = dict(x=x, a=np.ones(n), box=box, ids=rng.permutation(n).astype(np.int32))
+    p = env["dss"].default_params(box, cell_size=3.0 * (1.0 - 1e-12), capacity_M=64, shear_rate=1.0, dt=1e-6)
+    z = np.zeros_like(x)
+    s = env["dss"].Suspension(x, g["a"], box, p, ids=g["ids"], alpha_lin=z, alpha_ang=z, nstep=7)
+    assert s.counters()["ncell"] == cells
+    want = _want(env, g, 7, shear_rate=1.0, dt=1e-6)
+    assert want.shape[0] > 1000
+    for _ in range(3):
+        s.neighbour_build()
+        np.testing.assert_array_equal(s.pairs(), want)
+    s.close()
