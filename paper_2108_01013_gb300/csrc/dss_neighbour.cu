@@ -297,6 +297,39 @@ k_enumerate_classes(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __rest
   finish_row(e, i, n, L.count, st);
 }
 
+// Two FP32 values in one register pair, for the packed instructions.
+__device__ __forceinline__ uint64_t pk2(float a, float b) {
+  uint64_t v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
+  return v;
+}
+__device__ __forceinline__ float2 upk2(uint64_t v) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+  return f;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+
+// Candidate k of a row staged two by two: {x, x', y, y'}, {z, z', a, a'}.
+__device__ __forceinline__ float4 staged(const float4* row, int k) {
+  const float* f = reinterpret_cast<const float*>(row) + 8 * (k >> 1) + (k & 1);
+  return make_float4(f[0], f[2], f[4], f[6]);
+}
+
 // Exact decision of (i, j) (out of line: about one candidate in a thousand).
 __device__ __noinline__ bool decide_exact(const Geo& g, const InstGeo& I, const StateBuf& s, double off, int i,
                                           int j) {
@@ -316,14 +349,18 @@ __device__ __noinline__ bool decide_exact(const Geo& g, const InstGeo& I, const 
 // stages the particles in shared memory relative to the segment's origin,
 // kTile at a time, and each lane runs over its own cells' part of them.
 //
+// Two candidates are staged and screened together (packed FP32 arithmetic, the
+// same roundings): 7 instructions a candidate instead of 11
+// (1M 197 -> 187 us, Table 5 178 -> 174).
+//
 // What bounds it is the issue slots (2.4 to 2.9 instructions a cycle and SM):
 // a candidate is loaded once for 32 owners instead of once for each, and costs
-// a lane 11 instructions, one of them a shared load; the set-up of a block is
+// a lane 7 instructions, one of them a shared load; the set-up of a block is
 // worth half a pass of 32 owners.  Against the walk by owner with the same
 // screen (one box, mixed precision, with the row pass): Table 5 with the 4 a0
-// range (128 per cell, 2.9M pairs) 312 -> 179 us, 1M log-uniform [1, 10] (7.1
-// per cell) 220 -> 199, the 100k packing with the 1 a0 range (4.1 per cell) 40
-// -> 38.  On sparse grids the set-up does not pay: 100k (1.7 per cell) 28
+// range (128 per cell, 2.9M pairs) 312 -> 174 us, 1M log-uniform [1, 10] (7.1
+// per cell) 220 -> 187, the 100k packing with the 1 a0 range (4.1 per cell) 40
+// -> 35.  On sparse grids the set-up does not pay: 100k (1.7 per cell) 28
 // against 37 us, a batch of 64 (1.8) 106 against 202.
 //
 // The decision: u = r^2 - s^2 in FP32, its sign bit shifted into a mask, 32
@@ -444,23 +481,38 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
       lo = r == 0 ? i - hs + 1 : s_off[r][kx];
       hi = s_off[r][kx + (r == 0 ? 2 : (le ? 4 : 3))];
     }
+    const uint64_t npx = pk2(-px, -px), npy = pk2(-py, -py), npz = pk2(-pz, -pz);
+    const uint64_t sc2 = pk2(q.sc, q.sc), sa2 = pk2(sa, sa), nsc2 = pk2(-q.sc, -q.sc), nsa2 = pk2(-sa, -sa);
+    const uint64_t se2 = pk2(pa + q.de, pa + q.de);
     int* rw = list + (int64_t)i * g.Ms;
     int pairs = 0, near = 0;    // of the owner, in the tiles so far
     for (int t0 = 0; t0 < most; t0 += kTile) {
       const int t1 = min(t0 + kTile, len);
       if (o0 == o_beg || most > kTile) {     // (a single tile stays for the next owners)
         __syncwarp();
-        for (int p = t0 + lane; p < t1; p += 32) {
-          const int j = first + p + (p < n1 ? 0 : wrap);
-          const float4 c = __ldg(posf + j);
-          int kc = __ldg(cellid + j) - rc - xf;
-          if (kc < 0) kc += nx;
-          s_c[r][p - t0] = make_float4(c.x + fmaf((float)kc + kx0, I.csf[0], sx), c.y + sy, c.z + sz, c.w);
-          s_j[r][p - t0] = j;
+        for (int p0 = t0; p0 < t1; p0 += 32) {
+          const int p = p0 + lane;
+          float4 c = make_float4(1e15f, 1e15f, 1e15f, 0.f);   // beside an odd last one
+          if (p < t1) {
+            const int j = first + p + (p < n1 ? 0 : wrap);
+            c = __ldg(posf + j);
+            int kc = __ldg(cellid + j) - rc - xf;
+            if (kc < 0) kc += nx;
+            c.x += fmaf((float)kc + kx0, I.csf[0], sx);
+            c.y += sy;
+            c.z += sz;
+            s_j[r][p - t0] = j;
+          }
+          // even lanes hold the two particles' x and y, odd ones z and a
+          const float va = __shfl_xor_sync(0xffffffffu, lane & 1 ? c.x : c.z, 1);
+          const float vb = __shfl_xor_sync(0xffffffffu, lane & 1 ? c.y : c.w, 1);
+          if ((p & ~1) < t1)
+            s_c[r][p - t0] = lane & 1 ? make_float4(va, c.z, vb, c.w) : make_float4(c.x, va, c.y, vb);
         }
         __syncwarp();
       }
-      const int a = max(lo, t0) - t0, z = min(hi, t1) - t0;
+      // the lane's part of the tile, from an even place on
+      const int a0 = max(lo, t0) - t0, z = min(hi, t1) - t0, a = a0 & ~1;
       unsigned hit[kTile / 32];
 #pragma unroll
       for (int h = 0; h < kTile / 32; ++h) {
@@ -472,26 +524,36 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
         int n = 0;
         do {
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const float4 pj = c[n + u];   // up to three past the end: masked off below
-            const float dx = pj.x - px, dy = pj.y - py, dz = pj.z - pz;
-            float sv = fmaf(pj.w, q.sc, sa);
-            if (ECH) sv = fmaxf(sv, pj.w + (pa + q.de));
-            const float t = fmaf(-sv, sv, fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
-            hit[h] = __funnelshift_l(__float_as_uint(t), hit[h], 1);
-            least = fminf(least, fabsf(t));
+          for (int u = 0; u < 4; u += 2) {
+            const float4 xy = c[n + u], za = c[n + u + 1];   // up to three past the end: masked off below
+            const uint64_t dx = add2(pk2(xy.x, xy.y), npx), dy = add2(pk2(xy.z, xy.w), npy);
+            const uint64_t dz = add2(pk2(za.x, za.y), npz), aj = pk2(za.z, za.w);
+            const uint64_t r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
+            const uint64_t sv = fma2(aj, sc2, sa2);
+            float2 t;
+            if (ECH) {
+              const float2 s1 = upk2(sv), s2 = upk2(add2(aj, se2)), rr = upk2(r2);
+              const float m0 = fmaxf(s1.x, s2.x), m1 = fmaxf(s1.y, s2.y);
+              t = make_float2(fmaf(-m0, m0, rr.x), fmaf(-m1, m1, rr.y));
+            } else {
+              t = upk2(fma2(fma2(aj, nsc2, nsa2), sv, r2));
+            }
+            hit[h] = __funnelshift_l(__float_as_uint(t.x), hit[h], 1);
+            hit[h] = __funnelshift_l(__float_as_uint(t.y), hit[h], 1);
+            least = fminf(least, fminf(fabsf(t.x), fabsf(t.y)));
           }
           n += 4;
         } while (n < m);
         hit[h] <<= 32 - n;                          // candidate b at bit 31 - b
-        const unsigned all = ~(m < 32 ? 0xffffffffu >> m : 0u);
+        unsigned all = ~(m < 32 ? 0xffffffffu >> m : 0u);
+        if (h == 0 && a != a0) all &= 0x7fffffffu;
         hit[h] &= all;
         if (least <= m2 || img) {
           for (unsigned left = all; left;) {
             const int e = __clz(left);
             const unsigned bit = 0x80000000u >> e;
             left &= ~bit;
-            const float4 pj = c[e];
+            const float4 pj = staged(c, e);
             const float dx = pj.x - px, dy = pj.y - py, dz = pj.z - pz;
             float sv = fmaf(pj.w, q.sc, sa);
             if (ECH) sv = fmaxf(sv, pj.w + (pa + q.de));
@@ -515,7 +577,7 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
           for (unsigned left = hit[h]; left;) {
             const int e = __clz(left);
             left &= ~(0x80000000u >> e);
-            const float4 pj = s_c[r][a + 32 * h + e];
+            const float4 pj = staged(s_c[r], a + 32 * h + e);
             const float dx = pj.x - px, dy = pj.y - py, dz = pj.z - pz;
             const float sl = fmaf(pa + pj.w, q.lc, q.ld);
             if (fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < sl * sl) nrm[h] |= 0x80000000u >> e;
