@@ -394,7 +394,8 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
   __shared__ int4 s_par[kRows];            // rows: bin of their x = 0, x of their first cell, cells, image across y
   __shared__ int s_seg[4];                 // first bin, cells, part, first owner
   if (dev_err(st)) return;
-  const int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
+  int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
+  asm volatile("" : "+r"(lane), "+r"(r));     // kept, not taken anew in every loop
   const int inst = ONE ? 0 : blk_inst[blockIdx.x];
   const InstGeo& I = ONE ? I1 : ig[inst];
   const StepGeo sg = sgk[inst];
@@ -513,11 +514,13 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
       }
       // the lane's part of the tile, from an even place on
       const int a0 = max(lo, t0) - t0, z = min(hi, t1) - t0, a = a0 & ~1;
+      const int words = __reduce_max_sync(0xffffffffu, (z - a + 31) >> 5);
       unsigned hit[kTile / 32];
 #pragma unroll
       for (int h = 0; h < kTile / 32; ++h) {
-        const int m = min(32, z - a - 32 * h);
         hit[h] = 0u;
+        if (h >= words) continue;
+        const int m = min(32, z - a - 32 * h);
         if (m <= 0) continue;
         const float4* __restrict__ c = &s_c[r][a + 32 * h];
         float least = __int_as_float(0x7f800000);
@@ -571,8 +574,9 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
       unsigned nrm[kTile / 32];
 #pragma unroll
       for (int h = 0; h < kTile / 32; ++h) {
-        mine += __popc(hit[h]);
         nrm[h] = 0u;
+        if (h >= words) continue;
+        mine += __popc(hit[h]);
         if (SPLIT) {
           for (unsigned left = hit[h]; left;) {
             const int e = __clz(left);
@@ -597,7 +601,8 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
       // the warp's part of the owner's row
       int kn = SPLIT ? near + (at >> 16) : pairs + at, kf = SPLIT ? pairs - near + (at & 0xffff) - (at >> 16) : 0;
 #pragma unroll
-      for (int h = 0; h < kTile / 32; ++h)
+      for (int h = 0; h < kTile / 32; ++h) {
+        if (h >= words) break;
         for (unsigned left = hit[h]; left;) {
           const int e = __clz(left);
           const unsigned bit = 0x80000000u >> e;
@@ -611,6 +616,7 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
             ++kn;
           }
         }
+      }
       pairs += SPLIT ? tot & 0xffff : tot;
       near += SPLIT ? tot >> 16 : 0;
     }
