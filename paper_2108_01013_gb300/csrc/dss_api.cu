@@ -53,7 +53,7 @@ void free_buffers(dss_handle* h) {
   h->own = nullptr; h->bw_count = nullptr; h->bw_rec = nullptr; h->carry = nullptr; h->own_s = nullptr;
   h->pb_blocks = 0;
   dfree(h->io3); dfree(h->io3b); dfree(h->io_id); dfree(h->stage);
-  h->stage = nullptr; dfree(h->scan_status); dfree(h->scan_ticket);
+  h->stage = nullptr; dfree(h->scan_status); dfree(h->scan_ticket); dfree(h->row_sums);
   dfree(h->sigma);
   dfree(h->sigma_sum);
   dfree(h->a_by_id);
@@ -76,7 +76,7 @@ void free_buffers(dss_handle* h) {
   h->posf = nullptr; h->cellid = nullptr; h->perm = nullptr; h->key = nullptr; h->offs = nullptr;
   h->cell_count = nullptr; h->cell_start = nullptr; h->tmp = nullptr;
   h->spart = nullptr; h->io3 = nullptr; h->io3b = nullptr; h->io_id = nullptr; h->scan_status = nullptr;
-  h->scan_ticket = nullptr;
+  h->scan_ticket = nullptr; h->row_sums = nullptr;
   h->bytes = 0;
   h->sized = false;
 }
@@ -200,10 +200,10 @@ int alloc_buffers(dss_handle* h) {
       h->own_s = own_s;
     }
   }
-  const int tiles = std::max(scan_tiles_for(h->g.ncell), enum_scan_tiles_for((int)n));
-  h->scan_tiles_max = std::max(tiles, 1);
-  if ((r = dalloc(h, &h->scan_status, 2 * (size_t)h->scan_tiles_max)) ||
-      (r = dalloc(h, &h->scan_ticket, 2)))
+  h->scan_tiles_max = std::max(scan_tiles_for(h->g.ncell), 1);
+  row_sum_words((int)n, h->row_tiles, h->row_words);
+  if ((r = dalloc(h, &h->scan_status, (size_t)h->scan_tiles_max)) || (r = dalloc(h, &h->scan_ticket, 1)) ||
+      (r = dalloc(h, &h->row_sums, (size_t)h->row_words)))
     return r;
   CK(cudaMemsetAsync(h->cell_count, 0, sizeof(int) * h->g.ncell, h->stream));
   CK(cudaMemsetAsync(h->tile_count, 0, sizeof(int) * kTileCopies * kScanTiles, h->stream));
@@ -539,9 +539,7 @@ int ensure_pair_capacity(dss_handle* h, int list) {
   CK(cudaStreamSynchronize(h->stream));
   if (P > h->pcap) {
     if ((r = alloc_pair_buffers(h, (int64_t)(P * 1.25) + 1024, true))) return r;
-    CK(cudaMemsetAsync(h->scan_status + h->scan_tiles_max, 0, sizeof(unsigned long long) * h->scan_tiles_max,
-                       h->stream));
-    CK(cudaMemsetAsync(h->scan_ticket + 1, 0, sizeof(int), h->stream));
+    CK(cudaMemsetAsync(h->row_sums, 0, sizeof(int) * h->row_words, h->stream));
     CK(cudaMemsetAsync(&h->status->w[ST_BAND], 0, sizeof(int), h->stream));
     launch_enumerate(h, h->cur, list, 0);
     CK(cudaGetLastError());

@@ -724,8 +724,10 @@ struct dss_handle {
   unsigned char* cls_map;   // n: size class of each id
   unsigned int* done_blocks;  // last-block counter of the gather (reset by that block)
   // scans
-  unsigned long long* scan_status;  // tile status words (2 scans)
-  int* scan_ticket;                 // 2 tickets
+  unsigned long long* scan_status;  // tile status words of the cell scan
+  int* scan_ticket;
+  int* row_sums;                    // row_words: lengths of the lists over tiles of owners and groups of tiles
+  int row_tiles, row_words;
   int scan_tiles_max;
   // status
   DevStatus* status;
@@ -776,7 +778,7 @@ int pair_pb_blocks(const dss_handle* h);
 int scan_tiles_for(int count);
 int64_t enum_plan(dss_handle* h, std::vector<int>* blk_inst);
 double echem_range(const dss_params* p);
-int enum_scan_tiles_for(int n);
+void row_sum_words(int n, int& tiles, int& words);
 int bw_slot_values();
 // Marks the start of kernel k of a step when profiling (event record node
 // when the step is being captured).

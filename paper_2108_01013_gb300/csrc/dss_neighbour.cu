@@ -30,6 +30,7 @@ constexpr int kRows = 5;           // rows of cells in the half stencil, a warp 
 constexpr int kTile = 128;         // candidates of a row staged at a time
 constexpr int kSegMax = 28;        // cells of a segment (its stencil rows span three more)
 constexpr int kRowThreads = 256;   // row pass
+constexpr int kRowGroup = 16;      // tiles of a group
 
 // Cutoffs of the pair (i, j) in FP32, linear in the radii: s = (a_i + a_j) sc + sd
 // (the listing range) and (a_i + a_j) lc + ld (the lubrication range, row
@@ -128,9 +129,26 @@ __device__ __forceinline__ void scan_range(EnumCtx& e, int jb, int je, float cxo
   for (int j = jb; j < je; ++j) take_candidate<ECH>(e, __ldg(e.posf + j), j, px, py, pz);
 }
 
-// The length of the owner's row, and the exact decisions counted.
-__device__ __forceinline__ void finish_row(const EnumCtx& e, int i, int n, int* __restrict__ count, DevStatus* st) {
+// Sums of the rows' lengths, kept for the row pass: over its tiles of 2^shift
+// owners, and over kRowGroup tiles each.
+struct RowSums {
+  int* tile;
+  int* group;
+  int shift;
+};
+
+__device__ __forceinline__ void add_rows(const RowSums& R, int t, int v) {
+  atomicAdd(&R.tile[t], v);
+  atomicAdd(&R.group[t / kRowGroup], v);
+}
+
+// The length of the owner's row, its warp's sum (a warp lies in one tile), and
+// the exact decisions counted.
+__device__ __forceinline__ void finish_row(const EnumCtx& e, int i, int n, int* __restrict__ count, const RowSums& R,
+                                           DevStatus* st) {
   if (i < n) count[i] = e.cnt;
+  const int sum = __reduce_add_sync(0xffffffffu, i < n ? min(e.cnt, e.M) : 0);
+  if ((threadIdx.x & 31) == 0 && sum) add_rows(R, i >> R.shift, sum);
   const int b = __reduce_add_sync(0xffffffffu, i < n ? e.band : 0);
   if ((threadIdx.x & 31) == 0 && b) atomicAdd(&st->w[ST_BAND], b);
 }
@@ -139,7 +157,7 @@ template <bool ECH>
 __global__ void __launch_bounds__(kThreads, 8)
 k_enumerate(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sgk, StateBuf s,
             const float4* __restrict__ posf, const int* __restrict__ cellid,
-            const int* __restrict__ cell_start, ListBuf L, DevStatus* st, EnumCut q) {
+            const int* __restrict__ cell_start, ListBuf L, RowSums R, DevStatus* st, EnumCut q) {
   dep_wait();
   if (dev_err(st)) return;
   const int i = blockIdx.x * kThreads + threadIdx.x;
@@ -202,7 +220,7 @@ k_enumerate(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ s
       }
     }
   }
-  finish_row(e, i, n, L.count, st);
+  finish_row(e, i, n, L.count, R, st);
 }
 
 // Size classes (Sec. II A: cells smaller than 2 a_max, a larger stencil for
@@ -218,7 +236,7 @@ template <bool ECH>
 __global__ void __launch_bounds__(kThreads, 8)
 k_enumerate_classes(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sgk, StateBuf s,
                     const float4* __restrict__ posf, const int* __restrict__ cellid,
-                    const int* __restrict__ cell_start, ListBuf L, DevStatus* st, EnumCut q) {
+                    const int* __restrict__ cell_start, ListBuf L, RowSums R, DevStatus* st, EnumCut q) {
   dep_wait();
   if (dev_err(st)) return;
   const int i = blockIdx.x * kThreads + threadIdx.x;
@@ -294,7 +312,7 @@ k_enumerate_classes(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __rest
       }
     }
   }
-  finish_row(e, i, n, L.count, st);
+  finish_row(e, i, n, L.count, R, st);
 }
 
 // Two FP32 values in one register pair, for the packed instructions.
@@ -379,12 +397,12 @@ __device__ __noinline__ bool decide_exact(const Geo& g, const InstGeo& I, const 
 // k_rows closes the row up.
 // ------------------------------------------------------------------------
 template <bool ECH, bool SPLIT, bool ONE>
-__global__ void __launch_bounds__(32 * kRows, 6)
+__global__ void __launch_bounds__(32 * kRows, 7)
 k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I1, const InstGeo* __restrict__ ig,
             const StepGeo* __restrict__ sgk, const __grid_constant__ StateBuf s, const float4* __restrict__ posf,
             const int* __restrict__ cellid, const int* __restrict__ cell_start, int* __restrict__ list,
-            int* __restrict__ count, int* __restrict__ nnear, const int* __restrict__ blk_inst, DevStatus* st,
-            EnumCut q) {
+            int* __restrict__ count, int* __restrict__ nnear, const int* __restrict__ blk_inst, RowSums R,
+            DevStatus* st, EnumCut q) {
   dep_wait();
   __shared__ float4 s_c[kRows][kTile + 4];
   __shared__ int s_j[kRows][kTile];
@@ -620,9 +638,17 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
       pairs += SPLIT ? tot & 0xffff : tot;
       near += SPLIT ? tot >> 16 : 0;
     }
-    if (r == 0 && in) {
-      count[i] = pairs;
-      if (SPLIT) nnear[i] = near;
+    if (r == 0) {
+      if (in) {
+        count[i] = pairs;
+        if (SPLIT) nnear[i] = near;
+      }
+      // (owners from o0 on: in one tile or two)
+      const int t = o0 >> R.shift, v = in ? min(pairs, g.M) : 0;
+      const int s0 = __reduce_add_sync(0xffffffffu, i >> R.shift == t ? v : 0);
+      const int s1 = __reduce_add_sync(0xffffffffu, i >> R.shift == t ? 0 : v);
+      if (lane == 0 && s0) add_rows(R, t, s0);
+      if (lane == 0 && s1) add_rows(R, t + 1, s1);
     }
   }
   if (__any_sync(0xffffffffu, band != 0)) {
@@ -631,54 +657,61 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
   }
 }
 
-// Row pass: row lengths, counters, the id <-> row maps, the exclusive scan of
-// the row lengths (decoupled look-back over tiles of TILE owners) and the
-// compact pair arrays (owner and partner of every pair in owner order, the
-// order the pair kernel deals them out in), written by the block together,
-// coalesced; the first pairs are read while the first warp looks back.  SPLIT
-// rows are closed up in place here: the far block [M - far, M) moves down
-// behind the near one, ascending, every entry read before any write reaches
-// it (a source lies beyond its destination by the gap).  A kernel of its own:
-// with the look-back at the end of the search every block held its place
-// until the slowest before it was done (a third of the kernel at 1M).
+// Row pass: counters, the id <-> row maps, the exclusive scan of the row
+// lengths and the compact pair arrays (owner and partner of every pair in owner
+// order, the order the pair kernel deals them out in), written by the block
+// together, coalesced.  A tile's first pair is the sum of the groups and tiles
+// before it, which the search left: no block waits for another (with a
+// look-back over the tiles a step of 20,000 spheres took 38.5 us instead of
+// 36.2, Table 5's 446 instead of 440).  SPLIT rows are closed up in place here:
+// the far block [M - far, M) moves down behind the near one, ascending, every
+// entry read before any write reaches it (a source lies beyond its destination
+// by the gap).  A kernel of its own:
+// a row's place needs all rows before it.
 // TILE: 256 owners, or 64 where rows are long (a block's pairs are what its
 // time goes with).
 template <bool SPLIT, int TILE>
 __global__ void __launch_bounds__(kRowThreads)
 k_rows(int n, int M, int Ms, int64_t pcap, const int* __restrict__ ids, const __grid_constant__ ListBuf L,
-       const int* __restrict__ nnear, int* __restrict__ bw_count, unsigned long long* scan_status, int* scan_ticket,
-       DevStatus* st) {
+       const int* __restrict__ nnear, int* __restrict__ bw_count, RowSums R, DevStatus* st) {
   dep_wait();
-  constexpr int kAhead = 4;                  // pairs a thread reads before the offsets are known
-  __shared__ int s_tile, s_prefix;
-  __shared__ int s_warp[kRowThreads / 32];
+  constexpr int kAhead = 4;                  // pairs a thread has in flight
+  __shared__ int s_warp[kRowThreads / 32], s_pre[kRowThreads / 32];
   __shared__ int s_ex[TILE + 1], s_near[SPLIT ? TILE : 1];
-  // (a block that saw an error takes no ticket: no tile waits for it)
-  if (threadIdx.x == 0) s_tile = dev_err(st) ? -1 : atomicAdd(scan_ticket, 1);
-  __syncthreads();
-  const int tile = s_tile, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (tile < 0) return;
+  const int err = dev_err(st);
+  const int tile = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int i0 = tile * TILE, i = i0 + threadIdx.x;
   const bool own = threadIdx.x < TILE && i < n;
   const int cnt = own ? L.count[i] : 0;
   const int v = min(cnt, M);
   if (SPLIT && own) s_near[threadIdx.x] = min(nnear[i], v);
+  int pre = 0;
+  for (int t = threadIdx.x; t < tile / kRowGroup; t += kRowThreads) pre += R.group[t];
+  if (threadIdx.x < tile % kRowGroup) pre += R.tile[tile - 1 - threadIdx.x];
+  pre = __reduce_add_sync(0xffffffffu, pre);
   int incl = v;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
     const int t = __shfl_up_sync(0xffffffffu, incl, d);
     if (lane >= d) incl += t;
   }
-  if (lane == 31) s_warp[wid] = incl;
-  __syncthreads();
-  int before = 0, total = 0;
+  if (lane == 31) {
+    s_warp[wid] = incl;
+    s_pre[wid] = pre;
+  }
+  if (__syncthreads_or(err)) return;
+  int before = 0, total = 0, base = 0;
 #pragma unroll
   for (int w = 0; w < kRowThreads / 32; ++w) {
     if (w < wid) before += s_warp[w];
     total += s_warp[w];
+    base += s_pre[w];
   }
   if (threadIdx.x < TILE) s_ex[threadIdx.x] = before + incl - v;
-  if (threadIdx.x == 0) s_ex[TILE] = total;
+  if (threadIdx.x == 0) {
+    s_ex[TILE] = total;
+    if (i0 + TILE >= n) L.start[n] = base + total;
+  }
   __syncthreads();
   // pair t of the tile: its owner (the last whose row starts at or before t)
   // and its place there
@@ -705,13 +738,6 @@ k_rows(int n, int M, int Ms, int64_t pcap, const int* __restrict__ ids, const __
       if (src != k) ak[r] = k;
     }
   }
-  if (wid == 0) {
-    const int prefix = lookback_warp(scan_status, tile, total, st);
-    if (lane == 0) {
-      s_prefix = prefix;
-      if (i0 + TILE >= n) L.start[n] = prefix + total;
-    }
-  }
   const int wmax = __reduce_max_sync(0xffffffffu, cnt);
   if (lane == 0 && wmax > *(volatile int*)&st->w[ST_MAXROW]) atomicMax(&st->w[ST_MAXROW], wmax);
   if (own) {
@@ -723,10 +749,9 @@ k_rows(int n, int M, int Ms, int64_t pcap, const int* __restrict__ ids, const __
     const int id = ids[i];
     L.slot_of_id[id] = i;
     L.id_of_slot[i] = id;
+    L.start[i] = base + before + incl - v;
   }
-  __syncthreads();
-  const int base = s_prefix;
-  if (own) L.start[i] = base + before + incl - v;
+  if (SPLIT) __syncthreads();
 #pragma unroll
   for (int r = 0; r < kAhead; ++r) {
     const int t = threadIdx.x + r * kRowThreads;
@@ -757,7 +782,11 @@ k_rows(int n, int M, int Ms, int64_t pcap, const int* __restrict__ ids, const __
 }
 }  // namespace
 
-int enum_scan_tiles_for(int n) { return (n + kThreads - 1) / kThreads * (kThreads / 32); }
+// Tiles of 64 owners (the smaller ones), and with their groups.
+void row_sum_words(int n, int& tiles, int& words) {
+  tiles = (n + 63) / 64;
+  words = tiles + (tiles + kRowGroup - 1) / kRowGroup;
+}
 
 // Expected passes of 32 owners over a segment of mean owners (Poisson counts).
 static double seg_passes(double mean) {
@@ -841,11 +870,13 @@ void launch_enumerate(dss_handle* h, int stbuf, int dst_list, int adv) {
   // first, so that the pair kernel's warps meet runs of pairs without
   // lubrication (short rows gain less than the reordering costs)
   const bool split = g.de > 0.0 && !h->enum_walk && h->n >= 8 * (int64_t)g.ncell;
+  const int tile = split ? 64 : 256;
+  const RowSums R{h->row_sums, h->row_sums + h->row_tiles, split ? 6 : 8};
   const unsigned blocks = (unsigned)h->enum_blocks;
   if (h->enum_walk) {
     auto kw = g.nclass > 1 ? (ech ? k_enumerate_classes<true> : k_enumerate_classes<false>)
                            : (ech ? k_enumerate<true> : k_enumerate<false>);
-    launch_dep(kw, blocks, kThreads, h->stream, g, h->ig, h->sg, h->st[stbuf], h->posf, h->cellid, h->cell_start, L,
+    launch_dep(kw, blocks, kThreads, h->stream, g, h->ig, h->sg, h->st[stbuf], h->posf, h->cellid, h->cell_start, L, R,
                h->status, q);
   } else {
     const bool one = h->K == 1;
@@ -854,11 +885,10 @@ void launch_enumerate(dss_handle* h, int stbuf, int dst_list, int adv) {
                   : (split ? (one ? k_enumerate_seg<false, true, true> : k_enumerate_seg<false, true, false>)
                            : (one ? k_enumerate_seg<false, false, true> : k_enumerate_seg<false, false, false>));
     launch_dep(ks, blocks, 32 * kRows, h->stream, g, h->ig_host[0], h->ig, h->sg, h->st[stbuf], h->posf, h->cellid,
-                                             h->cell_start, L.list, L.count, h->offs, h->enum_inst, h->status, q);
+                                             h->cell_start, L.list, L.count, h->offs, h->enum_inst, R, h->status, q);
   }
-  const int tile = split ? 64 : 256;
   auto kr = split ? k_rows<true, 64> : k_rows<false, 256>;
   launch_dep(kr, ((int)h->n + tile - 1) / tile, kRowThreads, h->stream, (int)h->n, g.M, g.Ms, g.pcap, h->st[stbuf].id, L,
-             h->offs, h->bw_count, h->scan_status + h->scan_tiles_max, h->scan_ticket + 1, h->status);
+             h->offs, h->bw_count, R, h->status);
   h->last_list = dst_list;
 }

@@ -18,6 +18,8 @@ struct SortOut {
   unsigned long long* scan_status;   // the look-back state of the operation's scans
   int* scan_ticket;
   int scan_words;
+  int* row_sums;                     // and the row sums of its search
+  int row_words;
   StepGeo* sg;
 };
 
@@ -31,7 +33,9 @@ inline SortOut sort_out(const dss_handle* h) {
                  h->xc,
                  h->scan_status,
                  h->scan_ticket,
-                 2 * h->scan_tiles_max,
+                 h->scan_tiles_max,
+                 h->row_sums,
+                 h->row_words,
                  h->sg};
 }
 
@@ -199,9 +203,10 @@ __device__ __forceinline__ void set_step_geo(const Geo& g, const InstGeo* __rest
   }
 }
 
-// The look-back state of the operation's scans, by the threads of the grid.
+// The state of the operation's scans, by the threads of the grid.
 __device__ __forceinline__ void reset_scans(const SortOut& q) {
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < q.scan_words; t += gridDim.x * blockDim.x)
     q.scan_status[t] = 0ull;
-  if (blockIdx.x == 0 && threadIdx.x < 2) q.scan_ticket[threadIdx.x] = 0;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < q.row_words; t += gridDim.x * blockDim.x) q.row_sums[t] = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) q.scan_ticket[0] = 0;
 }
