@@ -910,8 +910,8 @@ __device__ __forceinline__ float fx_float(long long acc, int k) {
   return __ll2float_rn(acc) * __int_as_float((h + 127) << 23) * __int_as_float((k - h + 127) << 23);
 }
 
-// The long rows (more than kRankedMax FP32 records) of a warp's particles
-// (mask), four at a time, eight lanes to a row, in 64-bit fixed point.  Per
+// The sum t of a row of cc FP32 records by eight lanes (sub: 0..7; every group
+// of the warp calls it, with cc = 0 for no row) in 64-bit fixed point.  Per
 // component the largest exponent e of the row fixes the unit 2^(e - 126 -
 // bits), bits = 62 - ceil(log2(cc + 1)), so that every record is an integer
 // below 2^bits and the row's sum stays below 2^62 (a first pass finds e, a
@@ -919,11 +919,44 @@ __device__ __forceinline__ float fx_float(long long acc, int k) {
 // function of the set of records alone, whatever their order in the row and
 // the lanes, so no ranking is needed.  It is exact up to the dropped bits below
 // 2^-(bits - 24) of each record relative to the row's largest (more accurate
-// than an FP32 running sum).  A non-finite record makes the total NaN.  j, cnt:
-// the lane's particle and its records; F, T: the lane's sums.
+// than an FP32 running sum).  A non-finite record makes the total NaN.
+template <bool RW>
+__device__ __forceinline__ void fx_row_sum(const Rec8* row, int cc, int sub, float t[6]) {
+  int e[6] = {0, 0, 0, 0, 0, 0};   // largest exponent bits, in place
+  for (int k = sub; k < cc; k += 8) {
+    const Rec8 b = RW ? load_rec_rw(row + k) : load_rec(row + k);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) e[c] = max(e[c], __float_as_int(b.v[c]) & 0x7f800000);
+  }
+  bool bad = false;
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+#pragma unroll
+    for (int d = 4; d > 0; d >>= 1) e[c] = max(e[c], __shfl_xor_sync(0xffffffffu, e[c], d));
+    e[c] >>= 23;
+    bad |= e[c] == 0xff;
+  }
+  const int bits = 62 - (32 - __clz(cc));
+  long long acc[6] = {0, 0, 0, 0, 0, 0};
+  for (int k = sub; k < cc; k += 8) {
+    const Rec8 b = RW ? load_rec_rw(row + k) : load_rec(row + k);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) acc[c] += fx_of(b.v[c], e[c], bits);
+  }
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+#pragma unroll
+    for (int d = 4; d > 0; d >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], d);
+    t[c] = bad ? __int_as_float(0x7fc00000) : fx_float(acc[c], e[c] - 126 - bits);
+  }
+}
+
+// The long rows (more than kRankedMax FP32 records) of a warp's particles
+// (mask), four at a time.  j, cnt: the lane's particle and its records; F, T:
+// the lane's sums.
 // Neighbouring lanes read neighbouring sectors, and a warp's work is the sum of
 // its rows, not 32 times the longest: the corrector of Table 5 (45 records a
-// row, up to 216) 160 us with a thread to a row, 90 so.  On rows of 9 to 24
+// row, up to 216) 160 us with a thread to a row, 86 so.  On rows of 9 to 24
 // records the ranked sum of the whole warp is faster (100k with the 1 a0 range
 // 26 against 36 us).
 __device__ __forceinline__ void group_sum_rows(const float* __restrict__ bw, int M, unsigned mask, int j, int cnt,
@@ -940,36 +973,14 @@ __device__ __forceinline__ void group_sum_rows(const float* __restrict__ bw, int
     const int jj = __shfl_sync(0xffffffffu, j, mine & 31), c0 = __shfl_sync(0xffffffffu, cnt, mine & 31);
     const int cc = mine < 0 ? 0 : c0;
     const Rec8* row = reinterpret_cast<const Rec8*>(bw + (int64_t)jj * M * kSlot);
-    int e[6] = {0, 0, 0, 0, 0, 0};   // largest exponent bits, in place
-    for (int k = sub; k < cc; k += 8) {
-      const Rec8 b = load_rec(row + k);
-#pragma unroll
-      for (int c = 0; c < 6; ++c) e[c] = max(e[c], __float_as_int(b.v[c]) & 0x7f800000);
-    }
-    bool bad = false;
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-#pragma unroll
-      for (int d = 4; d > 0; d >>= 1) e[c] = max(e[c], __shfl_xor_sync(0xffffffffu, e[c], d));
-      e[c] >>= 23;
-      bad |= e[c] == 0xff;
-    }
-    const int bits = 62 - (32 - __clz(cc));
-    long long acc[6] = {0, 0, 0, 0, 0, 0};
-    for (int k = sub; k < cc; k += 8) {
-      const Rec8 b = load_rec(row + k);
-#pragma unroll
-      for (int c = 0; c < 6; ++c) acc[c] += fx_of(b.v[c], e[c], bits);
-    }
+    float tot[6];
+    fx_row_sum<false>(row, cc, sub, tot);
     // each row's total to its own lane
     const int from = lane == src[1] ? 8 : (lane == src[2] ? 16 : (lane == src[3] ? 24 : 0));
     const bool take = lane == src[0] || lane == src[1] || lane == src[2] || lane == src[3];
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
-#pragma unroll
-      for (int d = 4; d > 0; d >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], d);
-      float t = bad ? __int_as_float(0x7fc00000) : fx_float(acc[c], e[c] - 126 - bits);
-      t = __shfl_sync(0xffffffffu, t, from);
+      const float t = __shfl_sync(0xffffffffu, tot[c], from);
       if (take) {
         if (c < 3) F[c] += t;
         else T[c - 3] += t;
@@ -1304,6 +1315,31 @@ k_gather(Geo g, const InstGeo* __restrict__ ig, StateBuf s, const void* __restri
   }
 }
 
+// Crowded grids, where most rows are long: every row of more than 8 records
+// becomes one record, its sum, ahead of the corrector, which holds a thread a
+// particle and too few warps to hide the rows' loads.  Eight lanes a row, as in
+// group_sum_rows.  A step of Table 5 (45 records a row, up to 216) 440 -> 415
+// us, 12,000 spheres of it 629 -> 594, the attraction of Table 4 (35 a row)
+// 244 -> 228 with 60,000 spheres and 103 -> 76 with 6000.  Bound by the records'
+// way from L2 and the conversions.
+__global__ void __launch_bounds__(256, 5)
+k_long_rows(int n, int M, float* bw, int* bw_count, const DevStatus* st) {
+  dep_wait();
+  if (dev_err(st)) return;
+  const int t = blockIdx.x * 256 + threadIdx.x, j = t >> 3, sub = t & 7;
+  int cc = j < n ? min(bw_count[j], M) : 0;
+  if (cc <= 8) cc = 0;
+  if (!__any_sync(0xffffffffu, cc)) return;
+  Rec8* row = reinterpret_cast<Rec8*>(bw + (int64_t)(cc ? j : 0) * M * kSlot);
+  Rec8 sum;
+  fx_row_sum<true>(row, cc, sub, sum.v);
+  sum.v[6] = sum.v[7] = 0.f;
+  if (cc && sub == 0) {
+    store_rec(row, sum);
+    bw_count[j] = 1;
+  }
+}
+
 // Pairs of a list as (lo id, hi id) in owner order (for dss_get_pairs).
 __global__ void k_pairs_out(Geo g, ListBuf W, long long* __restrict__ out) {
   const int n = g.n;
@@ -1381,6 +1417,10 @@ void launch_forces_t(dss_handle* h, int stbuf, int work_list, int hist_list, int
       launch_dep(k_owner_stress<false, EXT>, h->g.K * kOsParts, kPairThreads, h->stream,
           h->g, h->ig, h->st[stbuf], own_s, carry, h->lb[work_list].start, h->spart, h->status);
   }
+  // (at 4.1 to 4.9 a cell, rows of 6, the pass costs more than it saves: 101 ->
+  // 114 us; at 5.6 even, at 7.5 125 -> 116, smaller systems gain sooner)
+  if (mixed && h->g.de > 0.0 && !h->enum_walk && h->n >= 6 * (int64_t)h->g.ncell)
+    launch_dep(k_long_rows, (n + 31) / 32, 256, h->stream, n, h->g.M, (float*)h->bw_rec, h->bw_count, h->status);
   auto kg = mixed ? (next ? k_gather<true, EXT, true> : k_gather<true, EXT, false>)
                   : (next ? k_gather<false, EXT, true> : k_gather<false, EXT, false>);
   launch_dep(kg, gb + (next ? 1 : 0), kThreads, h->stream, h->g, h->ig, h->st[stbuf], h->own, h->bw_count, h->bw_rec,

@@ -189,3 +189,28 @@ def test_cell_scan_at_tile_edges(env, cells):
         s.neighbour_build()
         np.testing.assert_array_equal(s.pairs(), want)
     s.close()
+
+
+@pytest.mark.parametrize("n,lam,cells", [(4000, 0.05, 5), (4000, 0.15, 4), (700, 0.05, 4)])
+def test_long_rows_summed_ahead_of_the_corrector(env, n, lam, cells):
+    """Forces of rows of 9 to some 100 records on a crowded grid (every such row
+    becomes its sum first) as with lists by size class (rows summed in the
+    corrector).  Both orders of at most 300 pair terms in FP32: they differ by
+    less than 300 roundings of 2^-23 of the packing's largest force."""
+    g = env["synth"].small(n, 0.50, 78)
+    kw = dict(shear_rate=1.0, precision="mixed", f_er=10.0, lambda_d=lam, delta_lub=0.1)
+    s = _handle(env, g, cells, 31, **kw)
+    assert n >= 6 * cells ** 3
+    p = env["dss"].default_params(g["box"], cell_mode=1, **kw)
+    z = np.zeros_like(g["x"])
+    c = env["dss"].Suspension(g["x"], g["a"], g["box"], p, ids=g["ids"], nstep=31, alpha_lin=z, alpha_ang=z)
+    out = []
+    for h in (s, c):
+        F, T = h.forces()
+        out.append((F.cpu().numpy(), T.cpu().numpy(), h.pairs()))
+    np.testing.assert_array_equal(out[0][2], out[1][2])
+    assert np.bincount(out[0][2].reshape(-1)).max() > 9
+    for a, b in zip(out[0][:2], out[1][:2]):
+        assert np.abs(a - b).max() <= 300 * 2.0 ** -23 * np.abs(b).max()
+    s.close()
+    c.close()
