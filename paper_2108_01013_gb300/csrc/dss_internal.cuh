@@ -532,6 +532,16 @@ __device__ __forceinline__ Rec8 load_rec(const Rec8* p) {
       : "l"(p));
   return r;
 }
+// The same of memory that the kernel writes.
+__device__ __forceinline__ Rec8 load_rec_rw(const Rec8* p) {
+  Rec8 r;
+  asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3]), "=f"(r.v[4]), "=f"(r.v[5]), "=f"(r.v[6]),
+                 "=f"(r.v[7])
+               : "l"(p)
+               : "memory");
+  return r;
+}
 __device__ __forceinline__ void store_rec(Rec8* p, const Rec8& r) {
   asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(r.v[0]), "f"(r.v[1]),
                "f"(r.v[2]), "f"(r.v[3]), "f"(r.v[4]), "f"(r.v[5]), "f"(r.v[6]), "f"(r.v[7])
@@ -749,6 +759,7 @@ struct dss_handle {
   int tune_enum_unr;
   // the enumeration's launch (enum_plan)
   bool enum_walk;
+  bool enum_narrow;          // boxes where the staged search meets separations past exact_beyond
   int64_t enum_blocks;
   int* enum_inst;            // instance of each of its blocks (batched instances; else null)
   int64_t enum_inst_cap;

@@ -214,3 +214,27 @@ def test_long_rows_summed_ahead_of_the_corrector(env, n, lam, cells):
         assert np.abs(a - b).max() <= 300 * 2.0 ** -23 * np.abs(b).max()
     s.close()
     c.close()
+
+
+@pytest.mark.parametrize("cells", [(4, 3, 3), (4, 4, 3), (5, 3, 4), (6, 5, 3), (4, 5, 6)])
+@pytest.mark.parametrize("nstep", [0, 250, 999, 54321])
+def test_narrow_boxes_pair_by_the_nearest_image(env, cells, nstep):
+    """Boxes of three to six cells, where the stencil meets separations beyond
+    half the box: the pairs of the nearest images, as the brute force has them.
+    Random centres, half of them on multiples of half a cell."""
+    rng = np.random.default_rng(sum(cells) + nstep)
+    edge = 2.9
+    box = edge * np.array(cells, dtype=np.float64)
+    n = 12 * int(np.prod(cells))
+    x = rng.uniform(0.0, 1.0, size=(3, n)) * box[:, None]
+    x[:, ::2] = np.round(x[:, ::2] / (0.5 * edge)) * (0.5 * edge) % box[:, None]
+    x[:, ::2] += rng.uniform(0.0, 1e-3, size=x[:, ::2].shape)
+    g = dict(x=x, a=rng.choice([1.0, 1.4], size=n), box=box, ids=rng.permutation(n).astype(np.int32))
+    kw = dict(shear_rate=1.3, dt=1e-3)
+    p = env["dss"].default_params(box, cell_size=edge * (1.0 - 1e-12), capacity_M=400, **kw)
+    z = np.zeros_like(x)
+    s = env["dss"].Suspension(x, g["a"], box, p, ids=g["ids"], nstep=nstep, alpha_lin=z, alpha_ang=z)
+    assert s.counters()["ncell"] == cells
+    s.neighbour_build()
+    np.testing.assert_array_equal(s.pairs(), _want(env, g, nstep, **kw))
+    s.close()
