@@ -812,9 +812,10 @@ static double seg_passes(double mean) {
 // The enumeration's kernel and launch for the current grid.  Grids of fewer
 // than four particles a cell, and of size classes, are walked by owner (the
 // two searches meet between 1.8 and 4.1 per cell, see k_enumerate_seg), except
-// single systems of up to 200 owners per SM: there the walk's chain of loads
+// single systems of up to 360 owners per SM: there the walk's chain of loads
 // is all that counts and five warps per segment shorten it (1,000 owners 19
-// -> 15 us, 20,000 22 -> 20; 50,000 24 both, 100,000 28 -> 33).
+// -> 13 us, 20,000 22 -> 16; a step of 40,000 45.7 -> 43.0, of 50,000 50.2 ->
+// 48.4, of 65,000 57.9 -> 58.0, of 100,000 71.7 -> 76.1).
 // Segments are cut so that the cost per owner is smallest: a block's set-up is
 // worth about half a pass of 32 owners.  Cells of more than 26 particles are
 // shared by as many blocks as hold their average and a quarter more.  Per
@@ -822,7 +823,7 @@ static double seg_passes(double mean) {
 // a segment, the first block.  Returns the number of blocks (and their
 // instances, when asked for).
 int64_t enum_plan(dss_handle* h, std::vector<int>* blk_inst) {
-  const bool sparse = h->n < 4 * (int64_t)h->g.ncell && (h->K > 1 || h->n > 200 * (int64_t)h->sms);
+  const bool sparse = h->n < 4 * (int64_t)h->g.ncell && (h->K > 1 || h->n > 360 * (int64_t)h->sms);
   const bool empty = h->n * 4 < (int64_t)h->g.ncell;   // most segments would hold nobody
   h->enum_walk = h->g.nclass > 1 || h->tune_enum_unr == 1 || (h->tune_enum_unr == 0 && (sparse || empty));
   int64_t blk = 0;
