@@ -1250,7 +1250,8 @@ __device__ __forceinline__ bool gather_one(const Geo& g, const InstGeo* __restri
 // Blocks 0..K-1 reduce the bulk stress of instance k (scheduled first, off
 // the particles' critical path); the blocks after them take one particle per
 // thread.  At most 80 registers, so that six blocks fit on an SM and a
-// 100k-particle grid runs in one wave.  The last block to finish commits the step; only the writes that
+// 100k-particle grid runs in one wave; eight blocks of 64 where the kernel is bound
+// by its loads' latency at half the memory's rate (1M 85.8 -> 80.3 us).  The last block to finish commits the step; only the writes that
 // block reads (the stresses, an error code) are fenced before the count.
 // NEXT (inside a run of steps): the first part of the next step rides along
 // (dss_predict.cuh), so that a run reads the state once where two kernels did
@@ -1258,7 +1259,7 @@ __device__ __forceinline__ bool gather_one(const Geo& g, const InstGeo* __restri
 // systems whose kernels are bound by latency (see chain_steps): 1,000 spheres
 // in FP64 54.8 -> 51.5 us a step, 20,000 43.9 -> 39.6, 100,000 76.6 -> 73.5.
 template <bool MIXED, bool EXT, bool NEXT>
-__global__ void __launch_bounds__(kThreads, 6)
+__global__ void __launch_bounds__(kThreads, MIXED && !NEXT ? 8 : 6)
 k_gather(Geo g, const InstGeo* __restrict__ ig, StateBuf s, const void* __restrict__ own_v,
          const int* __restrict__ bw_count, const void* __restrict__ bw_v, double* __restrict__ Fout,
          double* __restrict__ Tout, DevStatus* st, int mode, const double* __restrict__ spart,
