@@ -316,14 +316,14 @@ int dss_load(dss_handle *h, const void *buf, size_t len);
 int dss_autotune(dss_handle *h, int32_t trial_steps, int32_t ncand, const double *factors,
                  double *ms_per_step, double *cell_size);
 
-/* Kernel shapes (the tile parameters of the step; north star: "tile shape
- * picked by an autotuner"), timed at the current cell grid: the register
+/* Kernel shapes (the tile parameters of the step), timed at the current cell
+ * grid: the register
  * budget of the pair kernel (cut for 3 or 4 resident 256-thread blocks per
  * SM: 80 or 64 registers; more warps in flight against more spills) and the
  * enumeration's search (a thread walking each owner's stencil, or a block
- * staging the candidates of a few cells for their owners).  Each of the 4 combinations runs 2 + trial_steps
- * steps from a checkpoint of the current state; the fastest is kept and the
- * state restored.  ms_per_step (host, 4 doubles, may be NULL): ms per step of
+ * staging the candidates of a few cells for their owners).  Each of the 4
+ * combinations runs 2 + trial_steps steps from a checkpoint of the current
+ * state; the fastest is kept and the state restored.  ms_per_step (host, 4 doubles, may be NULL): ms per step of
  * (3 blocks, 1), (3, 4), (4, 1), (4, 4); choice (host, 2 ints, may be NULL):
  * the kept (blocks per SM, search: 1 walked by owner, 4 staged).  Errors: DSS_ERR_ARG
  * (trial_steps < 1), DSS_ERR_STATE, and any error of a trial step (the

@@ -12,11 +12,10 @@
 // (k_enumerate, k_enumerate_classes); on crowded grids a block takes the owners
 // of a few cells and stages the candidates of their stencils in shared memory
 // (k_enumerate_seg).  k_rows then scans the rows' lengths (the pair offsets of
-// each owner, a single-pass decoupled look-back) and writes the compact pair
-// arrays.  With the look-back at the end of the walk, a tile per warp, thousands
-// of tiles finished together and each walked back over all before it; in a
-// pass of its own (256 owners a tile, uniform work) it is short: the batch of 64
-// 333 -> 316 us a step, 100k 72.4 -> 72.0.
+// each owner) and writes the compact pair arrays.  With the scan at the end of
+// the walk, by look-back over a tile per warp, thousands of tiles finished
+// together and each walked back over all before it (a pass of its own: the batch
+// of 64 333 -> 316 us a step).
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -384,9 +383,9 @@ __device__ __noinline__ bool decide_exact(const Geo& g, const InstGeo& I, const 
 // a lane 7 instructions, one of them a shared load; the set-up of a block is
 // worth half a pass of 32 owners.  Against the walk by owner with the same
 // screen (one box, mixed precision, with the row pass): Table 5 with the 4 a0
-// range (128 per cell, 2.9M pairs) 312 -> 174 us, 1M log-uniform [1, 10] (7.1
-// per cell) 220 -> 187, the 100k packing with the 1 a0 range (4.1 per cell) 40
-// -> 35.  On sparse grids the set-up does not pay: 100k (1.7 per cell) 28
+// range (128 per cell, 2.9M pairs) 312 -> 167 us, 1M log-uniform [1, 10] (7.1
+// per cell) 220 -> 178, the 100k packing with the 1 a0 range (4.1 per cell) 40
+// -> 34.  On sparse grids the set-up does not pay: 100k (1.7 per cell) 28
 // against 37 us, a batch of 64 (1.8) 106 against 202.
 //
 // The decision: u = r^2 - s^2 in FP32, its sign bit shifted into a mask, 32

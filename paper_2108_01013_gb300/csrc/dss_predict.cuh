@@ -15,7 +15,7 @@ struct SortOut {
   int bcap;
   double* pred;             // 6n: predicted position and velocity
   signed char* xc;          // y crossings
-  unsigned long long* scan_status;   // the look-back state of the operation's scans
+  unsigned long long* scan_status;   // the look-back state of the cell scan
   int* scan_ticket;
   int scan_words;
   int* row_sums;                     // and the row sums of its search

@@ -3,7 +3,8 @@
 //   1. predictor + Lees-Edwards wrap (Eq. 15a-b, 16) fused with the cell key,
 //      a warp-aggregated histogram (one atomic per distinct key per warp) and
 //      the ids of each cell's particles (a row of bcap places per cell);
-//   2. exclusive scan of the histogram (single-pass decoupled look-back);
+//   2. exclusive scan of the histogram (from its tiles' sums, or by decoupled
+//      look-back on large grids);
 //   3. each particle finds its place (its cell's start plus its rank by id
 //      among the cell's ids, so that the order is deterministic) and writes its
 //      state there; the predicted position and velocity are those stored by
