@@ -1197,6 +1197,12 @@ int step_launch(dss_handle* h, int64_t remaining, StepRun& run) {
   int64_t left = remaining;
   for (int g = top; g >= 0; --g) {
     count[g] = left >> g;
+    // (capturing costs more than a few boundaries: the graphs of 4 and 2 steps
+    // are made when they are wanted a second time)
+    if (count[g] > 0 && g > 0 && g < DSS_GRAPHS - 1 && !h->graph_wanted[g]) {
+      h->graph_wanted[g] = true;
+      count[g] = 0;
+    }
     left -= count[g] << g;
     if (count[g] > 0 && !h->graph_ok[g][key] && (r = capture_steps(h, g, key))) return r;
     if (g == 0 && count[0] > 1 && !h->graph_ok[0][3 - key] && (r = capture_steps(h, 0, 3 - key))) return r;

@@ -752,6 +752,7 @@ struct dss_handle {
   // combination they start from; captured when first needed
   cudaGraphExec_t step_graph[DSS_GRAPHS][4];
   bool graph_ok[DSS_GRAPHS][4];
+  bool graph_wanted[DSS_GRAPHS];
   // kernel shapes chosen by dss_autotune_kernels (0: the built-in rule):
   // resident pair blocks per SM the register budget is cut for (3 or 4), and
   // the enumeration's search (1: walked by owner, 4: staged by segments)
