@@ -17,7 +17,7 @@
 // Bins a block of the cell scan takes, and the most blocks whose totals the
 // histogram keeps itself.
 constexpr int kScanTile = 2048;
-constexpr int kScanTiles = 128;
+constexpr int kScanTiles = 256;
 constexpr int kTileCopies = 8;
 
 // Device status word layout (int32 slots in DevStatus::w).

@@ -276,7 +276,8 @@ k_scan(const int* __restrict__ in, int* __restrict__ out, int count,
 // The same for grids of up to kScanTiles tiles, whose sums the histogram kept: a
 // tile's first bin is the sum of the tiles before it, so that no block waits
 // for another: one round of loads and one barrier.  The look-back of k_scan took 2
-// us more (8.2 -> 6.2 at 20k and 100k, 10.3 -> 8.0 at 140k bins).
+// us more (8.2 -> 6.2 at 20k and 100k, 10.3 -> 8.0 at 140k bins, 12.1 -> 8.1 at
+// 314k); a thread sums one tile's copies, so that 256 tiles are the limit.
 // The counts stay for the ranking kernel to clear.
 namespace {
 __global__ void __launch_bounds__(kScanThreads)

@@ -167,11 +167,12 @@ def test_runs_of_steps_as_single_steps(env, precision, ext):
         np.testing.assert_array_equal(a, b)
 
 
-@pytest.mark.parametrize("cells", [(16, 16, 8), (17, 11, 11), (12, 13, 13), (64, 64, 63), (64, 64, 64), (65, 64, 64)])
+@pytest.mark.parametrize("cells", [(16, 16, 8), (17, 11, 11), (12, 13, 13), (64, 64, 63), (64, 64, 64),
+                                   (65, 64, 64), (128, 64, 64), (129, 64, 64)])
 def test_cell_scan_at_tile_edges(env, cells):
     """Grids of one scan tile of 2048 cells exactly, a little more and less, of
-    128 tiles (the most whose sums the histogram keeps) and of one row more:
-    every search, also one behind another, finds the brute force's pairs."""
+    128 tiles, of 256 (the most whose sums the histogram keeps) and a little
+    more: every search, also one behind another, finds the brute force's pairs."""
     rng = np.random.default_rng(sum(cells))
     box = 3.0 * np.array(cells, dtype=np.float64)
     x = rng.uniform(0.0, 1.0, size=(3, 1500)) * box[:, None]
