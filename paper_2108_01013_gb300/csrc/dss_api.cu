@@ -270,7 +270,17 @@ int clear_err(dss_handle* h) {
     CK(cudaMemsetAsync(h->tile_count, 0, sizeof(int) * kTileCopies * kScanTiles, h->stream));
   }
   CK(cudaMemsetAsync(&h->status->w[ST_ERR], 0, sizeof(int), h->stream));
+  CK(cudaMemsetAsync(&h->status->w[ST_POVER], 0, sizeof(int), h->stream));
   return DSS_OK;
+}
+
+// The pairs of the evaluation that just failed when it failed because the pair
+// arrays hold fewer, else 0: rows that overflow are DSS_ERR_CAPACITY too, and
+// no growth of the pair arrays helps them.  From the host mirror, which
+// clear_err leaves as it was.
+int pairs_too_many(const dss_handle* h, int err) {
+  const int P = h->status_host->w[ST_POVER];
+  return err == DSS_ERR_CAPACITY && P > h->pcap ? P : 0;
 }
 
 // The committed state (sorted order) into id order: dst[k] is
@@ -361,6 +371,7 @@ __global__ void k_set_nstep(DevStatus* st, long long nstep) {
   st->w[ST_STEPS] = 0;
   st->w[ST_ERR] = 0;
   st->w[ST_CELL] = 0;
+  st->w[ST_POVER] = 0;
 }
 
 __global__ void k_iota(int n, int* __restrict__ v) {
@@ -1154,7 +1165,7 @@ int dss_force_eval(dss_handle* h, double* F, double* T) {
   CK(cudaGetLastError());
   int r = sync_status(h);
   if (r) return r;
-  if (status_error(h) == DSS_ERR_CAPACITY && h->status_host->w[ST_NPAIRS] > h->pcap) {
+  if (pairs_too_many(h, status_error(h))) {
     // more pairs than the pair arrays hold: grow them, list and evaluate again
     clear_err(h);
     if ((r = ensure_pair_capacity(h, list))) return r;
@@ -1250,8 +1261,7 @@ int step_run(dss_handle* h, int64_t nsteps) {
     if (!err) break;
     clear_err(h);
     // a pair-capacity overflow is recovered by growing the pair buffers
-    const int P = h->status_host->w[ST_NPAIRS];
-    if (err == DSS_ERR_CAPACITY && P > h->pcap && retries < 4) {
+    if (const int P = pairs_too_many(h, err); P && retries < 4) {
       ++retries;
       r = alloc_pair_buffers(h, (int64_t)(P * 1.25) + 1024, true);
       if (r) return r;
@@ -1309,8 +1319,8 @@ int dss_step_io(dss_handle* h, const double* const in[5], int64_t nsteps, double
     // finish as dss_step would, then read the state and the stress again
     if (err) {
       clear_err(h);
-      const int P = h->status_host->w[ST_NPAIRS];
-      if (err != DSS_ERR_CAPACITY || P <= h->pcap) return err;
+      const int P = pairs_too_many(h, err);
+      if (!P) return err;
       r = alloc_pair_buffers(h, (int64_t)(P * 1.25) + 1024, true);
       if (r) return r;
     }
@@ -2137,10 +2147,9 @@ int dss_adjoint(dss_handle* h, int64_t nsteps, int32_t ckpt_every, const double*
         // a step did not commit (e.g. the pair capacity grew): the segment
         // again from its checkpoint, one synchronised step at a time
         if (err) clear_err(h);
+        const int P = pairs_too_many(h, err);
         if ((r = snap_restore(h, ck[(size_t)s]))) return r;
-        const int P = h->status_host->w[ST_NPAIRS];
-        if (err == DSS_ERR_CAPACITY && P > h->pcap &&
-            (r = alloc_pair_buffers(h, (int64_t)(P * 1.25) + 1024, true)))
+        if (P && (r = alloc_pair_buffers(h, (int64_t)(P * 1.25) + 1024, true)))
           return r;
         // J back to its value at the segment's start: the sum so far
         CK(cudaMemcpy(h->adj->J, &Jacc, sizeof(double), cudaMemcpyHostToDevice));

@@ -648,7 +648,7 @@ k_pairs_pb(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sg
   const HistRef hr{perm, *((volatile const int*)&st->w[ST_IDORDER])};
   if (P > g.pcap) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-      st->w[ST_NPAIRS] = P;
+      st->w[ST_POVER] = P;
       set_err(st, DSS_ERR_CAPACITY);
     }
     return;

@@ -33,6 +33,8 @@ enum {
   ST_BADPOS = 8,     // set_state: positions outside the box
   ST_CELL = 10,      // a cell of more particles than its row of ids holds (0: none so far)
   ST_IDORDER = 9,    // 1 after dss_load_state: the committed state is not in the history's row order
+  ST_POVER = 11,     // pairs of the evaluation that failed because the pair arrays hold fewer; 0 beside
+                     // every other error (cleared with it)
   ST_WORDS = 16
 };
 
