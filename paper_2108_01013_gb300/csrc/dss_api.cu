@@ -48,7 +48,7 @@ void free_buffers(dss_handle* h) {
   h->pred = nullptr;
   dfree(h->xc); dfree(h->mark);
   h->xc = nullptr; h->mark = nullptr; h->marked = false;
-  dfree(h->cell_count); dfree(h->tile_count); h->tile_count = nullptr; dfree(h->cell_ids); h->cell_ids = nullptr; dfree(h->cell_start); dfree(h->tmp); dfree(h->spart);
+  dfree(h->cell_count); dfree(h->tile_count); h->tile_count = nullptr; dfree(h->cell_ids); h->cell_ids = nullptr; dfree(h->cell_more); h->cell_more = nullptr; dfree(h->cell_start); dfree(h->tmp); dfree(h->spart);
   dfree(h->own); dfree(h->bw_count); dfree(h->bw_rec); dfree(h->carry); dfree(h->own_s);
   h->own = nullptr; h->bw_count = nullptr; h->bw_rec = nullptr; h->carry = nullptr; h->own_s = nullptr;
   h->pb_blocks = 0;
@@ -209,10 +209,14 @@ int alloc_buffers(dss_handle* h) {
   CK(cudaMemsetAsync(h->tile_count, 0, sizeof(int) * kTileCopies * kScanTiles, h->stream));
   {
     // rows of ids: four times the average cell and twelve more (random
-    // packings stay within), shorter on grids of mostly empty cells
+    // packings stay within), shorter on grids of mostly empty cells; what lies
+    // beyond goes into chains
     const double per = (double)n / (double)h->g.ncell;
     h->cell_cap = per < 0.1 ? 4 : (per < 0.5 ? 8 : ((int)std::min(4.0 * per, 1e6) + 12 + 3) & ~3);
-    if ((r = dalloc(h, &h->cell_ids, (size_t)h->g.ncell * h->cell_cap))) return r;
+    if ((r = dalloc(h, &h->cell_ids, (size_t)h->g.ncell * h->cell_cap)) ||
+        (r = dalloc(h, &h->cell_more, (size_t)h->g.ncell)))
+      return r;
+    CK(cudaMemsetAsync(h->cell_more, 0, sizeof(int) * h->g.ncell, h->stream));
   }
   h->pcap = 0;
   int per = h->p.pair_capacity > 0 ? h->p.pair_capacity : 16;
@@ -221,30 +225,8 @@ int alloc_buffers(dss_handle* h) {
   return DSS_OK;
 }
 
-// Longer rows of ids after an operation that met a fuller cell.
-int grow_cells(dss_handle* h) {
-  CK(cudaStreamSynchronize(h->stream));
-  const int cap = (h->status_host->w[ST_CELL] + h->status_host->w[ST_CELL] / 2 + 3) & ~3;
-  int* ids = nullptr;
-  int r = dalloc(h, &ids, (size_t)h->g.ncell * cap);
-  if (r) {
-    cudaGetLastError();
-    return DSS_OK;   // the short rows still serve
-  }
-  dfree(h->cell_ids);
-  h->bytes -= (int64_t)(sizeof(int) * (size_t)h->g.ncell * h->cell_cap);
-  h->cell_ids = ids;
-  h->cell_cap = cap;
-  drop_graphs(h);
-  return DSS_OK;
-}
-
 // Orders the library's stream after everything queued on the caller's stream.
 int enter(dss_handle* h) {
-  if (h->sized && h->status_host->w[ST_CELL] > h->cell_cap) {
-    const int r = grow_cells(h);
-    if (r) return r;
-  }
   if (!h->own_stream) return DSS_OK;
   CK(cudaEventRecord(h->ev_enter, h->user_stream));
   CK(cudaStreamWaitEvent(h->stream, h->ev_enter, 0));
@@ -264,8 +246,10 @@ int sync_status(dss_handle* h) {
 }
 
 int clear_err(dss_handle* h) {
-  // (a step that failed in its corrector may have begun the next histogram)
+  // (a step that failed in its corrector may have begun the next histogram and
+  // its chains)
   if (h->sized) {
+    CK(cudaMemsetAsync(h->cell_more, 0, sizeof(int) * h->g.ncell, h->stream));
     CK(cudaMemsetAsync(h->cell_count, 0, sizeof(int) * h->g.ncell, h->stream));
     CK(cudaMemsetAsync(h->tile_count, 0, sizeof(int) * kTileCopies * kScanTiles, h->stream));
   }

@@ -31,7 +31,7 @@ enum {
   ST_NSTEP_LO = 6,   // time step counter (64 bit, lo/hi)
   ST_NSTEP_HI = 7,
   ST_BADPOS = 8,     // set_state: positions outside the box
-  ST_CELL = 10,      // a cell of more particles than its row of ids holds (0: none so far)
+  ST_CELL = 10,      // 1 once a cell held more particles than its row of ids
   ST_IDORDER = 9,    // 1 after dss_load_state: the committed state is not in the history's row order
   ST_POVER = 11,     // pairs of the evaluation that failed because the pair arrays hold fewer; 0 beside
                      // every other error (cleared with it)
@@ -706,13 +706,15 @@ struct dss_handle {
   bool marked;
   // counting sort scratch
   int* key;          // n
-  int* offs;         // n
+  int* offs;         // n: links' lanes while sorting, near pairs of a row while searching
   int* cell_count;   // ncell
   int* tile_count;   // kTileCopies x kScanTiles: counts of kScanTile bins each (grids of up to kScanTiles of them)
   int* cell_ids;     // ncell rows of cell_cap ids (a multiple of four)
   int cell_cap;
+  int* cell_more;    // ncell: the chain of the ids beyond the cell's row (index + 1 of its first
+                     // link, 0: none; its links in tmp and offs, see SortOut)
   int* cell_start;   // ncell+1
-  int* tmp;          // n
+  int* tmp;          // n: links of the cells' chains
   // lists: hist = committed (history source), work = being built
   ListBuf lb[2];
   int hist;

@@ -683,12 +683,13 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
 template <bool SPLIT, int TILE>
 __global__ void __launch_bounds__(kRowThreads)
 k_rows(int n, int M, int Ms, int64_t pcap, const int* __restrict__ ids, const __grid_constant__ ListBuf L,
-       const int* __restrict__ nnear, int* __restrict__ bw_count, RowSums R, DevStatus* st) {
+       const int* __restrict__ nnear, int* __restrict__ bw_count, const int* __restrict__ cellid,
+       int* __restrict__ cell_more, RowSums R, DevStatus* st) {
   dep_wait();
   constexpr int kAhead = 4;                  // pairs a thread has in flight
   __shared__ int s_warp[kRowThreads / 32], s_pre[kRowThreads / 32];
   __shared__ int s_ex[TILE + 1], s_near[SPLIT ? TILE : 1];
-  const int err = dev_err(st);
+  const int err = dev_err(st), chains = st->w[ST_CELL];
   const int tile = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int i0 = tile * TILE, i = i0 + threadIdx.x;
   const bool own = threadIdx.x < TILE && i < n;
@@ -756,6 +757,7 @@ k_rows(int n, int M, int Ms, int64_t pcap, const int* __restrict__ ids, const __
       set_err(st, DSS_ERR_CAPACITY);
     }
     bw_count[i] = 0;
+    if (chains) cell_more[cellid[i]] = 0;      // the sort's, for the next one
     const int id = ids[i];
     L.slot_of_id[id] = i;
     L.id_of_slot[i] = id;
@@ -912,6 +914,6 @@ void launch_enumerate(dss_handle* h, int stbuf, int dst_list, int adv) {
   }
   auto kr = split ? k_rows<true, 64> : k_rows<false, 256>;
   launch_dep(kr, ((int)h->n + tile - 1) / tile, kRowThreads, h->stream, (int)h->n, g.M, g.Ms, g.pcap, h->st[stbuf].id, L,
-             h->offs, h->bw_count, R, h->status);
+             h->offs, h->bw_count, h->cellid, h->cell_more, R, h->status);
   h->last_list = dst_list;
 }

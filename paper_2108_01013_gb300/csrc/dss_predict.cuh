@@ -13,6 +13,13 @@ struct SortOut {
   int* tile_count;          // its sums over the scan's tiles (null: too many)
   int* cell_ids;            // per cell a row of bcap ids
   int bcap;
+  // ids beyond a cell's row: a chain of links per cell, each the particles that
+  // one warp brought (a mask of its lanes), kept at the first one's index.
+  // Consecutive particles are neighbours in space, so that a link holds many of
+  // the cell; no cell's fullness costs memory or work elsewhere.
+  int* more;                // per cell: index + 1 of its last link (cleared by the row pass)
+  int* link_next;
+  unsigned* link_lanes;
   double* pred;             // 6n: predicted position and velocity
   signed char* xc;          // y crossings
   unsigned long long* scan_status;   // the look-back state of the cell scan
@@ -29,6 +36,9 @@ inline SortOut sort_out(const dss_handle* h) {
                  scan_tiles_for(h->g.ncell) <= kScanTiles ? h->tile_count : nullptr,
                  h->cell_ids,
                  h->cell_cap,
+                 h->cell_more,
+                 h->tmp,
+                 reinterpret_cast<unsigned*>(h->offs),
                  h->pred,
                  h->xc,
                  h->scan_status,
@@ -146,8 +156,9 @@ __device__ __forceinline__ int cell_key(const InstGeo& I, int cls, double x, dou
   return I.cell_base + cls * I.ncell_layer + (cz * I.nc[1] + cy) * I.nc[0] + cx;
 }
 
-// The particle's key, its count and its id in the cell's row (called by all
-// active lanes of a warp together).
+// The particle's key, its count and its id in the cell's row, or in a link of the
+// cell's chain (called by all active lanes of a warp together; i lies at the
+// lane's place in a row of 32).
 __device__ __forceinline__ void key_insert(const SortOut& q, int i, int k, int id) {
   const unsigned act = __activemask();
   const unsigned peers = __match_any_sync(act, k);
@@ -171,7 +182,12 @@ __device__ __forceinline__ void key_insert(const SortOut& q, int i, int k, int i
   }
   base = __shfl_sync(peers, base, leader) + rank;
   q.key[i] = k;
-  if (base < q.bcap) q.cell_ids[(int64_t)k * q.bcap + base] = id;
+  if (base < q.bcap) {
+    q.cell_ids[(int64_t)k * q.bcap + base] = id;
+  } else if (base == q.bcap || rank == 0) {   // the first of the warp's beyond the row
+    q.link_lanes[i] = peers & (0xffffffffu << lane);
+    q.link_next[i] = atomicExch(&q.more[k], i + 1);
+  }
 }
 
 __device__ __forceinline__ void store_pred(const SortOut& q, int n, int i, const Pred& p) {

@@ -53,17 +53,53 @@ k_key_hist(const __grid_constant__ Geo g, const InstGeo* __restrict__ ig, const 
   key_insert(q, i, cell_key(I, cls, x, y, z), id);
 }
 
+// The ids below mine among those beyond a full cell's row, in its chain of links
+// (SortOut): a link is a round or more of loads for up to 32 ids, the next one on
+// its way.  The work is the cell's own, quadratic in its particles as for every
+// other cell.  20,000 small spheres segregated from the large ones, a thousand to
+// a cell whose row holds 168: 59 us for the kernel (41 with all ids of a cell side
+// by side, written by a kernel of its own that every step paid for).  A clump of
+// 50,000 in a dilute box, rows of four: 10.3 us, a step 60 us from the first on.
+// (Ranked over all particles' keys, with longer rows from the host's next call,
+// the steps of the first call took 1380 us each.)
+__device__ __noinline__ int rank_beyond_row(const int* __restrict__ id, int mine, int first, int left,
+                                            const int* __restrict__ next, const unsigned* __restrict__ lanes) {
+  int rank = 0, e = first;
+  unsigned m = e ? lanes[e - 1] : 0u;
+  int to = e ? next[e - 1] : 0;
+  while (e && left > 0) {
+    const int base = (e - 1) & ~31;
+    unsigned cur = m;
+    left -= __popc(cur);
+    // the next link comes while this one's ids do
+    e = to;
+    m = e ? lanes[e - 1] : 0u;
+    to = e ? next[e - 1] : 0;
+    while (cur) {
+      int v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        v[u] = cur ? id[base + __ffs(cur) - 1] : 0x7fffffff;
+        cur &= cur - 1u;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) rank += v[u] < mine;
+    }
+  }
+  return rank;
+}
+
 // 3. the place of each particle: inside a cell by id, so that the sorted order,
 // and with it every summation order downstream, is a function of positions and
 // ids alone; its state written there (WAVE: the wave of Eq. 17 is on, compiled
-// out otherwise).  A cell of more particles than its row of ids holds is
-// ranked over all particles' keys, and the host gives the next operation longer
-// rows (ST_CELL).
+// out otherwise).
 template <bool WAVE>
 __global__ void __launch_bounds__(kThreads, 4)
 k_rank_gather(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sgk, StateBuf src,
               StateBuf dst, const int* __restrict__ key, const int* __restrict__ cell_start,
-              const int* __restrict__ cell_ids, int bcap, int* __restrict__ cell_count,
+              const int* __restrict__ cell_ids, int bcap, const int* __restrict__ more,
+              const int* __restrict__ link_next, const unsigned* __restrict__ link_lanes,
+              int* __restrict__ cell_count,
               int* __restrict__ tile_count, int clear, int* __restrict__ perm, int* __restrict__ cellid,
               float4* __restrict__ posf, DevStatus* st, bool predict,
               const double* __restrict__ pred, const signed char* __restrict__ xc) {
@@ -98,15 +134,15 @@ k_rank_gather(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__
     wa[c] = src.aw[c * n + o];
   }
   int rank = 0;
-  if (cnt <= bcap) {
-    const int4* __restrict__ row = reinterpret_cast<const int4*>(cell_ids + (int64_t)k * bcap);
-    for (int q = 0; q < cnt; q += 4) {
-      const int4 v = __ldg(row + (q >> 2));
-      rank += (v.x < id) + (q + 1 < cnt && v.y < id) + (q + 2 < cnt && v.z < id) + (q + 3 < cnt && v.w < id);
-    }
-  } else {
-    for (int q = 0; q < n; ++q) rank += key[q] == k && src.id[q] < id;
-    if (rank == 0) atomicMax(&st->w[ST_CELL], cnt);
+  const int4* __restrict__ row = reinterpret_cast<const int4*>(cell_ids + (int64_t)k * bcap);
+  const int held = min(cnt, bcap);
+  for (int q = 0; q < held; q += 4) {
+    const int4 v = __ldg(row + (q >> 2));
+    rank += (v.x < id) + (q + 1 < held && v.y < id) + (q + 2 < held && v.z < id) + (q + 3 < held && v.w < id);
+  }
+  if (cnt > bcap) {
+    rank += rank_beyond_row(src.id, id, more[k], cnt - bcap, link_next, link_lanes);
+    if (rank == 0) st->w[ST_CELL] = 1;
   }
   const int f = c0 + rank;
   perm[f] = o;
@@ -366,14 +402,15 @@ void launch_sort(dss_handle* h, bool predict, int src, int dst, bool keyed) {
   prof_mark(h, 2);
   prof_mark(h, 3);
   const int clear = scan_tiles_for(h->g.ncell) <= kScanTiles ? h->g.ncell : 0;
+  const SortOut so = sort_out(h);
   if (h->g.wave)
     launch_dep(k_rank_gather<true>, blocks, kThreads, h->stream, h->g, h->ig, h->sg, h->st[src], h->st[dst], h->key,
-                                                            h->cell_start, h->cell_ids, h->cell_cap,
+                                                            h->cell_start, h->cell_ids, h->cell_cap, so.more, so.link_next, so.link_lanes,
                h->cell_count, h->tile_count, clear, h->perm, h->cellid,
                                                             h->posf, h->status, predict, h->pred, h->xc);
   else
     launch_dep(k_rank_gather<false>, blocks, kThreads, h->stream, h->g, h->ig, h->sg, h->st[src], h->st[dst], h->key,
-                                                             h->cell_start, h->cell_ids, h->cell_cap,
+                                                             h->cell_start, h->cell_ids, h->cell_cap, so.more, so.link_next, so.link_lanes,
                h->cell_count, h->tile_count, clear, h->perm, h->cellid,
                                                              h->posf, h->status, predict, h->pred, h->xc);
 }
