@@ -355,6 +355,7 @@ __global__ void k_set_nstep(DevStatus* st, long long nstep) {
   st->w[ST_STEPS] = 0;
   st->w[ST_ERR] = 0;
   st->w[ST_CELL] = 0;
+  st->w[ST_LONG] = 0;
   st->w[ST_POVER] = 0;
 }
 

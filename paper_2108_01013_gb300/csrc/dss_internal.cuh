@@ -33,6 +33,7 @@ enum {
   ST_BADPOS = 8,     // set_state: positions outside the box
   ST_CELL = 10,      // 1 once a cell held more particles than its row of ids
   ST_IDORDER = 9,    // 1 after dss_load_state: the committed state is not in the history's row order
+  ST_LONG = 12,      // 1 once a segment of the staged search may have held more owners than its blocks take
   ST_POVER = 11,     // pairs of the evaluation that failed because the pair arrays hold fewer; 0 beside
                      // every other error (cleared with it)
   ST_WORDS = 16
@@ -766,6 +767,8 @@ struct dss_handle {
   bool enum_walk;
   bool enum_narrow;          // boxes where the staged search meets separations past exact_beyond
   int64_t enum_blocks;
+  int enum_most_seg;         // cells of the longest segment of the staged search
+  int enum_long_seg;         // owners beyond which a segment's are shared out (ST_LONG)
   int* enum_inst;            // instance of each of its blocks (batched instances; else null)
   int64_t enum_inst_cap;
   int64_t bytes;

@@ -406,59 +406,61 @@ __device__ __noinline__ bool decide_exact(const Geo& g, const InstGeo& I, const 
 // an FP32 test go to the row's front, the others to its back from the end;
 // k_rows closes the row up.
 // ------------------------------------------------------------------------
-template <bool ECH, bool SPLIT, bool ONE, bool NARROW>
-__global__ void __launch_bounds__(32 * kRows, 7)
-k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I1, const InstGeo* __restrict__ ig,
-            const StepGeo* __restrict__ sgk, const __grid_constant__ StateBuf s, const float4* __restrict__ posf,
-            const int* __restrict__ cellid, const int* __restrict__ cell_start, int* __restrict__ list,
-            int* __restrict__ count, int* __restrict__ nnear, const int* __restrict__ blk_inst, RowSums R,
-            DevStatus* st, EnumCut q) {
-  dep_wait();
-  __shared__ float4 s_c[kRows][kTile + 4];
-  __shared__ int s_j[kRows][kTile];
-  __shared__ int s_off[kRows][32];
-  __shared__ int s_len[kRows];
-  __shared__ int s_cnt[2][kRows][32];      // pairs of each owner in each row (near ones << 16: SPLIT)
-  __shared__ int4 s_par[kRows];            // rows: bin of their x = 0, x of their first cell, cells, image across y
-  __shared__ int s_seg[4];                 // first bin, cells, part, first owner
-  if (dev_err(st)) return;
-  int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
-  asm volatile("" : "+r"(lane), "+r"(r));     // kept, not taken anew in every loop
-  const int inst = ONE ? 0 : blk_inst[blockIdx.x];
-  const InstGeo& I = ONE ? I1 : ig[inst];
-  const StepGeo sg = sgk[inst];
-  const int nx = I.nc[0], ny = I.nc[1], nz = I.nc[2];
-  if (r == 0) {
-    // the first warp finds the segment, a lane for each of its rows
-    unsigned item = blockIdx.x - (ONE ? 0 : I.enum_blk);
-    const int seg = I.enum_seg, subs = I.enum_subs;
-    int sub = 0;
-    if (subs > 1) {
-      const unsigned h = item / (unsigned)subs;
-      sub = (int)(item - h * subs);
-      item = h;
-    }
-    const int row = (int)(item / (unsigned)I.enum_hx);
-    const int x0 = ((int)item - row * I.enum_hx) * seg;
-    const int cz = row / ny, cy = row - cz * ny;
-    const int bxe = min(seg, nx - x0);
-    const bool img = lane >= 2 && cy == ny - 1;
-    int xf = lane == 0 ? x0 : (img ? wrapi(x0 - 2 - sg.fsh, nx) : x0 - 1);
-    if (xf < 0) xf += nx;
-    const int qy = lane < 2 ? cy : (cy == ny - 1 ? 0 : cy + 1);
-    int qz = lane == 0 ? cz : (lane == 1 ? cz + 1 : cz + lane - 3);
-    qz = qz < 0 ? nz - 1 : (qz == nz ? 0 : qz);
-    if (lane < kRows)
-      s_par[lane] = make_int4(I.cell_base + (qz * ny + qy) * nx, xf, bxe + (lane == 0 ? 1 : (img ? 3 : 2)), img);
-    if (lane == 0) {
-      s_seg[0] = I.cell_base + row * nx + x0;
-      s_seg[1] = bxe;
-      s_seg[2] = sub + 1 < subs ? sub : -1 - sub;
-    }
+// What a block of the staged search keeps in shared memory.
+struct SegShared {
+  float4 c[kRows][kTile + 4];
+  int j[kRows][kTile];
+  int off[kRows][32];
+  int len[kRows];
+  int cnt[2][kRows][32];      // pairs of each owner in each row (near ones << 16: SPLIT)
+  int4 par[kRows];            // rows: bin of their x = 0, x of their first cell, cells, image across y
+  int seg[4];                 // first bin, cells, part, first owner
+  int far;                    // the group to take after the block's own owners (-1: none is left)
+};
+
+// The segment from x0 on in a row of cells: its half stencil's rows, a lane each
+// (by one warp).
+__device__ __forceinline__ void set_segment(SegShared& sh, const InstGeo& I, int fsh, int row, int x0, int part) {
+  const int nx = I.nc[0], ny = I.nc[1], nz = I.nc[2], lane = threadIdx.x & 31;
+  const int cz = row / ny, cy = row - cz * ny;
+  const int bxe = min(I.enum_seg, nx - x0);
+  const bool img = lane >= 2 && cy == ny - 1;
+  int xf = lane == 0 ? x0 : (img ? wrapi(x0 - 2 - fsh, nx) : x0 - 1);
+  if (xf < 0) xf += nx;
+  const int qy = lane < 2 ? cy : (cy == ny - 1 ? 0 : cy + 1);
+  int qz = lane == 0 ? cz : (lane == 1 ? cz + 1 : cz + lane - 3);
+  qz = qz < 0 ? nz - 1 : (qz == nz ? 0 : qz);
+  if (lane < kRows)
+    sh.par[lane] = make_int4(I.cell_base + (qz * ny + qy) * nx, xf, bxe + (lane == 0 ? 1 : (img ? 3 : 2)), img);
+  if (lane == 0) {
+    sh.seg[0] = I.cell_base + row * nx + x0;
+    sh.seg[1] = bxe;
+    sh.seg[2] = part;
   }
-  __syncthreads();
+}
+
+// Owners of a segment of len that its own blocks take (and on to a multiple of
+// 32 in the sorted order): all, up to seven passes more than its average blocks
+// have; of a longer one, whose stencil rows are long too, those blocks' alone.
+__host__ __device__ __forceinline__ int seg_long(const InstGeo& I) { return 32 * I.enum_subs + 224; }
+__device__ __forceinline__ int seg_limit(const InstGeo& I, int len) {
+  return len <= seg_long(I) ? len : 32 * I.enum_subs;
+}
+
+// Group k of those a block looks at for owners beyond their segment's limit: 32 owners
+// from a multiple of 32 in the sorted order on, one in gridDim.x.
+__device__ __forceinline__ int64_t far_group(int k) { return blockIdx.x + (int64_t)k * gridDim.x; }
+
+// The segment in sh.par and sh.seg (complete at a barrier before the call): the
+// owners of the block's part of it, or (grp >= 0) a group of its owners.
+template <bool ECH, bool SPLIT, bool NARROW>
+__device__ __forceinline__ void search_segment(
+    SegShared& sh, const Geo& g, const InstGeo& I, const StepGeo& sg, const StateBuf& s, const float4* __restrict__ posf,
+    const int* __restrict__ cellid, const int* __restrict__ cell_start, int* __restrict__ list, int* __restrict__ count,
+    int* __restrict__ nnear, const RowSums& R, DevStatus* st, const EnumCut& q, int lane, int r, int grp) {
+  const int nx = I.nc[0], ny = I.nc[1], nz = I.nc[2];
   // the warp's row: w cells from x = xf on, of the row of cells at rc
-  const int4 par = s_par[r];
+  const int4 par = sh.par[r];
   const int rc = par.x, xf = par.y, w = par.z;
   const bool le = par.w != 0;
   // lane k: the boundary before its cell k, as a place in the row's sequence;
@@ -475,16 +477,17 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
   } else {
     b -= first;
   }
-  s_off[r][lane] = b;
+  sh.off[r][lane] = b;
   const int len = __shfl_sync(0xffffffffu, b, w);
   if (lane == 0) {
-    s_len[r] = len;
-    if (r == 0) s_seg[3] = first;
+    sh.len[r] = len;
+    if (r == 0) sh.seg[3] = first;
   }
   __syncthreads();
-  const int c0 = s_seg[0], part = s_seg[2], hs = s_seg[3], he = hs + s_off[0][s_seg[1]];
-  const int o_beg = hs + 32 * (part < 0 ? -1 - part : part), o_end = part < 0 ? he : min(o_beg + 32, he);
-  const int most = max(max(max(s_len[0], s_len[1]), max(s_len[2], s_len[3])), s_len[4]);
+  const int c0 = sh.seg[0], part = sh.seg[2], hs = sh.seg[3], he = hs + sh.off[0][sh.seg[1]];
+  const int o_beg = grp >= 0 ? 32 * grp : hs + 32 * (part < 0 ? -1 - part : part);
+  const int o_end = min(grp >= 0 || part >= 0 ? o_beg + 32 : (hs + seg_limit(I, he - hs) + 31) & ~31, he);
+  const int most = max(max(max(sh.len[0], sh.len[1]), max(sh.len[2], sh.len[3])), sh.len[4]);
   const float kx0 = r == 0 ? 0.f : (le ? -2.f : -1.f), sx = le ? sg.offr_hi : 0.f;
   const float sy = r < 2 ? 0.f : I.csf[1];
   const float sz = r == 0 ? 0.f : (r == 1 ? I.csf[2] : (float)(r - 3) * I.csf[2]);
@@ -507,8 +510,8 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
       pz = p.z;
       pa = p.w;
       sa = fmaf(p.w, q.sc, q.sd);
-      lo = r == 0 ? i - hs + 1 : s_off[r][kx];
-      hi = s_off[r][kx + (r == 0 ? 2 : (le ? 4 : 3))];
+      lo = r == 0 ? i - hs + 1 : sh.off[r][kx];
+      hi = sh.off[r][kx + (r == 0 ? 2 : (le ? 4 : 3))];
     }
     const uint64_t npx = pk2(-px, -px), npy = pk2(-py, -py), npz = pk2(-pz, -pz);
     const uint64_t sc2 = pk2(q.sc, q.sc), sa2 = pk2(sa, sa), nsc2 = pk2(-q.sc, -q.sc), nsa2 = pk2(-sa, -sa);
@@ -530,13 +533,13 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
             c.x += fmaf((float)kc + kx0, I.csf[0], sx);
             c.y += sy;
             c.z += sz;
-            s_j[r][p - t0] = j;
+            sh.j[r][p - t0] = j;
           }
           // even lanes hold the two particles' x and y, odd ones z and a
           const float va = __shfl_xor_sync(0xffffffffu, lane & 1 ? c.x : c.z, 1);
           const float vb = __shfl_xor_sync(0xffffffffu, lane & 1 ? c.y : c.w, 1);
           if ((p & ~1) < t1)
-            s_c[r][p - t0] = lane & 1 ? make_float4(va, c.z, vb, c.w) : make_float4(c.x, va, c.y, vb);
+            sh.c[r][p - t0] = lane & 1 ? make_float4(va, c.z, vb, c.w) : make_float4(c.x, va, c.y, vb);
         }
         __syncwarp();
       }
@@ -550,7 +553,7 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
         if (h >= words) continue;
         const int m = min(32, z - a - 32 * h);
         if (m <= 0) continue;
-        const float4* __restrict__ c = &s_c[r][a + 32 * h];
+        const float4* __restrict__ c = &sh.c[r][a + 32 * h];
         float least = __int_as_float(0x7f800000);
         int n = 0;
         do {
@@ -592,7 +595,7 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
             if (!(fabsf(t) > m2) ||
                 (img && (fabsf(dx) > exact_beyond(I, 0) || fabsf(dy) > exact_beyond(I, 1) || fabsf(dz) > exact_beyond(I, 2)))) {
               ++band;
-              if (decide_exact(g, I, s, sg.off, i, s_j[r][a + 32 * h + e])) hit[h] |= bit;
+              if (decide_exact(g, I, s, sg.off, i, sh.j[r][a + 32 * h + e])) hit[h] |= bit;
               else hit[h] &= ~bit;
             }
           }
@@ -609,7 +612,7 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
           for (unsigned left = hit[h]; left;) {
             const int e = __clz(left);
             left &= ~(0x80000000u >> e);
-            const float4 pj = staged(s_c[r], a + 32 * h + e);
+            const float4 pj = staged(sh.c[r], a + 32 * h + e);
             const float dx = pj.x - px, dy = pj.y - py, dz = pj.z - pz;
             const float sl = fmaf(pa + pj.w, q.lc, q.ld);
             if (fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < sl * sl) nrm[h] |= 0x80000000u >> e;
@@ -617,13 +620,13 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
           mine += __popc(nrm[h]) << 16;
         }
       }
-      s_cnt[buf][r][lane] = mine;
+      sh.cnt[buf][r][lane] = mine;
       __syncthreads();
       int at = 0, tot = 0;
 #pragma unroll
       for (int v = 0; v < kRows; ++v) {
         if (v == r) at = tot;
-        tot += s_cnt[buf][v][lane];
+        tot += sh.cnt[buf][v][lane];
       }
       buf ^= 1;
       // the warp's part of the owner's row
@@ -635,7 +638,7 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
           const int e = __clz(left);
           const unsigned bit = 0x80000000u >> e;
           left &= ~bit;
-          const int j = s_j[r][a + 32 * h + e];
+          const int j = sh.j[r][a + 32 * h + e];
           if (SPLIT) {
             if (kn + kf < g.M) rw[nrm[h] & bit ? kn : g.M - 1 - kf] = j;
             if (nrm[h] & bit) ++kn; else ++kf;
@@ -665,6 +668,80 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
     band = __reduce_add_sync(0xffffffffu, band);
     if (lane == 0) atomicAdd(&st->w[ST_BAND], band);
   }
+}
+
+// The owners beyond their segments' limits (few cells that hold most of the
+// particles: segregated sizes), a group after another, after the block's own.
+// Out of line and behind the sort's word that there are any (ST_LONG): looking
+// for them in every block cost 2% of the search of 1M.  The search of 20,000
+// small spheres beside a few large ones, a thousand to a cell of 512, 0.56 ms
+// instead of 4.0 with such a cell's owners left to its last block (walked by
+// owner 0.60); of 200,000 in 1000 cells 1.8 instead of 5.4 (4.4).
+template <bool ECH, bool SPLIT, bool ONE, bool NARROW>
+__device__ __noinline__ void search_far(
+    SegShared& sh, const Geo& g, const InstGeo& I1, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sgk,
+    const StateBuf& s, const float4* __restrict__ posf, const int* __restrict__ cellid,
+    const int* __restrict__ cell_start, int* __restrict__ list, int* __restrict__ count, int* __restrict__ nnear,
+    const RowSums& R, DevStatus* st, const EnumCut& q) {
+  const int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
+  for (int k = 0;; ++k) {
+    __syncthreads();
+    if (r == 0) {
+      int found = -1;
+      for (; found < 0 && 32 * far_group(k) < g.n; ++k) {
+        const int64_t gk = far_group(k);
+        const int i = 32 * (int)gk, inst = ONE ? 0 : s.inst[i];
+        const InstGeo& I = ONE ? I1 : ig[inst];
+        const int c = cellid[i], x = (c - I.cell_base) % I.nc[0], dx = x % I.enum_seg;
+        const int hs = cell_start[c - dx], he = cell_start[c - dx + min(I.enum_seg, I.nc[0] - x + dx)];
+        if (i - hs < seg_limit(I, he - hs)) continue;
+        found = (int)gk;
+        set_segment(sh, I, sgk[inst].fsh, (c - I.cell_base) / I.nc[0], x - dx, -1);
+        break;
+      }
+      if (lane == 0) sh.far = found;
+    }
+    __syncthreads();
+    const int grp = sh.far;
+    if (grp < 0) return;
+    const int inst = ONE ? 0 : s.inst[32 * grp];
+    search_segment<ECH, SPLIT, NARROW>(sh, g, ONE ? I1 : ig[inst], sgk[inst], s, posf, cellid, cell_start, list, count,
+                                       nnear, R, st, q, lane, r, grp);
+  }
+}
+
+template <bool ECH, bool SPLIT, bool ONE, bool NARROW>
+__global__ void __launch_bounds__(32 * kRows, 7)
+k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I1, const InstGeo* __restrict__ ig,
+            const StepGeo* __restrict__ sgk, const __grid_constant__ StateBuf s, const float4* __restrict__ posf,
+            const int* __restrict__ cellid, const int* __restrict__ cell_start, int* __restrict__ list,
+            int* __restrict__ count, int* __restrict__ nnear, const int* __restrict__ blk_inst,
+            const __grid_constant__ RowSums R, DevStatus* st, const __grid_constant__ EnumCut q) {
+  dep_wait();
+  __shared__ SegShared sh;
+  if (dev_err(st)) return;
+  int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
+  asm volatile("" : "+r"(lane), "+r"(r));     // kept, not taken anew in every loop
+  const int inst = ONE ? 0 : blk_inst[blockIdx.x];
+  const InstGeo& I = ONE ? I1 : ig[inst];
+  const StepGeo sg = sgk[inst];
+  if (r == 0) {
+    // the first warp finds the segment
+    unsigned item = blockIdx.x - (ONE ? 0 : I.enum_blk);
+    const int subs = I.enum_subs;
+    int sub = 0;
+    if (subs > 1) {
+      const unsigned h = item / (unsigned)subs;
+      sub = (int)(item - h * subs);
+      item = h;
+    }
+    const int row = (int)(item / (unsigned)I.enum_hx);
+    set_segment(sh, I, sg.fsh, row, ((int)item - row * I.enum_hx) * I.enum_seg, sub + 1 < subs ? sub : -1 - sub);
+  }
+  __syncthreads();
+  search_segment<ECH, SPLIT, NARROW>(sh, g, I, sg, s, posf, cellid, cell_start, list, count, nnear, R, st, q, lane, r, -1);
+  if (st->w[ST_LONG])
+    search_far<ECH, SPLIT, ONE, NARROW>(sh, g, I1, ig, sgk, s, posf, cellid, cell_start, list, count, nnear, R, st, q);
 }
 
 // Row pass: counters, the id <-> row maps, the exclusive scan of the row
@@ -829,6 +906,8 @@ int64_t enum_plan(dss_handle* h, std::vector<int>* blk_inst) {
   h->enum_walk = h->g.nclass > 1 || h->tune_enum_unr == 1 || (h->tune_enum_unr == 0 && (sparse || empty));
   int64_t blk = 0;
   h->enum_narrow = false;
+  h->enum_most_seg = 0;
+  h->enum_long_seg = INT_MAX;
   if (blk_inst) blk_inst->clear();
   for (int k = 0; k < h->K; ++k) {
     InstGeo& I = h->ig_host[k];
@@ -854,12 +933,17 @@ int64_t enum_plan(dss_handle* h, std::vector<int>* blk_inst) {
     }
     I.enum_hx = hx;
     I.enum_seg = (nx + hx - 1) / hx;
+    h->enum_most_seg = std::max(h->enum_most_seg, I.enum_seg);
+    h->enum_long_seg = std::min(h->enum_long_seg, seg_long(I));
     I.enum_blk = (int)blk;
     const int64_t items = (int64_t)hx * I.nc[1] * I.nc[2] * I.enum_subs;
     if (blk_inst && !h->enum_walk) blk_inst->insert(blk_inst->end(), (size_t)items, k);
     blk += items;
   }
-  if (h->enum_walk) blk = (h->n + kThreads - 1) / kThreads;
+  if (h->enum_walk) {
+    blk = (h->n + kThreads - 1) / kThreads;
+    h->enum_long_seg = INT_MAX;
+  }
   h->enum_blocks = blk;
   return blk;
 }

@@ -101,7 +101,7 @@ k_rank_gather(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__
               const int* __restrict__ link_next, const unsigned* __restrict__ link_lanes,
               int* __restrict__ cell_count,
               int* __restrict__ tile_count, int clear, int* __restrict__ perm, int* __restrict__ cellid,
-              float4* __restrict__ posf, DevStatus* st, bool predict,
+              float4* __restrict__ posf, DevStatus* st, int most_seg, int long_seg, bool predict,
               const double* __restrict__ pred, const signed char* __restrict__ xc) {
   dep_wait();
   if (dev_err(st)) return;
@@ -144,6 +144,9 @@ k_rank_gather(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__
     rank += rank_beyond_row(src.id, id, more[k], cnt - bcap, link_next, link_lanes);
     if (rank == 0) st->w[ST_CELL] = 1;
   }
+  // (the search's segments: a segment's cells lie among the most_seg from its
+  // first particle's on)
+  if (rank == 0 && cell_start[min(k + most_seg, g.ncell)] - c0 > long_seg) st->w[ST_LONG] = 1;
   const int f = c0 + rank;
   perm[f] = o;
   cellid[f] = k;
@@ -407,12 +410,12 @@ void launch_sort(dss_handle* h, bool predict, int src, int dst, bool keyed) {
     launch_dep(k_rank_gather<true>, blocks, kThreads, h->stream, h->g, h->ig, h->sg, h->st[src], h->st[dst], h->key,
                                                             h->cell_start, h->cell_ids, h->cell_cap, so.more, so.link_next, so.link_lanes,
                h->cell_count, h->tile_count, clear, h->perm, h->cellid,
-                                                            h->posf, h->status, predict, h->pred, h->xc);
+                                                            h->posf, h->status, h->enum_most_seg, h->enum_long_seg, predict, h->pred, h->xc);
   else
     launch_dep(k_rank_gather<false>, blocks, kThreads, h->stream, h->g, h->ig, h->sg, h->st[src], h->st[dst], h->key,
                                                              h->cell_start, h->cell_ids, h->cell_cap, so.more, so.link_next, so.link_lanes,
                h->cell_count, h->tile_count, clear, h->perm, h->cellid,
-                                                             h->posf, h->status, predict, h->pred, h->xc);
+                                                             h->posf, h->status, h->enum_most_seg, h->enum_long_seg, predict, h->pred, h->xc);
 }
 
 // Self-test of the integer-operation conversions (f32_rn, f32_split, f64_of,
