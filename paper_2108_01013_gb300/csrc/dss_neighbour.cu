@@ -766,7 +766,7 @@ k_rows(int n, int M, int Ms, int64_t pcap, const int* __restrict__ ids, const __
   constexpr int kAhead = 4;                  // pairs a thread has in flight
   __shared__ int s_warp[kRowThreads / 32], s_pre[kRowThreads / 32];
   __shared__ int s_ex[TILE + 1], s_near[SPLIT ? TILE : 1];
-  const int err = dev_err(st), chains = st->w[ST_CELL];
+  const int err = dev_err(st);
   const int tile = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int i0 = tile * TILE, i = i0 + threadIdx.x;
   const bool own = threadIdx.x < TILE && i < n;
@@ -834,7 +834,6 @@ k_rows(int n, int M, int Ms, int64_t pcap, const int* __restrict__ ids, const __
       set_err(st, DSS_ERR_CAPACITY);
     }
     bw_count[i] = 0;
-    if (chains) cell_more[cellid[i]] = 0;      // the sort's, for the next one
     const int id = ids[i];
     L.slot_of_id[id] = i;
     L.id_of_slot[i] = id;
@@ -852,6 +851,7 @@ k_rows(int n, int M, int Ms, int64_t pcap, const int* __restrict__ ids, const __
       if (SPLIT && ak[r] >= 0) L.list[(int64_t)(i0 + ao[r]) * Ms + ak[r]] = aj[r];
     }
   }
+  if (own && st->w[ST_CELL]) cell_more[cellid[i]] = 0;   // the sort's chains, for the next one
   for (int t0 = kAhead * kRowThreads; t0 < total; t0 += kRowThreads) {
     const int t = t0 + threadIdx.x;
     int o = 0, k = 0, src = 0, j = 0;
