@@ -202,13 +202,13 @@ __device__ __forceinline__ PairRes<double> pair_eval_fp64(const Geo& g, const In
   return q;
 }
 
-// Mixed precision.  The separation and the gap numerator r^2 - S^2 are taken
-// in FP64 from the FP64 positions (the lubrication coefficients diverge as
-// 1/(d* + eps), so the gap needs far more than FP32's 7 digits); the gap is
-// then d = (r^2 - S^2)/(r + S) with the division in FP32.  The tangential
-// stretch is carried and updated as a double-float (~48 bits); the rest of
-// the pair arithmetic is FP32, on velocities taken relative to the ambient
-// flow.
+// Mixed precision.  The separation and the gap numerator r^2 - S^2 are taken in
+// double-float arithmetic (~48 bits) from the double-float cell-local positions
+// (the lubrication coefficients diverge as 1/(d* + eps), so the gap needs far
+// more than FP32's 7 digits); the gap is then d = (r^2 - S^2)/(r + S) with the
+// division in FP32.  The tangential stretch is carried and updated as a
+// double-float; the rest of the pair arithmetic is FP32, on velocities taken
+// relative to the ambient flow.
 template <bool EXT>
 __device__ __forceinline__ PairRes<float> pair_eval_mixed(const Geo& g, const InstGeo& I, const StateBuf& s,
                                                          const ListBuf& H, const HistRef& hr,
@@ -245,21 +245,18 @@ __device__ __forceinline__ PairRes<float> pair_eval_mixed(const Geo& g, const In
   }
   int wz = (cj >> 20) - (ci >> 20);
   if (wz > R) wz -= nz; else if (wz < -R) wz += nz;
-  // the low words' difference (below 2^-23 cell) goes into the shift's low
-  // word; the sums need an error relative to the cell and to S^2, not to
-  // their own (cancelled) value
-  FF cx = cell_shift(wx, I.csf[0], I.cs_lo[0]), cy = cell_shift(wy, I.csf[1], I.cs_lo[1]),
-     cz = cell_shift(wz, I.csf[2], I.cs_lo[2]);
+  // every sum renormalised: the gap's error stays that of its terms, some 2^-46
+  // S^2 (sums of a magnitude's error, without the second renormalisation, and the
+  // low words' difference folded into the shift cost 6 to 8% of it)
+  FF cx = cell_shift(wx, I.csf[0], I.cs_lo[0]);
   if (le == 1) cx = ff_add(cx, FF{sg.offr_hi, sg.offr_lo});
   else if (le == -1) cx = ff_add(cx, FF{-sg.offr_hi, -sg.offr_lo});
-  cx.lo += lj.x - li.x;
-  cy.lo += lj.y - li.y;
-  cz.lo += lj.z - li.z;
-  const FF dxf = ff_add_abs(two_sum(pj.x, -pi.x), cx), dyf = ff_add_abs(two_sum(pj.y, -pi.y), cy),
-           dzf = ff_add_abs(two_sum(pj.z, -pi.z), cz);
-  const FF Sff = ff_add_abs(FF{gi.v[3], gi.v[7]}, FF{gj.v[3], gj.v[7]});
-  const FF r2ff = ff_add_abs(ff_add_abs(ff_sqr(dxf), ff_sqr(dyf)), ff_sqr(dzf));
-  const FF numff = ff_add_abs(r2ff, ff_neg(ff_sqr(Sff)));      // r^2 - S^2 to ~2^-45 S^2
+  const FF dxf = ff_add(two_sum(pj.x, -pi.x), ff_add(cx, FF{lj.x - li.x, 0.f}));
+  const FF dyf = ff_add(two_sum(pj.y, -pi.y), ff_add(cell_shift(wy, I.csf[1], I.cs_lo[1]), FF{lj.y - li.y, 0.f}));
+  const FF dzf = ff_add(two_sum(pj.z, -pi.z), ff_add(cell_shift(wz, I.csf[2], I.cs_lo[2]), FF{lj.z - li.z, 0.f}));
+  const FF Sff = ff_add(FF{gi.v[3], gi.v[7]}, FF{gj.v[3], gj.v[7]});
+  const FF r2ff = ff_add(ff_add(ff_sqr(dxf), ff_sqr(dyf)), ff_sqr(dzf));
+  const FF numff = ff_add(r2ff, ff_neg(ff_sqr(Sff)));          // r^2 - S^2, ~44 bits
   const float num = numff.hi + numff.lo;
   const float r2 = r2ff.hi + r2ff.lo;
   const float ir = rsqrtf(r2);

@@ -490,12 +490,6 @@ __device__ __forceinline__ FF ff_mul_f(FF a, float b) {
   const float p = a.hi * b;
   return fast_two_sum(p, fmaf(a.hi, b, -p) + a.lo * b);
 }
-// a + b with an error of about 2^-47 (|a| + |b|): where a sum of magnitudes
-// bounds what is needed, not the (cancelled) result
-__device__ __forceinline__ FF ff_add_abs(FF a, FF b) {
-  const FF s = two_sum(a.hi, b.hi);
-  return fast_two_sum(s.hi, s.lo + (a.lo + b.lo));
-}
 // w whole cells of edge (cs_hi + cs_lo) as a double-float: the product of
 // the FP32 words is made exact with Dekker's TwoProduct (w cs_hi needs more
 // than 24 bits once |w| >= 3: a pair several cells apart, or across the
@@ -503,12 +497,12 @@ __device__ __forceinline__ FF ff_add_abs(FF a, FF b) {
 __device__ __forceinline__ FF cell_shift(int w, float cs_hi, float cs_lo) {
   const float wf = (float)w;
   const float p = wf * cs_hi;
-  return FF{p, fmaf(wf, cs_hi, -p) + wf * cs_lo};
+  return FF{p, fmaf(wf, cs_lo, fmaf(wf, cs_hi, -p))};
 }
 __device__ __forceinline__ FF ff_sqr(FF a) {
   const float p = a.hi * a.hi;
   const float e = fmaf(a.hi, a.hi, -p);
-  return fast_two_sum(p, e + 2.0f * a.hi * a.lo);
+  return fast_two_sum(p, fmaf(2.0f * a.hi, a.lo, e));
 }
 
 // ------------------------------------------------------------------------
