@@ -389,6 +389,15 @@ int dss_selftest_conversions(const double *v, int64_t n, double inv, float *hi, 
                              float *split_lo, double *back, int32_t *floor_out, const int32_t *ints,
                              double *ints_out, void *cuda_stream);
 
+/* Self-test of the FP64 quotients that the kernels take from a reciprocal:
+ * quot[k] = a[k] / b[k] by its corrected estimate, and of a pair with centre
+ * distance a[k], radii b[k] together and c[k] = b[k] (gap + eps), the three
+ * reciprocals 1/a, 1/b and b/c (rec, 3n: one plane after another).  Device
+ * memory, n values each; cuda_stream the stream to run on (NULL: legacy
+ * default).  Errors: DSS_ERR_ARG (NULL with n > 0, n < 0), DSS_ERR_CUDA. */
+int dss_selftest_quotients(const double *a, const double *b, const double *c, int64_t n, double *quot,
+                           double *rec, void *cuda_stream);
+
 /* ---- Analysis pass (not part of the time step; each call synchronises) ---- */
 
 /* Rheology of every instance from its bulk stress (Sec. II, after Eq. 9):

@@ -111,6 +111,7 @@ SIGNATURES = {
     "dss_selftest_bounded_wait": (c_int, [c_void_p]),
     "dss_selftest_conversions": (c_int, [_vp, c_int64, c_double, _vp, _vp, _vp, _vp, _vp, _vp, _vp,
                                          c_void_p]),
+    "dss_selftest_quotients": (c_int, [_vp, _vp, _vp, c_int64, _vp, _vp, c_void_p]),
     "dss_rheology": (c_int, [c_void_p, c_int, _vp]),
     "dss_get_images": (c_int, [c_void_p, _vp]),
     "dss_dispersion_mark": (c_int, [c_void_p]),

@@ -105,11 +105,10 @@ __device__ __noinline__ void pair_vjp(const Geo& g, const InstGeo& I, const Pair
   const V3d r = mk3<double>(in.r[0], in.r[1], in.r[2]);
   const double rr = ::sqrt(dot(r, r));
   const double d = rr - S;
-  // 1/r, 1/S and 1/(gap + eps) from one reciprocal (dss_pair_model.cuh)
   const bool clamped = d < 0.0;
   const double num = fma(g.eps, S, clamped ? 0.0 : 2.0 * d);   // S (max(2 d / S, 0) + eps)
-  const double pr = rr * S, inv = 1.0 / (pr * num);
-  const double X = S * (inv * pr), iq = inv * num, iS = iq * rr, ir = iq * S;
+  const PairRecips rc = pair_recips(rr, S, num);
+  const double ir = rc.ir, iS = rc.iS, X = rc.X;
   const V3d n = r * ir;
   const V3d ui = mk3<double>(in.ui[0], in.ui[1], in.ui[2]), uj = mk3<double>(in.uj[0], in.uj[1], in.uj[2]);
   const V3d wi = mk3<double>(in.wi[0], in.wi[1], in.wi[2]), wj = mk3<double>(in.wj[0], in.wj[1], in.wj[2]);
@@ -437,7 +436,8 @@ k_adj_pre(Geo g, const InstGeo* __restrict__ ig, AdjTape t, const double* __rest
   const int id = t.id[s];
   const double a = a_by_id[id];
   const double m = 4.0 / 3.0 * DSS_PI * g.rho * a * a * a;
-  const double im = 1.0 / m, iI = 1.0 / (0.4 * m * a * a);
+  const double Iner = 0.4 * m * a * a;
+  const double im = 1.0 / m, iI = 1.0 / Iner;
   const double hdt = 0.5 * g.dt;
   const double gd = ig[0].gdot;
   double F[3], T[3];
@@ -445,8 +445,8 @@ k_adj_pre(Geo g, const InstGeo* __restrict__ ig, AdjTape t, const double* __rest
   for (int c = 0; c < 3; ++c) {
     const double at = initial ? ab[c * n + id] : ab[c * n + id] + hdt * ub[c * n + id];
     const double bt = initial ? bb[c * n + id] : bb[c * n + id] + hdt * wb[c * n + id];
-    F[c] = at * im;
-    T[c] = bt * iI;
+    F[c] = div_by(at, m, im);
+    T[c] = div_by(bt, Iner, iI);
     Fb[c * n + s] = F[c];
     Tb[c * n + s] = T[c];
   }

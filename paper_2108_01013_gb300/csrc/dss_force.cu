@@ -1024,14 +1024,6 @@ __device__ __forceinline__ void warp_sum_row(const R* __restrict__ row, int cc, 
   }
 }
 
-// a / b from r = 1/b rounded: the quotient estimate a r corrected by its exact
-// remainder (Markstein): the rounded quotient, three operations instead of a
-// division's ten on GB300's narrow FP64 pipe.
-__device__ __forceinline__ double div_by(double a, double b, double r) {
-  const double q = a * r;
-  return fma(fma(-q, b, a), r, q);
-}
-
 // Total force and torque on particle j (its own pair sum, its partner
 // records, Stokes drag), then the accelerations and, in a step, the velocity
 // half-kick of Eq. 15d.  Returns true when the sums are not finite (the
@@ -1338,6 +1330,19 @@ k_long_rows(int n, int M, float* bw, int* bw_count, const DevStatus* st) {
   }
 }
 
+// Self-test of the quotients from a reciprocal (div_by, pair_recips).
+__global__ void k_selftest_quotients(const double* __restrict__ a, const double* __restrict__ b,
+                                     const double* __restrict__ c, int64_t n, double* __restrict__ quot,
+                                     double* __restrict__ rec) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+    quot[k] = div_by(a[k], b[k], __drcp_rn(b[k]));
+    const PairRecips q = pair_recips(a[k], b[k], c[k]);
+    rec[k] = q.ir;
+    rec[n + k] = q.iS;
+    rec[2 * n + k] = q.X;
+  }
+}
+
 // Pairs of a list as (lo id, hi id) in owner order (for dss_get_pairs).
 __global__ void k_pairs_out(Geo g, ListBuf W, long long* __restrict__ out) {
   const int n = g.n;
@@ -1438,4 +1443,14 @@ void launch_forces(dss_handle* h, int stbuf, int work_list, int hist_list, int a
 
 void launch_pairs_out(dss_handle* h, int list, long long* out) {
   k_pairs_out<<<pair_grid_blocks(h), kPairThreads, 0, h->stream>>>(h->g, h->lb[list], out);
+}
+
+extern "C" int dss_selftest_quotients(const double* a, const double* b, const double* c, int64_t n, double* quot,
+                                      double* rec, void* cuda_stream) {
+  if (n < 0 || (n > 0 && (!a || !b || !c || !quot || !rec))) return DSS_ERR_ARG;
+  if (n == 0) return DSS_OK;
+  cudaStream_t s = (cudaStream_t)cuda_stream;
+  k_selftest_quotients<<<(int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096), 256, 0, s>>>(a, b, c, n, quot, rec);
+  if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return DSS_ERR_CUDA;
+  return DSS_OK;
 }
