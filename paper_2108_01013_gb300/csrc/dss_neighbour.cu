@@ -415,7 +415,7 @@ struct SegShared {
   int cnt[2][kRows][32];      // pairs of each owner in each row (near ones << 16: SPLIT)
   int4 par[kRows];            // rows: bin of their x = 0, x of their first cell, cells, image across y
   int seg[4];                 // first bin, cells, part, first owner
-  int far;                    // the group to take after the block's own owners (-1: none is left)
+  int far;                    // ST_LONG, then the group to take after the block's own owners (-1: none is left)
 };
 
 // The segment from x0 on in a row of cells: its half stencil's rows, a lane each
@@ -725,6 +725,7 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
   const int inst = ONE ? 0 : blk_inst[blockIdx.x];
   const InstGeo& I = ONE ? I1 : ig[inst];
   const StepGeo sg = sgk[inst];
+  if (threadIdx.x == 32) sh.far = st->w[ST_LONG];
   if (r == 0) {
     // the first warp finds the segment
     unsigned item = blockIdx.x - (ONE ? 0 : I.enum_blk);
@@ -740,7 +741,7 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
   }
   __syncthreads();
   search_segment<ECH, SPLIT, NARROW>(sh, g, I, sg, s, posf, cellid, cell_start, list, count, nnear, R, st, q, lane, r, -1);
-  if (st->w[ST_LONG])
+  if (sh.far)
     search_far<ECH, SPLIT, ONE, NARROW>(sh, g, I1, ig, sgk, s, posf, cellid, cell_start, list, count, nnear, R, st, q);
 }
 
