@@ -249,7 +249,8 @@ int dss_get_pairs(dss_handle *h, int64_t *lohi, int64_t cap, int64_t *count);
 /* One force evaluation at the current state with the committed history,
  * without advancing or committing: total force F and torque T on every
  * particle (pairs + Stokes drag), in id order; either may be NULL.  Also
- * sets the stress read by dss_stress. */
+ * sets the stress read by dss_stress.  After an error the contents of F and T
+ * are undefined. */
 int dss_force_eval(dss_handle *h, double *F, double *T);
 
 /* Advances nsteps time steps (Eq. 15, 16): predictor and wrap, counting
@@ -374,6 +375,12 @@ int dss_adjoint(dss_handle *h, int64_t nsteps, int32_t ckpt_every, const double 
  * mean the wait did not notice).  The context stays usable.  cuda_stream:
  * stream to run on (NULL: legacy default stream); synchronises it. */
 int dss_selftest_bounded_wait(void *cuda_stream);
+
+/* Whether a kernel on `device` accesses in place a buffer of doubles at p that
+ * cudaPointerGetAttributes reports as memory_type (cudaMemoryType) of
+ * memory_device: 1 for aligned memory of the same device; everything else goes
+ * through a copy (0).  Host-only, needs no GPU. */
+int dss_selftest_reach(int32_t memory_type, int32_t memory_device, int32_t device, const void *p);
 
 /* Self-test of the conversions the sort kernels take by integer operations
  * on the IEEE-754 bit patterns instead of GB300's narrow FP64 pipe; each must

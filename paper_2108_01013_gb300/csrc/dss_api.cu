@@ -321,26 +321,36 @@ __global__ void k_state_in(int n, Src5 src, StateBuf s, const double* __restrict
   s.id[i] = i;
 }
 
-// Address through which a kernel may access a caller's buffer: device and
-// managed memory as is, pinned host memory through its mapped device
-// pointer; nullptr for pageable host memory (copy engines only).
-const void* device_view(const void* p) {
+// Whether a kernel of the handle's device may access a caller's buffer of
+// doubles: memory of that device, at a double's alignment. Memory of another one
+// (an illegal address without peer access) and odd addresses are copied by the
+// copy engines instead, which take both.
+bool kernel_reaches(int type, int at_device, int device, const void* p) {
+  return type == cudaMemoryTypeDevice && at_device == device && reinterpret_cast<uintptr_t>(p) % sizeof(double) == 0;
+}
+
+// Address through which a kernel may access a caller's buffer: device memory
+// (kernel_reaches) and managed memory as is, pinned host memory through its
+// mapped device pointer; nullptr otherwise (copy engines only).
+const void* device_view(const dss_handle* h, const void* p) {
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
   }
-  if (at.type == cudaMemoryTypeDevice) return p;
-  if ((at.type == cudaMemoryTypeHost || at.type == cudaMemoryTypeManaged) && at.devicePointer)
+  if (at.type == cudaMemoryTypeDevice) return kernel_reaches(at.type, at.device, h->device, p) ? p : nullptr;
+  if ((at.type == cudaMemoryTypeHost || at.type == cudaMemoryTypeManaged) && at.devicePointer &&
+      reinterpret_cast<uintptr_t>(p) % sizeof(double) == 0)
     return at.devicePointer;
   return nullptr;
 }
 
-bool is_device(const void* p) {
+// Whether a kernel writes a caller's buffer in place.
+bool in_place(const dss_handle* h, const void* p) {
   cudaPointerAttributes at;
-  const bool dev = cudaPointerGetAttributes(&at, p) == cudaSuccess && at.type == cudaMemoryTypeDevice;
+  const bool ok = cudaPointerGetAttributes(&at, p) == cudaSuccess && kernel_reaches(at.type, at.device, h->device, p);
   cudaGetLastError();
-  return dev;
+  return ok;
 }
 
 // Tile 1 of a look-back whose tile 0 never publishes: the wait must give up.
@@ -1050,11 +1060,11 @@ int get_state_enqueue(dss_handle* h, double* const out[5]) {
   for (int k = 0; k < 5; ++k) {
     direct.d[k] = staged.d[k] = views.d[k] = nullptr;
     if (!out[k]) continue;
-    if (is_device(out[k])) {
+    if (in_place(h, out[k])) {
       direct.d[k] = out[k];
     } else {
       staged.d[k] = h->stage + (size_t)k * 3 * n;
-      views.d[k] = static_cast<double*>(const_cast<void*>(device_view(out[k])));
+      views.d[k] = static_cast<double*>(const_cast<void*>(device_view(h, out[k])));
     }
   }
   Dst5 all = direct;
@@ -1071,7 +1081,7 @@ int get_state_enqueue(dss_handle* h, double* const out[5]) {
       dst_c.d[k] = views.d[k];
       any_view = true;
     } else {
-      CK(cudaMemcpyAsync(out[k], staged.d[k], sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, h->stream));
+      CK(cudaMemcpyAsync(out[k], staged.d[k], sizeof(double) * 3 * n, cudaMemcpyDefault, h->stream));
     }
   }
   if (any_view) k_copy5<<<std::min((3 * n + 255) / 256, 8 * h->sms), 256, 0, h->stream>>>(3 * (int64_t)n, src_c, dst_c);
@@ -1141,8 +1151,8 @@ int dss_force_eval(dss_handle* h, double* F, double* T) {
   ENTER(h);
   const size_t b3 = sizeof(double) * 3 * (size_t)h->n;
   // (device outputs are written by the kernel itself)
-  double* const Fd = F && !is_device(F) ? h->io3 : F;
-  double* const Td = T && !is_device(T) ? h->io3b : T;
+  double* const Fd = F && !in_place(h, F) ? h->io3 : F;
+  double* const Td = T && !in_place(h, T) ? h->io3b : T;
   const int list = 1 - h->hist;
   seq_sort_enum(h, false, 0);
   h->cur = 1 - h->cur;
@@ -1641,10 +1651,10 @@ int load_state_enqueue(dss_handle* h, const double* const in[5]) {
     // host buffers go through the staging area with the copy engine first
     Src5 src;
     for (int k = 0; k < 5; ++k) {
-      src.d[k] = static_cast<const double*>(device_view(in[k]));
+      src.d[k] = static_cast<const double*>(device_view(h, in[k]));
       if (!src.d[k]) {
         double* st = h->stage + (size_t)k * 3 * h->n;
-        CK(cudaMemcpyAsync(st, in[k], b, cudaMemcpyHostToDevice, h->stream));
+        CK(cudaMemcpyAsync(st, in[k], b, cudaMemcpyDefault, h->stream));
         src.d[k] = st;
       }
     }
@@ -2204,6 +2214,10 @@ int dss_adjoint(dss_handle* h, int64_t nsteps, int32_t ckpt_every, const double*
     if (J) *J = Jacc;
     return snap_restore(h, ck_end);
   });
+}
+
+int dss_selftest_reach(int32_t memory_type, int32_t memory_device, int32_t device, const void* p) {
+  return kernel_reaches(memory_type, memory_device, device, p) ? 1 : 0;
 }
 
 int dss_selftest_bounded_wait(void* cuda_stream) {
