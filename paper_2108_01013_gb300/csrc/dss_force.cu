@@ -635,7 +635,7 @@ k_pairs_pb(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sg
   dep_wait();
   using R = typename std::conditional<MIXED, float, double>::type;
   constexpr int NV = pb_slot<PERS>();
-  if (dev_err(st)) return;
+  if (warp_err(st)) return;   // (a full partner row sets one while blocks start)
   R* __restrict__ own = static_cast<R*>(own_v);
   R* __restrict__ own_s = static_cast<R*>(own_s_v);
   R* __restrict__ carry = static_cast<R*>(carry_v);
@@ -1262,9 +1262,10 @@ k_gather(Geo g, const InstGeo* __restrict__ ig, StateBuf s, const void* __restri
   // would write can be the committed one.  Every block still reaches the
   // counter below.
   __shared__ int s_slot[kThreads / 32][MIXED ? 32 : kHeavyWin];
-  // (the stress blocks meet at barriers and decide together; elsewhere a warp
-  // for itself)
-  bool err0 = dev_err(st) != 0;
+  // (the stress blocks meet at barriers and decide together; elsewhere a warp for
+  // itself, all its lanes alike: a non-finite sum sets the error while blocks
+  // start)
+  bool err0 = warp_err(st);
   if (blockIdx.x < (unsigned)g.K) err0 = __syncthreads_or(err0) != 0;
   bool fence = false;
   if (!err0) {

@@ -144,6 +144,10 @@ inline void launch_dep(void (*kernel)(K...), int64_t grid, int block, cudaStream
 __device__ __forceinline__ int dev_err(const DevStatus* s) {
   return *((volatile const int*)&s->w[ST_ERR]);
 }
+// The same, one answer for the warp (all 32 lanes call it): in kernels whose own
+// blocks may set an error while others start, and whose warps vote and shuffle
+// after the test.
+__device__ __forceinline__ bool warp_err(const DevStatus* s) { return __any_sync(0xffffffffu, dev_err(s) != 0); }
 __device__ __forceinline__ void set_err(DevStatus* s, int code) {
   atomicCAS(&s->w[ST_ERR], 0, code);
 }

@@ -1,0 +1,38 @@
+"""Orders that the step's kernels have to state in their source, since no test on
+the GPU can be relied on to show their absence."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2108_01013_gb300", "csrc")
+
+
+def source(name):
+    text = open(os.path.join(CSRC, name)).read()
+    return re.sub(r"//[^\n]*", "", text)
+
+
+def kernels():
+    """{name: body} of every __global__ function."""
+    out = {}
+    for name in sorted(os.listdir(CSRC)):
+        text = source(name)
+        for m in re.finditer(r"__global__[^;{]*?\b(k_\w+)\s*\(", text):
+            i = text.index("{", m.end())
+            depth, j = 1, i + 1
+            while depth:
+                depth += {"{": 1, "}": -1}.get(text[j], 0)
+                j += 1
+            out[m.group(1)] = text[i + 1:j - 1]
+    return out
+
+
+ALL = kernels()
+
+
+def test_error_read_alike_by_a_warp_where_blocks_may_set_it():
+    """The kernels that raise errors of their own (a full row of partner records,
+    sums that are not finite) and vote or shuffle over full warps afterwards."""
+    for k in ("k_pairs_pb", "k_gather"):
+        head = ALL[k][:1600]
+        assert "warp_err(st)" in head
+        assert not re.search(r"[^_]dev_err\(st\)\s*(\)|!=)", head.split("warp_err")[0]), k
