@@ -525,9 +525,11 @@ struct __align__(32) Rec8 {
 // 108, of 100k, whose arrays sit in the L2, 26.5 both.
 __host__ __device__ constexpr int64_t rec_geometry(int64_t i) { return 2 * i; }
 __host__ __device__ constexpr int64_t rec_motion(int64_t i) { return 2 * i + 1; }
+// (volatile: it stays behind the kernel's wait for its predecessor, dep_wait,
+// also where its address depends on the thread alone)
 __device__ __forceinline__ Rec8 load_rec(const Rec8* p) {
   Rec8 r;
-  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+  asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
       : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3]), "=f"(r.v[4]), "=f"(r.v[5]), "=f"(r.v[6]),
         "=f"(r.v[7])
       : "l"(p));

@@ -36,3 +36,29 @@ def test_error_read_alike_by_a_warp_where_blocks_may_set_it():
         head = ALL[k][:1600]
         assert "warp_err(st)" in head
         assert not re.search(r"[^_]dev_err\(st\)\s*(\)|!=)", head.split("warp_err")[0]), k
+
+
+def test_kernels_wait_before_they_read():
+    """Every kernel that looks at the step's error word starts by waiting for its
+    predecessor (programmatic dependent launch): first statement but for shared
+    arrays and names."""
+    seen = 0
+    for k, body in ALL.items():
+        if not re.search(r"dev_err\(|warp_err\(", body):
+            continue
+        head = body.split("dep_wait();")[0]
+        assert "dep_wait();" in body, k
+        assert not re.sub(r"(__shared__|constexpr|using)[^;]*;", "", head).strip(), (k, head)
+        seen += 1
+    assert seen >= 10
+
+
+def test_loads_in_assembly_stay_behind_the_wait():
+    """A load written in assembly is not moved across the wait only when it is
+    volatile, as the wait is."""
+    loads = 0
+    for name in sorted(os.listdir(CSRC)):
+        for m in re.finditer(r"\basm\b(\s+volatile)?\s*\(\s*\"ld\.", source(name)):
+            loads += 1
+            assert m.group(1), (name, source(name)[m.start():m.start() + 60])
+    assert loads >= 3
