@@ -382,6 +382,13 @@ int dss_selftest_bounded_wait(void *cuda_stream);
  * through a copy (0).  Host-only, needs no GPU. */
 int dss_selftest_reach(int32_t memory_type, int32_t memory_device, int32_t device, const void *p);
 
+/* Forces the enumeration's search of a handle with a state (1: walked by owner,
+ * 4: staged by segments of cells, 0: the built-in rule's again), as
+ * dss_autotune_kernels does with the faster one; *ran (may be NULL) receives
+ * the search that now runs (size classes are always walked).  For tests that
+ * compare the two.  Errors: DSS_ERR_ARG, DSS_ERR_STATE, DSS_ERR_CUDA. */
+int dss_selftest_search(dss_handle *h, int32_t which, int32_t *ran);
+
 /* Self-test of the conversions the sort kernels take by integer operations
  * on the IEEE-754 bit patterns instead of GB300's narrow FP64 pipe; each must
  * equal the hardware conversion bit for bit.  For k < n: hi[k] =

@@ -109,6 +109,7 @@ SIGNATURES = {
     "dss_autotune": (c_int, [c_void_p, c_int32, c_int32, _dp, _dp, _dp]),
     "dss_autotune_kernels": (c_int, [c_void_p, c_int32, _dp, _ip]),
     "dss_selftest_bounded_wait": (c_int, [c_void_p]),
+    "dss_selftest_search": (c_int, [c_void_p, c_int32, _ip]),
     "dss_selftest_reach": (c_int, [c_int32, c_int32, c_int32, c_void_p]),
     "dss_selftest_conversions": (c_int, [_vp, c_int64, c_double, _vp, _vp, _vp, _vp, _vp, _vp, _vp,
                                          c_void_p]),

@@ -2216,6 +2216,23 @@ int dss_adjoint(dss_handle* h, int64_t nsteps, int32_t ckpt_every, const double*
   });
 }
 
+int dss_selftest_search(dss_handle* h, int32_t which, int32_t* ran) {
+  return guard([&]() -> int {
+    if (!h || (which != 0 && which != 1 && which != 4)) return DSS_ERR_ARG;
+    if (!h->have_state) return DSS_ERR_STATE;
+    ENTER(h);
+    CK(cudaStreamSynchronize(h->stream));
+    h->tune_enum_unr = which;
+    drop_graphs(h);
+    const int r = plan_enumeration(h);
+    if (r) return r;
+    CK(cudaMemcpyAsync(h->ig, h->ig_host, sizeof(InstGeo) * h->K, cudaMemcpyHostToDevice, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+    if (ran) *ran = h->enum_walk ? 1 : 4;
+    return DSS_OK;
+  });
+}
+
 int dss_selftest_reach(int32_t memory_type, int32_t memory_device, int32_t device, const void* p) {
   return kernel_reaches(memory_type, memory_device, device, p) ? 1 : 0;
 }
