@@ -300,9 +300,11 @@ int dss_save(dss_handle *h, void *buf, size_t *len);
 
 /* Restores a checkpoint written by dss_save into a handle created with the
  * same instances, boxes, shear rates, dashpots and model constants
- * (DSS_ERR_ARG otherwise, or for a damaged buffer).  Because the library's
- * sorted order depends only on positions and ids, the resumed run repeats the
- * uninterrupted one bit for bit.  Synchronises the stream. */
+ * (DSS_ERR_ARG otherwise, or for a damaged buffer).  The library's sorted order
+ * depends only on positions and ids (on the same cell edge), and the checkpoint
+ * carries the kernel shapes of the handle that wrote it (dss_autotune_kernels),
+ * which the handle takes over: the resumed run repeats the uninterrupted one bit
+ * for bit.  Synchronises the stream. */
 int dss_load(dss_handle *h, const void *buf, size_t len);
 
 /* Chooses the cell edge from timed trials.  Candidate k uses a cell edge of
@@ -326,7 +328,10 @@ int dss_autotune(dss_handle *h, int32_t trial_steps, int32_t ncand, const double
  * combinations runs 2 + trial_steps steps from a checkpoint of the current
  * state; the fastest is kept and the state restored.  ms_per_step (host, 4 doubles, may be NULL): ms per step of
  * (3 blocks, 1), (3, 4), (4, 1), (4, 4); choice (host, 2 ints, may be NULL):
- * the kept (blocks per SM, search: 1 walked by owner, 4 staged).  Errors: DSS_ERR_ARG
+ * the kept (blocks per SM, search: 1 walked by owner, 4 staged).  The shapes
+ * fix the order in which a row's pairs (on crowded grids) and the stress are
+ * summed: runs of different shapes agree to rounding, those of one repeat each
+ * other bit for bit.  Errors: DSS_ERR_ARG
  * (trial_steps < 1), DSS_ERR_STATE, and any error of a trial step (the
  * built-in rule is kept then). */
 int dss_autotune_kernels(dss_handle *h, int32_t trial_steps, double *ms_per_step, int32_t *choice);

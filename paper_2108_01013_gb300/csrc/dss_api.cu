@@ -1731,6 +1731,19 @@ struct CkptHeader {
   uint64_t config;
 };
 constexpr char kMagic[8] = {'D', 'S', 'S', 'C', 'K', 'P', 'T', '1'};
+// The version word: the format (1) and the kernel shapes chosen by
+// dss_autotune_kernels (search << 8, pair blocks << 12; 0: the built-in rule's),
+// which fix the order of the sums and so belong to what a resumed run repeats.
+constexpr uint32_t kVersion = 1;
+uint32_t ckpt_version(const dss_handle* h) {
+  return kVersion | (uint32_t)h->tune_enum_unr << 8 | (uint32_t)h->tune_pairs_minb << 12;
+}
+bool ckpt_shapes(uint32_t version, int& search, int& minb) {
+  search = (int)(version >> 8 & 15);
+  minb = (int)(version >> 12 & 15);
+  return (version & 255) == kVersion && version >> 16 == 0 && (search == 0 || search == 1 || search == 4) &&
+         (minb == 0 || minb == 3 || minb == 4);
+}
 
 uint64_t fnv1a(uint64_t hsh, const void* p, size_t len) {
   const unsigned char* b = static_cast<const unsigned char*>(p);
@@ -1803,7 +1816,7 @@ int dss_save(dss_handle* h, void* buf, size_t* len) {
     CkptHeader hd;
     memset(&hd, 0, sizeof(hd));
     memcpy(hd.magic, kMagic, 8);
-    hd.version = 1;
+    hd.version = ckpt_version(h);
     hd.K = h->K;
     hd.n = n;
     hd.nhist = nh;
@@ -1837,12 +1850,14 @@ int dss_save(dss_handle* h, void* buf, size_t* len) {
   });
 }
 
-int dss_load(dss_handle* h, const void* buf, size_t len) {
+// dss_load; shapes: with the kernel shapes the checkpoint was written with.
+static int load_checkpoint(dss_handle* h, const void* buf, size_t len, bool shapes) {
   return guard([&]() -> int {
     if (!h || !buf || len < sizeof(CkptHeader)) return DSS_ERR_ARG;
     CkptHeader hd;
     memcpy(&hd, buf, sizeof(hd));
-    if (memcmp(hd.magic, kMagic, 8) != 0 || hd.version != 1 || hd.K != h->K || hd.n != h->n ||
+    int search = 0, minb = 0;
+    if (memcmp(hd.magic, kMagic, 8) != 0 || !ckpt_shapes(hd.version, search, minb) || hd.K != h->K || hd.n != h->n ||
         hd.nhist < 0 || hd.nstep < 0 || hd.mean_steps < 0 || hd.config != config_hash(h))
       return DSS_ERR_ARG;
     const int64_t n = hd.n, nh = hd.nhist;
@@ -1871,6 +1886,10 @@ int dss_load(dss_handle* h, const void* buf, size_t len) {
     std::vector<double> sig(18 * (size_t)h->K);
     memcpy(sig.data(), in, sizeof(double) * 18 * h->K);
     const double* x = st.data();
+    if (shapes) {
+      h->tune_enum_unr = search;
+      h->tune_pairs_minb = minb;
+    }
     int r = dss_set_state(h, x, x + 15 * n, nullptr, x + 3 * n, x + 6 * n, x + 9 * n, x + 12 * n, hd.nstep);
     if (r) return r;
     if ((r = dss_set_history_rolling(h, nh, keys.data(), xi.data(), rolling ? xr.data() : nullptr))) return r;
@@ -1882,6 +1901,8 @@ int dss_load(dss_handle* h, const void* buf, size_t len) {
     return DSS_OK;
   });
 }
+
+int dss_load(dss_handle* h, const void* buf, size_t len) { return load_checkpoint(h, buf, len, true); }
 
 int dss_autotune(dss_handle* h, int32_t trial_steps, int32_t ncand, const double* factors,
                  double* ms_per_step, double* cell_size) {
@@ -1963,7 +1984,7 @@ int dss_autotune_kernels(dss_handle* h, int32_t trial_steps, double* ms_per_step
         h->tune_enum_unr = kUnr[b];
         drop_graphs(h);
         double ms = INFINITY;
-        r = dss_load(h, ck.data(), len);
+        r = load_checkpoint(h, ck.data(), len, false);
         if (r == DSS_OK) r = dss_step(h, 2);
         double t = 0.0;
         if (r == DSS_OK) r = dss_step(h, trial_steps);
@@ -1971,7 +1992,7 @@ int dss_autotune_kernels(dss_handle* h, int32_t trial_steps, double* ms_per_step
         if (r != DSS_OK) {
           h->tune_pairs_minb = h->tune_enum_unr = 0;
           drop_graphs(h);
-          dss_load(h, ck.data(), len);
+          load_checkpoint(h, ck.data(), len, false);
           h->profiling = prof_was;
           return r;
         }
@@ -1985,7 +2006,7 @@ int dss_autotune_kernels(dss_handle* h, int32_t trial_steps, double* ms_per_step
     h->tune_pairs_minb = bm;
     h->tune_enum_unr = bu;
     drop_graphs(h);
-    r = dss_load(h, ck.data(), len);
+    r = load_checkpoint(h, ck.data(), len, false);
     h->profiling = prof_was;
     if (r) return r;
     if (choice) {
