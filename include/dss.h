@@ -281,7 +281,9 @@ int dss_set_profiling(dss_handle *h, int on);
  * number of profiled steps. */
 int dss_get_profile(dss_handle *h, double *ms, int64_t *steps);
 
-/* Name of profiled kernel k (0 <= k < DSS_PROF_KERNELS), "" otherwise. */
+/* Name of profiled kernel k (0 <= k < DSS_PROF_KERNELS), "" otherwise.  The
+ * batched instances' stresslet sums and the crowded grids' long rows, kernels of
+ * their own ahead of the corrector, count with it (k_gather). */
 const char *dss_profile_name(int k);
 
 /* GPU time in milliseconds of the step graphs of the last dss_step call

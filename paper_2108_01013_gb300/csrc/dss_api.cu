@@ -1697,9 +1697,8 @@ int dss_get_profile(dss_handle* h, double* ms, int64_t* steps) {
 }
 
 const char* dss_profile_name(int k) {
-  static const char* names[DSS_PROF_KERNELS] = {"k_key_hist", "k_scan_cells", "k_scatter",
-                                                  "k_rank_gather", "k_enumerate", "k_pairs",
-                                                  "k_gather"};
+  static const char* names[DSS_PROF_KERNELS] = {"k_key_hist", "k_scan", "k_rank_gather", "k_enumerate",
+                                                  "k_rows", "k_pairs", "k_gather"};
   return (k >= 0 && k < DSS_PROF_KERNELS) ? names[k] : "";
 }
 

@@ -966,7 +966,7 @@ void launch_enumerate(dss_handle* h, int stbuf, int dst_list, int adv) {
   (void)adv;
   ListBuf& L = h->lb[dst_list];
   const Geo& g = h->g;
-  prof_mark(h, 4);
+  prof_mark(h, 3);
   // FP32 cutoffs.  The electro-chemical range beats the pair-mean lubrication
   // cutoff for every pair when it beats the largest; only between the two do
   // both enter the candidate test.
@@ -997,6 +997,7 @@ void launch_enumerate(dss_handle* h, int stbuf, int dst_list, int adv) {
     launch_dep(ks, blocks, 32 * kRows, h->stream, g, h->ig_host[0], h->ig, h->sg, h->st[stbuf], h->posf, h->cellid,
                                              h->cell_start, L.list, L.count, h->offs, h->enum_inst, R, h->status, q);
   }
+  prof_mark(h, 4);
   auto kr = split ? k_rows<true, 64> : k_rows<false, 256>;
   launch_dep(kr, ((int)h->n + tile - 1) / tile, kRowThreads, h->stream, (int)h->n, g.M, g.Ms, g.pcap, h->st[stbuf].id, L,
              h->offs, h->bw_count, h->cellid, h->cell_more, R, h->status);

@@ -403,7 +403,6 @@ void launch_sort(dss_handle* h, bool predict, int src, int dst, bool keyed) {
   prof_mark(h, 1);
   launch_cell_scan(h);
   prof_mark(h, 2);
-  prof_mark(h, 3);
   const int clear = scan_tiles_for(h->g.ncell) <= kScanTiles ? h->g.ncell : 0;
   const SortOut so = sort_out(h);
   if (h->g.wave)

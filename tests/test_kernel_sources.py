@@ -62,3 +62,18 @@ def test_loads_in_assembly_stay_behind_the_wait():
             loads += 1
             assert m.group(1), (name, source(name)[m.start():m.start() + 60])
     assert loads >= 3
+
+
+def test_profiled_kernels_exist():
+    """The names that the per-kernel times go by are those of kernels in the sources
+    (or begin theirs), and the byte tables of the benchmark go by the same."""
+    import bench
+    from paper_2108_01013_gb300 import _native
+    _native.build()
+    lib = _native.load()
+    names = [lib.dss_profile_name(k).decode() for k in range(_native.PROF_KERNELS)]
+    assert names == list(bench.METHOD_BYTES) == list(bench.IMPL_BYTES)
+    for name in names:
+        assert any(k.startswith(name) for k in ALL), name
+    # a single step launches each once: the headline's count
+    assert bench.KERNELS_PER_STEP == len(names)
