@@ -1133,9 +1133,13 @@ int dss_get_pairs(dss_handle* h, int64_t* lohi, int64_t cap, int64_t* count) {
     std::vector<long long> hp(2 * (size_t)P);
     CK(cudaMemcpyAsync(hp.data(), dev, sizeof(long long) * 2 * P, cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
-    std::vector<std::pair<long long, long long>> v(P);
-    for (int p = 0; p < P; ++p) v[p] = {hp[2 * p], hp[2 * p + 1]};
+    std::vector<std::pair<long long, long long>> v;
+    v.reserve(P);
+    for (int p = 0; p < P; ++p)
+      if (hp[2 * p] >= 0) v.push_back({hp[2 * p], hp[2 * p + 1]});
     std::sort(v.begin(), v.end());
+    P = (int)v.size();
+    *count = P;
     int64_t m = std::min<int64_t>(cap, P);
     for (int64_t p = 0; p < m; ++p) {
       lohi[2 * p] = v[p].first;

@@ -1344,7 +1344,9 @@ __global__ void k_selftest_quotients(const double* __restrict__ a, const double*
   }
 }
 
-// Pairs of a list as (lo id, hi id) in owner order (for dss_get_pairs).
+// Pairs of a list as (lo id, hi id) in owner order (for dss_get_pairs).  A list
+// whose build ended in an error (rows that overflow) has the offsets of an older
+// one where the row pass stopped short: a place outside its row gives (-1, -1).
 __global__ void k_pairs_out(Geo g, ListBuf W, long long* __restrict__ out) {
   const int n = g.n;
   const int P = W.start[n];
@@ -1354,7 +1356,12 @@ __global__ void k_pairs_out(Geo g, ListBuf W, long long* __restrict__ out) {
       int mid = (lo + hi) >> 1;
       if (W.start[mid] <= p) lo = mid; else hi = mid;
     }
-    const int j = W.list[(int64_t)lo * g.Ms + (p - W.start[lo])];
+    const int k = p - W.start[lo];
+    if (k < 0 || k >= min(W.count[lo], g.M)) {
+      out[2 * (int64_t)p] = out[2 * (int64_t)p + 1] = -1;
+      continue;
+    }
+    const int j = W.list[(int64_t)lo * g.Ms + k];
     const int a = W.id_of_slot[lo], b = W.id_of_slot[j];
     out[2 * (int64_t)p] = a < b ? a : b;
     out[2 * (int64_t)p + 1] = a < b ? b : a;

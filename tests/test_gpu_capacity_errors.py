@@ -65,3 +65,27 @@ def test_pair_arrays_still_grow(env):
         s.close()
     for a, b in zip(*out):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("n", [3000, 400_000])
+def test_pairs_after_rows_that_overflow(env, n):
+    """Reading a list whose build was refused is safe: what it gives are pairs of
+    ids, no more than the rows hold, and the handle goes on."""
+    dss = env["dss"]
+    rng = np.random.default_rng(n)
+    L = (n * 12.0) ** (1.0 / 3.0)
+    x = rng.uniform(0.0, L, size=(3, n))
+    z = np.zeros_like(x)
+    s = dss.Suspension(x, np.ones(n), [L] * 3, dss.default_params(capacity_M=40), alpha_lin=z, alpha_ang=z)
+    s.neighbour_build()
+    full = s.pairs()
+    s.close()
+    s = dss.Suspension(x, np.ones(n), [L] * 3, dss.default_params(capacity_M=1), alpha_lin=z, alpha_ang=z)
+    for _ in range(3):
+        with pytest.raises(dss.DssError) as e:
+            s.neighbour_build()
+        assert e.value.code == -3
+        p = s.pairs()
+        assert len(p) <= n and (p >= 0).all() and (p < n).all() and (p[:, 0] < p[:, 1]).all()
+    assert len(full) > n
+    s.close()
