@@ -48,7 +48,9 @@ void free_buffers(dss_handle* h) {
   h->pred = nullptr;
   dfree(h->xc); dfree(h->mark);
   h->xc = nullptr; h->mark = nullptr; h->marked = false;
-  dfree(h->cell_count); dfree(h->tile_count); h->tile_count = nullptr; dfree(h->cell_ids); h->cell_ids = nullptr; dfree(h->cell_more); h->cell_more = nullptr; dfree(h->cell_start); dfree(h->tmp); dfree(h->spart);
+  dfree(h->cell_count); dfree(h->cell_start); dfree(h->tmp); dfree(h->spart);
+  dfree(h->tile_count); dfree(h->cell_ids); dfree(h->cell_more);
+  h->tile_count = nullptr; h->cell_ids = nullptr; h->cell_more = nullptr;
   dfree(h->own); dfree(h->bw_count); dfree(h->bw_rec); dfree(h->carry); dfree(h->own_s);
   h->own = nullptr; h->bw_count = nullptr; h->bw_rec = nullptr; h->carry = nullptr; h->own_s = nullptr;
   h->pb_blocks = 0;
@@ -144,7 +146,6 @@ int alloc_pair_buffers(dss_handle* h, int64_t pcap, bool keep_hist) {
   if ((r = dalloc(h, &sp, 9 * (size_t)pb))) return r;
   dfree(h->spart);
   h->spart = sp;
-  h->spart_blocks = pb;
   drop_graphs(h);
   return DSS_OK;
 }
@@ -172,7 +173,8 @@ int alloc_buffers(dss_handle* h) {
   if ((r = dalloc(h, &h->posf, n)) || (r = dalloc(h, &h->cellid, n)) || (r = dalloc(h, &h->perm, n)) ||
       (r = dalloc(h, &h->pred, 6 * n)) || (r = dalloc(h, &h->xc, n)) ||
       (r = dalloc(h, &h->key, n)) || (r = dalloc(h, &h->offs, n)) ||
-      (r = dalloc(h, &h->cell_count, (size_t)h->g.ncell)) || (r = dalloc(h, &h->tile_count, (size_t)kTileCopies * kScanTiles)) ||
+      (r = dalloc(h, &h->cell_count, (size_t)h->g.ncell)) ||
+      (r = dalloc(h, &h->tile_count, (size_t)kTileCopies * kScanTiles)) ||
       (r = dalloc(h, &h->cell_start, (size_t)h->g.ncell + 1)) || (r = dalloc(h, &h->tmp, n)) ||
       (r = dalloc(h, &h->io3, 3 * n)) || (r = dalloc(h, &h->io3b, 3 * n)) ||
       (r = dalloc(h, &h->stage, 15 * n)) ||

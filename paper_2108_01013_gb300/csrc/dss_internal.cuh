@@ -381,11 +381,6 @@ __device__ __forceinline__ void stencil_shift(const InstGeo& g, int ox, int oy, 
   cz = (float)oz * g.csf[2];
 }
 
-__device__ __forceinline__ float pair_delta_f(const Geo& g, float ai, float aj) {
-  if (g.mode == 1) return (float)(g.delta * g.a0);
-  return (float)g.delta * (ai + aj) * 0.5f;
-}
-
 // ------------------------------------------------------------------------
 // Decoupled look-back for single-pass scans (tiles taken in launch order
 // through an atomic ticket, so every predecessor is already running).  One
@@ -725,13 +720,12 @@ struct dss_handle {
                      // from the previous warp and into the next: force and torque (6 + 6;
                      // batched instances also the stresslet, 15 + 15)
   void* own_s;       // batched instances: 9n, each owner's stresslet sum (Eq. 9)
-  int pb_blocks;     // blocks of the pair-balanced pair kernel (0: owner rows)
+  int pb_blocks;     // blocks of the pair kernel
   int* bw_count;     // n: records appended to each particle's partner row
   void* bw_rec;      // n*M slots of 8 values: partner force (3), torque (3), owner index
   int64_t pcap;
   // stress
   double* spart;     // 9 per pair block (batched instances: per stress slice): stresslet sums
-  int spart_blocks;
   double* sigma;     // 9K: stress of each instance at the last force pass
   double* sigma_sum; // 9K: sum over committed steps since the last reset
   int64_t mean_steps;         // steps summed in sigma_sum

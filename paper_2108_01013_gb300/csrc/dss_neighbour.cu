@@ -455,9 +455,10 @@ __device__ __forceinline__ int64_t far_group(int k) { return blockIdx.x + (int64
 // owners of the block's part of it, or (grp >= 0) a group of its owners.
 template <bool ECH, bool SPLIT, bool NARROW>
 __device__ __forceinline__ void search_segment(
-    SegShared& sh, const Geo& g, const InstGeo& I, const StepGeo& sg, const StateBuf& s, const float4* __restrict__ posf,
-    const int* __restrict__ cellid, const int* __restrict__ cell_start, int* __restrict__ list, int* __restrict__ count,
-    int* __restrict__ nnear, const RowSums& R, DevStatus* st, const EnumCut& q, int lane, int r, int grp) {
+    SegShared& sh, const Geo& g, const InstGeo& I, const StepGeo& sg, const StateBuf& s,
+    const float4* __restrict__ posf, const int* __restrict__ cellid, const int* __restrict__ cell_start,
+    int* __restrict__ list, int* __restrict__ count, int* __restrict__ nnear, const RowSums& R, DevStatus* st,
+    const EnumCut& q, int lane, int r, int grp) {
   const int nx = I.nc[0], ny = I.nc[1], nz = I.nc[2];
   // the warp's row: w cells from x = xf on, of the row of cells at rc
   const int4 par = sh.par[r];
@@ -740,7 +741,8 @@ k_enumerate_seg(const __grid_constant__ Geo g, const __grid_constant__ InstGeo I
     set_segment(sh, I, sg.fsh, row, ((int)item - row * I.enum_hx) * I.enum_seg, sub + 1 < subs ? sub : -1 - sub);
   }
   __syncthreads();
-  search_segment<ECH, SPLIT, NARROW>(sh, g, I, sg, s, posf, cellid, cell_start, list, count, nnear, R, st, q, lane, r, -1);
+  search_segment<ECH, SPLIT, NARROW>(sh, g, I, sg, s, posf, cellid, cell_start, list, count, nnear, R, st, q, lane, r,
+                                     -1);
   if (sh.far)
     search_far<ECH, SPLIT, ONE, NARROW>(sh, g, I1, ig, sgk, s, posf, cellid, cell_start, list, count, nnear, R, st, q);
 }

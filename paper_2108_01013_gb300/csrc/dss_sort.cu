@@ -95,13 +95,11 @@ __device__ __noinline__ int rank_beyond_row(const int* __restrict__ id, int mine
 // out otherwise).
 template <bool WAVE>
 __global__ void __launch_bounds__(kThreads, 4)
-k_rank_gather(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__ sgk, StateBuf src,
-              StateBuf dst, const int* __restrict__ key, const int* __restrict__ cell_start,
-              const int* __restrict__ cell_ids, int bcap, const int* __restrict__ more,
-              const int* __restrict__ link_next, const unsigned* __restrict__ link_lanes,
-              int* __restrict__ cell_count,
-              int* __restrict__ tile_count, int clear, int* __restrict__ perm, int* __restrict__ cellid,
-              float4* __restrict__ posf, DevStatus* st, int most_seg, int long_seg, bool predict,
+k_rank_gather(Geo g, const InstGeo* __restrict__ ig, StateBuf src, StateBuf dst, const int* __restrict__ key,
+              const int* __restrict__ cell_start, const int* __restrict__ cell_ids, int bcap,
+              const int* __restrict__ more, const int* __restrict__ link_next,
+              const unsigned* __restrict__ link_lanes, int* __restrict__ cell_count, int* __restrict__ tile_count,
+              int clear, int* __restrict__ perm, int* __restrict__ cellid, float4* __restrict__ posf, DevStatus* st, int most_seg, int long_seg, bool predict,
               const double* __restrict__ pred, const signed char* __restrict__ xc) {
   dep_wait();
   if (dev_err(st)) return;
@@ -215,7 +213,6 @@ k_rank_gather(Geo g, const InstGeo* __restrict__ ig, const StepGeo* __restrict__
     store_rec(dst.rec + rec_geometry(f), Rec8{pf.x, pf.y, pf.z, pf.w, pl.x, pl.y, pl.z, pl.w});
     store_rec(dst.rec + rec_motion(f), mv);
   }
-  (void)sgk;
 }
 
 }  // namespace
@@ -405,16 +402,10 @@ void launch_sort(dss_handle* h, bool predict, int src, int dst, bool keyed) {
   prof_mark(h, 2);
   const int clear = scan_tiles_for(h->g.ncell) <= kScanTiles ? h->g.ncell : 0;
   const SortOut so = sort_out(h);
-  if (h->g.wave)
-    launch_dep(k_rank_gather<true>, blocks, kThreads, h->stream, h->g, h->ig, h->sg, h->st[src], h->st[dst], h->key,
-                                                            h->cell_start, h->cell_ids, h->cell_cap, so.more, so.link_next, so.link_lanes,
-               h->cell_count, h->tile_count, clear, h->perm, h->cellid,
-                                                            h->posf, h->status, h->enum_most_seg, h->enum_long_seg, predict, h->pred, h->xc);
-  else
-    launch_dep(k_rank_gather<false>, blocks, kThreads, h->stream, h->g, h->ig, h->sg, h->st[src], h->st[dst], h->key,
-                                                             h->cell_start, h->cell_ids, h->cell_cap, so.more, so.link_next, so.link_lanes,
-               h->cell_count, h->tile_count, clear, h->perm, h->cellid,
-                                                             h->posf, h->status, h->enum_most_seg, h->enum_long_seg, predict, h->pred, h->xc);
+  auto k = h->g.wave ? k_rank_gather<true> : k_rank_gather<false>;
+  launch_dep(k, blocks, kThreads, h->stream, h->g, h->ig, h->st[src], h->st[dst], h->key, h->cell_start, h->cell_ids,
+             h->cell_cap, so.more, so.link_next, so.link_lanes, h->cell_count, h->tile_count, clear, h->perm, h->cellid,
+             h->posf, h->status, h->enum_most_seg, h->enum_long_seg, predict, h->pred, h->xc);
 }
 
 // Self-test of the integer-operation conversions (f32_rn, f32_split, f64_of,
