@@ -99,18 +99,17 @@ KERNELS_PER_STEP = 7
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) from
 # an ncu capture of the kernel, keyed by kernel, precision and particle count,
 # with the sources it was built from and their hash; reported only while
-# those files are unchanged (pair kernel: profiles/ncu_full_c2_mixed_100k.md,
-# profiles/ncu_full_c3_mixed_1m.md; enumeration:
-# profiles/ncu_enumerate_screened_c3_mixed_1m.md; the 1M captures ran with the
-# row capacity cut to 64, which changes the rows' stride, not the pairs or the
+# those files are unchanged (profiles/ncu_step_kernels.md; the 1M capture ran with
+# the row capacity cut to 64, which changes the rows' stride, not the pairs or the
 # work).
 _PAIR_SRC = ("dss_force.cu", "dss_internal.cuh", "dss_pair_model.cuh")
 _ENUM_SRC = ("dss_neighbour.cu", "dss_internal.cuh")
 NCU_TRAFFIC = {
-    ("k_pairs", "mixed", 100_000): (30_699_520, _PAIR_SRC, "9557dfb1c9e0b948"),
-    ("k_enumerate", "mixed", 100_000): (7_125_760, _ENUM_SRC, "614103effa34d4d4"),
-    ("k_pairs", "mixed", 1_000_000): (300_538_112, _PAIR_SRC, "9557dfb1c9e0b948"),
-    ("k_enumerate", "mixed", 1_000_000): (110_382_848, _ENUM_SRC, "614103effa34d4d4"),
+    ("k_pairs", "mixed", 100_000): (30_039_296, _PAIR_SRC, "30d6533a08d2ec65"),
+    ("k_enumerate", "mixed", 100_000): (3_340_288, _ENUM_SRC, "fee88b4488e6c92e"),
+    ("k_pairs", "fp64", 100_000): (29_491_200, _PAIR_SRC, "30d6533a08d2ec65"),
+    ("k_pairs", "mixed", 1_000_000): (287_442_176, _PAIR_SRC, "30d6533a08d2ec65"),
+    ("k_enumerate", "mixed", 1_000_000): (53_195_776, _ENUM_SRC, "fee88b4488e6c92e"),
 }
 
 

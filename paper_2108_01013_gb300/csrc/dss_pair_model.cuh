@@ -24,7 +24,7 @@
 // two fifths of the operations of the separate resistance functions.  With it,
 // one reciprocal for three, the tangent projection taken once, comparisons on
 // bit patterns and the stresslet from r (x) F and r x F^L, the FP64 pair kernel
-// (85% of the FP64 pipe's rate before and after) went from 274 to 189 us on
+// (85% of the FP64 pipe's rate before, 81% after) went from 274 to 189 us on
 // 267k pairs (the step of 100k spheres 355 -> 266 us).
 #pragma once
 
