@@ -99,9 +99,9 @@ KERNELS_PER_STEP = 7
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) from
 # an ncu capture of the kernel, keyed by kernel, precision and particle count,
 # with the sources it was built from and their hash; reported only while
-# those files are unchanged (profiles/ncu_step_kernels.md; the 1M capture ran with
-# the row capacity cut to 64, which changes the rows' stride, not the pairs or the
-# work).
+# those files are unchanged (captures summarised under profiles/; the 1M one ran
+# with the row capacity cut to 64, which changes the rows' stride, not the pairs
+# or the work).
 _PAIR_SRC = ("dss_force.cu", "dss_internal.cuh", "dss_pair_model.cuh")
 _ENUM_SRC = ("dss_neighbour.cu", "dss_internal.cuh")
 NCU_TRAFFIC = {
