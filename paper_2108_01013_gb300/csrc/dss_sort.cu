@@ -99,8 +99,9 @@ k_rank_gather(Geo g, const InstGeo* __restrict__ ig, StateBuf src, StateBuf dst,
               const int* __restrict__ cell_start, const int* __restrict__ cell_ids, int bcap,
               const int* __restrict__ more, const int* __restrict__ link_next,
               const unsigned* __restrict__ link_lanes, int* __restrict__ cell_count, int* __restrict__ tile_count,
-              int clear, int* __restrict__ perm, int* __restrict__ cellid, float4* __restrict__ posf, DevStatus* st, int most_seg, int long_seg, bool predict,
-              const double* __restrict__ pred, const signed char* __restrict__ xc) {
+              int clear, int* __restrict__ perm, int* __restrict__ cellid, float4* __restrict__ posf, DevStatus* st,
+              int most_seg, int long_seg, bool predict, const double* __restrict__ pred,
+              const signed char* __restrict__ xc) {
   dep_wait();
   if (dev_err(st)) return;
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
